@@ -196,7 +196,7 @@ int encode_map(PFN_cuTensorMapEncodeTiled_v12000 enc, CUtensorMap* m, const void
     for (int i = 0; i + 1 < rank; ++i)
         if (strides[i] % 16) return fail(SSD_ERR_INVALID_ARG, "tensor stride not a multiple of 16 bytes for TMA");
     if (dims[0] < 64 || box[0] != 64) return fail(SSD_ERR_INVALID_ARG, "tensor row shorter than one TMA box");
-    cuuint32_t estr[4] = {1, 1, 1, 1};
+    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     CUresult r = enc(m, dtype, (cuuint32_t)rank, const_cast<void*>(base), dims, strides,
                      box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -265,10 +265,16 @@ int build_tmaps(ssd_handle* h) {
     return SSD_OK;
 }
 
-// TMA maps of the prefill GEMMs: every matrix [rows][K] bf16 viewed as
-// {K, rows}, box 64 (k) x 128 rows, 128-byte swizzle (the tcgen05 operand
-// layout); layer l's wq wk wv wo w_gate w_up w_down at 7l + 0..6, then the
-// activation planes x hi / lo, attention output hi / lo, SwiGLU output hi / lo.
+// TMA maps of the prefill GEMMs (128-byte swizzle, the tcgen05 operand layout),
+// 64 wide in k: layer l's wq wk wv wo w_gate w_up w_down at 7l + 0..6, then the
+// token planes x, attention output, SwiGLU output at 7L + 8 b + class.
+//   wo, w_down   {K, rows}, box of 128 rows
+//   w_gate, w_up {K, rows}, box of 16 rows: a tile's TMEM lanes alternate 16
+//                gate and 16 up rows, so that both are in one warp
+//   wq wk wv     {K, 16, 2, hd / 32, heads} with strides of 1 row, hd / 2 rows,
+//                16 rows and hd rows: one box is 128 rows, 16 of the first
+//                half of a head's dims, then their 16 rotation partners, ...
+//   planes       {K, rows, 2}, box of tok / 2 rows of hi and of lo
 int build_prefill(ssd_handle* h) {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -279,27 +285,40 @@ int build_prefill(ssd_handle* h) {
     const ssd_config& c = h->cfg;
     const int L = c.n_layers, d = c.d_model, qd = c.n_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim;
     PrefillPlan& P = h->pf;
-    std::vector<CUtensorMap> maps((size_t)7 * L + 6);
-    auto map2 = [&](CUtensorMap* m, const void* base, int K, int rows) {
-        cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-        cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-        cuuint32_t box[2] = {64, 128};
-        return encode_map(enc, m, base, 2, dims, strides, box);
+    std::vector<CUtensorMap> maps((size_t)7 * L + 3 * kPfTokClasses);
+    auto rows2 = [&](CUtensorMap* m, const void* base, int K, int rows, int box_rows) {
+        return encode_weight(enc, m, base, K, rows, box_rows);
+    };
+    auto heads5 = [&](CUtensorMap* m, const void* base, int heads) {
+        const cuuint64_t row = (cuuint64_t)d * 2, hd = (cuuint64_t)c.head_dim;
+        cuuint64_t dims[5] = {(cuuint64_t)d, 16, 2, hd / 32, (cuuint64_t)heads};
+        cuuint64_t strides[4] = {row, row * (hd / 2), row * 16, row * hd};
+        cuuint32_t box[5] = {64, 16, 2, (cuuint32_t)(hd / 32), (cuuint32_t)(128 / hd)};
+        return encode_map(enc, m, base, 5, dims, strides, box);
+    };
+    auto planes3 = [&](CUtensorMap* m, const void* base, int K, int tok) {
+        cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)P.rows, 2};
+        cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)K * 2 * P.rows};
+        cuuint32_t box[3] = {64, (cuuint32_t)(tok / 2), 2};
+        return encode_map(enc, m, base, 3, dims, strides, box);
     };
     int rc = 0;
     for (int l = 0; l < L && !rc; ++l) {
-        const bf16* w[7] = {h->wq[l], h->wk[l], h->wv[l], h->wo[l], h->w_gate[l], h->w_up[l], h->w_down[l]};
-        const int K[7] = {d, d, d, qd, d, d, c.ffn};
-        const int N[7] = {qd, kvd, kvd, d, c.ffn, c.ffn, d};
-        for (int i = 0; i < 7 && !rc; ++i) rc = map2(&maps[7 * l + i], w[i], K[i], N[i]);
+        CUtensorMap* m = &maps[(size_t)7 * l];
+        if (!rc) rc = heads5(m + 0, h->wq[l], c.n_heads);
+        if (!rc) rc = heads5(m + 1, h->wk[l], c.n_kv_heads);
+        if (!rc) rc = heads5(m + 2, h->wv[l], c.n_kv_heads);
+        if (!rc) rc = rows2(m + 3, h->wo[l], qd, d, 128);
+        if (!rc) rc = rows2(m + 4, h->w_gate[l], d, c.ffn, 16);
+        if (!rc) rc = rows2(m + 5, h->w_up[l], d, c.ffn, 16);
+        if (!rc) rc = rows2(m + 6, h->w_down[l], c.ffn, d, 128);
     }
     const size_t a0 = (size_t)7 * L;
-    if (!rc) rc = map2(&maps[a0 + 0], P.x_hi, d, P.rows);
-    if (!rc) rc = map2(&maps[a0 + 1], P.x_lo, d, P.rows);
-    if (!rc) rc = map2(&maps[a0 + 2], P.at_hi, qd, P.rows);
-    if (!rc) rc = map2(&maps[a0 + 3], P.at_lo, qd, P.rows);
-    if (!rc) rc = map2(&maps[a0 + 4], P.ac_hi, c.ffn, P.rows);
-    if (!rc) rc = map2(&maps[a0 + 5], P.ac_lo, c.ffn, P.rows);
+    for (int t = 0; t < kPfTokClasses && !rc; ++t) {
+        if (!rc) rc = planes3(&maps[a0 + t], P.x_hi, d, 32 * (t + 1));
+        if (!rc) rc = planes3(&maps[a0 + kPfTokClasses + t], P.at_hi, qd, 32 * (t + 1));
+        if (!rc) rc = planes3(&maps[a0 + 2 * kPfTokClasses + t], P.ac_hi, c.ffn, 32 * (t + 1));
+    }
     if (rc) return rc;
     CUDA_TRY(cudaMemcpy(h->pf_tmaps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice),
              "prefill tensor map upload");
@@ -312,12 +331,11 @@ int build_prefill(ssd_handle* h) {
         Ly.k_cache = h->kc + (size_t)l * h->kv_layer;
         Ly.v_cache = h->vc + (size_t)l * h->kv_layer;
     }
-    P.tm_x[0] = h->pf_tmaps + a0 + 0;
-    P.tm_x[1] = h->pf_tmaps + a0 + 1;
-    P.tm_at[0] = h->pf_tmaps + a0 + 2;
-    P.tm_at[1] = h->pf_tmaps + a0 + 3;
-    P.tm_ac[0] = h->pf_tmaps + a0 + 4;
-    P.tm_ac[1] = h->pf_tmaps + a0 + 5;
+    for (int t = 0; t < kPfTokClasses; ++t) {
+        P.tm_x[t] = h->pf_tmaps + a0 + t;
+        P.tm_at[t] = h->pf_tmaps + a0 + kPfTokClasses + t;
+        P.tm_ac[t] = h->pf_tmaps + a0 + 2 * kPfTokClasses + t;
+    }
     P.layers = h->pf_layers.data();
     return SSD_OK;
 }
@@ -768,8 +786,13 @@ int ssd_create(const ssd_config* cfg, const ssd_weights* w, void* cuda_stream, s
         if ((rc = dalloc(h, &P.h, R * d, &B)) || (rc = dalloc(h, &P.x_hi, 2 * R * d, &B)) ||
             (rc = dalloc(h, &P.q, R * qd, &B)) || (rc = dalloc(h, &P.at_hi, 2 * R * qd, &B)) ||
             (rc = dalloc(h, &P.ac_hi, 2 * R * F, &B)) ||
-            (rc = dalloc(h, &h->pf_tmaps, (size_t)7 * L + 6, &B)))
+            (rc = dalloc(h, &P.ws, prefill_ws_floats(h->n_sms / 2), &B)) ||
+            (rc = dalloc(h, &P.flags, prefill_flag_words(h->n_sms / 2), &B)) ||
+            (rc = dalloc(h, &h->pf_tmaps, (size_t)7 * L + 3 * kPfTokClasses, &B)))
             return bail(rc);
+        P.pairs = h->n_sms / 2;
+        cudaError_t ef = cudaMemset(P.flags, 0, prefill_flag_words(P.pairs) * sizeof(unsigned));
+        if (ef != cudaSuccess) return bail(fail(SSD_ERR_CUDA, std::string("prefill flags: ") + cudaGetErrorString(ef)));
         P.x_lo = P.x_hi + R * d;
         P.at_lo = P.at_hi + R * qd;
         P.ac_lo = P.ac_hi + R * F;

@@ -291,11 +291,28 @@ int prefill_configure() {
     return e;
 }
 
+size_t prefill_ws_floats(int pairs) { return (size_t)pairs * 2 * tc::kMaxTok * 128; }
+size_t prefill_flag_words(int pairs) { return (size_t)pairs * 2 * tc::kEpiWarps; }
+
 // One chunk of prompt rows at positions pos0 .. pos0 + n - 1 through every
 // layer (launches only).  toks: device token ids of the chunk.
-int prefill_chunk(const PrefillPlan& P, const int* toks, int n, int pos0, cudaStream_t s) {
+int prefill_chunk(PrefillPlan& P, const int* toks, int n, int pos0, cudaStream_t s) {
     const int d = P.d, qd = P.n_heads * P.head_dim, kvd = P.n_kv_heads * P.head_dim;
-    const int row_tiles = (n + tc::kBM - 1) / tc::kBM;
+    // the arguments every GEMM shares: n_out outputs in n_ft tiles of 256 weight rows, K inputs
+    auto gemm = [&](const void* const* tm_x, int n_out, int n_ft, int K) {
+        tc::TcArgs a{};
+        a.rows = n;
+        a.N = n_out;
+        a.n_kb = (K + tc::kBK - 1) / tc::kBK;
+        tc::tc_plan(a, n_ft, P.pairs);
+        a.tm_x = tm_x[a.nt / 32 - 1];
+        a.ws = P.ws;
+        a.flags = P.flags;
+        if (++P.epoch == 0) ++P.epoch;
+        a.epoch = P.epoch;
+        a.err = P.err;
+        return a;
+    };
     pf_embed_kernel<<<n, kNormThreads, 0, s>>>(P.embed, toks, d, P.h);
     int e = (int)cudaGetLastError();
     for (int l = 0; l < P.n_layers && !e; ++l) {
@@ -303,16 +320,10 @@ int prefill_chunk(const PrefillPlan& P, const int* toks, int n, int pos0, cudaSt
         pf_norm_kernel<<<n, kNormThreads, 0, s>>>(P.h, L.attn_norm, d, P.eps, P.x_hi, P.x_lo);
         e = (int)cudaGetLastError();
         if (e) break;
-        tc::TcArgs a{};
-        a.tm_a_hi = P.tm_x[0];
-        a.tm_a_lo = P.tm_x[1];
-        a.tm_b[0] = L.tm_w[0];
-        a.tm_b[1] = L.tm_w[1];
-        a.tm_b[2] = L.tm_w[2];
-        a.rows = n;
-        a.K = d;
-        a.n_kb = (d + tc::kBK - 1) / tc::kBK;
-        a.n_tiles = (qd + 2 * kvd + tc::kBN - 1) / tc::kBN;
+        tc::TcArgs a = gemm(P.tm_x, qd + 2 * kvd, (qd + 2 * kvd + tc::kFeat - 1) / tc::kFeat, d);
+        a.tm_w[0] = L.tm_w[0];
+        a.tm_w[1] = L.tm_w[1];
+        a.tm_w[2] = L.tm_w[2];
         a.n_heads = P.n_heads;
         a.n_kv_heads = P.n_kv_heads;
         a.head_dim = P.head_dim;
@@ -322,8 +333,7 @@ int prefill_chunk(const PrefillPlan& P, const int* toks, int n, int pos0, cudaSt
         a.k_cache = L.k_cache;
         a.v_cache = L.v_cache;
         a.rope = P.rope;
-        a.err = P.err;
-        e = tc::tc_launch<tc::TC_QKV>(a, row_tiles, s);
+        e = tc::tc_launch<tc::TC_QKV>(a, s);
         if (e) break;
         const dim3 ag((n + kAttQ - 1) / kAttQ, P.n_heads);
         const float scale = 1.0f / std::sqrt((float)P.head_dim);
@@ -335,52 +345,25 @@ int prefill_chunk(const PrefillPlan& P, const int* toks, int n, int pos0, cudaSt
                                                           P.n_kv_heads, P.max_seq, scale, P.at_hi, P.at_lo);
         e = (int)cudaGetLastError();
         if (e) break;
-        tc::TcArgs o{};
-        o.tm_a_hi = P.tm_at[0];
-        o.tm_a_lo = P.tm_at[1];
-        o.tm_b[0] = o.tm_b[1] = o.tm_b[2] = L.tm_w[3];
-        o.rows = n;
-        o.K = qd;
-        o.n_kb = (qd + tc::kBK - 1) / tc::kBK;
-        o.n_tiles = (d + tc::kBN - 1) / tc::kBN;
-        o.N = d;
+        tc::TcArgs o = gemm(P.tm_at, d, (d + tc::kFeat - 1) / tc::kFeat, qd);
+        o.tm_w[0] = L.tm_w[3];
         o.out = P.h;
-        o.ldo = d;
-        o.err = P.err;
-        e = tc::tc_launch<tc::TC_RESID>(o, row_tiles, s);
+        e = tc::tc_launch<tc::TC_RESID>(o, s);
         if (e) break;
         pf_norm_kernel<<<n, kNormThreads, 0, s>>>(P.h, L.mlp_norm, d, P.eps, P.x_hi, P.x_lo);
         e = (int)cudaGetLastError();
         if (e) break;
-        tc::TcArgs gu{};
-        gu.tm_a_hi = P.tm_x[0];
-        gu.tm_a_lo = P.tm_x[1];
-        gu.tm_b[0] = L.tm_w[4];
-        gu.tm_b[1] = L.tm_w[5];
-        gu.tm_b[2] = L.tm_w[4];
-        gu.rows = n;
-        gu.K = d;
-        gu.n_kb = (d + tc::kBK - 1) / tc::kBK;
-        gu.n_tiles = (P.ffn + 127) / 128;
-        gu.ffn = P.ffn;
+        tc::TcArgs gu = gemm(P.tm_x, P.ffn, (P.ffn + 127) / 128, d);  // 128 features: gate and up rows
+        gu.tm_w[0] = L.tm_w[4];
+        gu.tm_w[1] = L.tm_w[5];
         gu.act_hi = P.ac_hi;
         gu.act_lo = P.ac_lo;
-        gu.err = P.err;
-        e = tc::tc_launch<tc::TC_SWIGLU>(gu, row_tiles, s);
+        e = tc::tc_launch<tc::TC_SWIGLU>(gu, s);
         if (e) break;
-        tc::TcArgs dn{};
-        dn.tm_a_hi = P.tm_ac[0];
-        dn.tm_a_lo = P.tm_ac[1];
-        dn.tm_b[0] = dn.tm_b[1] = dn.tm_b[2] = L.tm_w[6];
-        dn.rows = n;
-        dn.K = P.ffn;
-        dn.n_kb = (P.ffn + tc::kBK - 1) / tc::kBK;
-        dn.n_tiles = (d + tc::kBN - 1) / tc::kBN;
-        dn.N = d;
+        tc::TcArgs dn = gemm(P.tm_ac, d, (d + tc::kFeat - 1) / tc::kFeat, P.ffn);
+        dn.tm_w[0] = L.tm_w[6];
         dn.out = P.h;
-        dn.ldo = d;
-        dn.err = P.err;
-        e = tc::tc_launch<tc::TC_RESID>(dn, row_tiles, s);
+        e = tc::tc_launch<tc::TC_RESID>(dn, s);
     }
     return e;
 }

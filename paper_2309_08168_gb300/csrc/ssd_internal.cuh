@@ -169,8 +169,9 @@ struct FwdParams {
 // ---------------------------------------------------------------------------
 // prefill on the tensor cores (prefill.cu, tc_gemm.cuh)
 // ---------------------------------------------------------------------------
+constexpr int kPfTokClasses = 8;  // token tiles of 32 (class + 1) rows
 struct PrefillLayer {
-    const void* tm_w[7];  // TMA maps (box 64 x 128) of wq wk wv wo w_gate w_up w_down
+    const void* tm_w[7];  // TMA maps of wq wk wv wo w_gate w_up w_down (TcArgs::tm_w)
     const bf16* attn_norm;
     const bf16* mlp_norm;
     f16* k_cache;  // this layer's [Hkv][max_seq][hd]
@@ -190,14 +191,21 @@ struct PrefillPlan {
     bf16* at_lo;
     bf16* ac_hi;        // [rows][ffn] SwiGLU output, hi / lo
     bf16* ac_lo;
-    const void* tm_x[2];   // TMA maps of x_hi / x_lo  (box 64 x 128)
-    const void* tm_at[2];  // of at_hi / at_lo
-    const void* tm_ac[2];  // of ac_hi / ac_lo
+    // TMA maps of the hi / lo planes of x, at and ac for token tiles of 32, 64, .. 256 rows
+    const void* tm_x[kPfTokClasses];
+    const void* tm_at[kPfTokClasses];
+    const void* tm_ac[kPfTokClasses];
+    int pairs;             // CTA pairs of the GEMMs (half the SMs)
+    float* ws;             // split tiles: partial sums [pairs][2][256][128]
+    unsigned* flags;       // and their flags [pairs][2][8] (TcArgs)
+    unsigned epoch;        // of the last GEMM launch
     const PrefillLayer* layers;  // host array
     int* err;
 };
 int prefill_configure();
-int prefill_chunk(const PrefillPlan& P, const int* toks, int n, int pos0, cudaStream_t s);
+size_t prefill_ws_floats(int pairs);
+size_t prefill_flag_words(int pairs);
+int prefill_chunk(PrefillPlan& P, const int* toks, int n, int pos0, cudaStream_t s);
 
 int forward_configure();
 int launch_forward(const FwdParams& p, int head_dim, int grid, cudaStream_t s);

@@ -1,25 +1,36 @@
 // tc_gemm.cuh - the prompt-encoding GEMM on the 5th-generation tensor cores
-// (tcgen05, sm_103a): D[rows x 256] = A[rows x K] * B[256 x K]^T per CTA
-// tile, with the fused epilogues of the prefill.
+// (tcgen05, sm_103a), with the fused epilogues of the prefill:
+//     D[feature][token] = W[feature][K] * (X_hi + X_lo)[token][K]^T.
 //
 // The prefill (Sec. 3.1: the prompt is encoded before Algorithms 1 / 2 start
 // decoding) runs every prompt row through the full model at once, so its
-// projections are dense GEMMs with M = 128 .. 2048 token rows: compute-bound,
-// unlike the decode forwards.  One CTA computes a 128-row x 256-column tile:
-//   warp 0, one thread : TMA producer.  Per 64-wide k block it copies the
-//                        activation tile twice (bf16 hi and lo planes, 128 x 64
-//                        each) and the weight tile as two 128-row boxes (so
-//                        the 256 columns can come from two matrices, e.g. the
-//                        gate and up rows of the same features), 128-byte
-//                        swizzle, into a ring of kTcStages stages;
-//   warp 1, one thread : MMA issuer.  tcgen05.mma kind::f16 (bf16 x bf16 ->
-//                        fp32), M = 128, N = 256, K = 16, eight per k block
-//                        (four k steps x hi and lo), accumulating in TMEM;
-//                        tcgen05.commit releases each stage and finally
-//                        signals the epilogue;
-//   warps 0-3          : epilogue.  Warp w reads TMEM lanes 32w..32w+31 (one
-//                        token row per thread) with tcgen05.ld and applies
-//                        the op's epilogue.
+// projections are dense GEMMs over 17 .. 2048 token rows: bound by HBM (the
+// weights) below ~140 rows, by the tensor cores above.
+//
+// Weights are the M side and tokens the N side: M is always full (a pair of
+// CTAs holds 256 weight rows) and N can be any multiple of 32 up to 256, so a
+// ragged token count is padded to 32 rows per tile instead of a full tile, and
+// the epilogue's lanes are consecutive features (coalesced rows).  Two CTAs of
+// a cluster work on one tile (tcgen05 cta_group::2): each stages its own 128
+// weight rows and half of the token rows, so a k block of 64 costs 16 KB +
+// nt * 128 bytes of shared-memory traffic per CTA for 2 * 128 * nt * 64
+// multiply-adds (hi and lo), 25 % less L2 -> SM traffic than a CTA alone with a
+// 128 x 256 tile.  Per CTA:
+//   warp 8, one thread : TMA producer, a ring of S stages (as many as fit);
+//                        the copies of both CTAs complete on the even CTA's
+//                        barrier;
+//   warp 9, one thread : (even CTA) MMA issuer: tcgen05.mma kind::f16 (bf16 x
+//                        bf16 -> fp32), M = 256, N = nt, K = 16, eight per k
+//                        block (four k steps x hi and lo), into one of two
+//                        TMEM accumulators of up to 256 columns;
+//   warps 0-7          : epilogue of a finished accumulator while the next one
+//                        fills.  Warp w reads TMEM lanes 32 (w mod 4) .. +31 and
+//                        the columns of half w / 4.
+// The grid is persistent, one CTA pair per two SMs.  Work = tiles (256 features
+// x nt tokens; token tiles fastest, so pairs that share weights run together)
+// x k blocks of 64.  A remainder that would leave a wave of tiles part empty
+// is split over all pairs by k block instead (TcSched below).
+//
 // Operands are K-major with the canonical 128-byte-swizzle layout that TMA
 // writes: row r of a tile at r * 128 bytes, 8-row groups 1024 bytes apart
 // (the descriptor's stride byte offset), each k step of 16 moves the start
@@ -30,8 +41,8 @@
 // TMEM accumulator (~16 mantissa bits of x).
 //
 // Every wait is bounded (~2 s): on a timeout the thread records the error
-// code and stops waiting; the CTA then gives its copies and MMAs in flight
-// time to finish, frees its TMEM and returns.
+// code and stops waiting; the CTAs then give copies and MMAs in flight time to
+// finish, free their TMEM and return.
 #pragma once
 
 #include "ssd_internal.cuh"
@@ -39,37 +50,49 @@
 namespace ssd {
 namespace tc {
 
-constexpr int kBM = 128;          // token rows per tile (TMEM lanes)
-constexpr int kBN = 256;          // output columns per tile (TMEM columns)
-constexpr int kBK = 64;           // k per stage: 128 bytes of bf16 = one swizzle row
-constexpr int kStages = 3;
-constexpr int kThreads = 128;
-constexpr int kATile = kBM * kBK * 2;        // 16 KB (one plane)
-constexpr int kBTile = kBN * kBK * 2;        // 32 KB
-constexpr int kStage = 2 * kATile + kBTile;  // 64 KB
-constexpr size_t kSmemBytes = 1024 + (size_t)kStages * kStage + 256;
+constexpr int kBK = 64;            // k per stage: 128 bytes of bf16 = one swizzle row
+constexpr int kFeat = 256;         // weight rows per tile (two CTAs x 128 TMEM lanes)
+constexpr int kMaxTok = 256;       // token columns per tile (TMEM columns of one accumulator)
+constexpr int kEpiWarps = 8;
+constexpr int kThreads = (kEpiWarps + 2) * 32;
+constexpr int kATile = 128 * kBK * 2;         // 16 KB: this CTA's weight rows of a k block
+constexpr int kRingBytes = 224 * 1024;
+constexpr int kMaxStages = 11;                // 20 KB stages at 32 tokens
+constexpr size_t kSmemBytes = 1024 + (size_t)kRingBytes;
+constexpr int kTmemCols = 512;                // two accumulators of 256 columns
 constexpr unsigned long long kWaitNs = 2000000000ull;
 constexpr int kErrTimeout = 1;
+constexpr int kMinSplit = 8;                  // k blocks a pair gets at least when tiles are split
 
 // epilogues of the prefill GEMMs
-enum TcEpi { TC_STORE = 0, TC_RESID = 1, TC_SWIGLU = 2, TC_QKV = 3 };
+enum TcEpi { TC_RESID = 1, TC_SWIGLU = 2, TC_QKV = 3 };
+
+// How tiles are spread over the pairs: the first n_split tiles by k block over
+// split_pairs pairs, in contiguous ranges (a tile cut by a range end is summed
+// by the pair holding its first k blocks, in range order; the others leave
+// their partial sums in the workspace), the others whole, pair by pair.
+struct TcSched {
+    int n_tiles, n_split, split_pairs, pairs;
+};
 
 struct TcArgs {
-    // TMA maps: activation planes (hi, lo) viewed as {K, rows}, box {64, 128};
-    // weight matrices viewed as {K, N}, box {64, 128}
-    const void* tm_a_hi;
-    const void* tm_a_lo;
-    const void* tm_b[3];   // weight matrices (QKV: wq, wk, wv; SWIGLU: gate, up; else [0])
+    // TMA maps.  Weights: RESID {K, N}, box {64, 128}; SWIGLU gate, up {K, N},
+    // box {64, 16}; QKV wq, wk, wv as {K, 16, 2, hd / 32, heads}, box = 128 rows.
+    // Tokens: planes as {K, rows, 2}, box {64, nt / 2, 2}.
+    const void* tm_w[3];
+    const void* tm_x;
     int rows;              // valid token rows
-    int K;
+    int nt;                // token rows per tile: a multiple of 32, at most 256
+    int n_tt;              // token tiles
     int n_kb;              // ceil(K / 64)
-    int n_tiles;           // column tiles (gridDim.y)
-    int N;                 // valid output columns (STORE / RESID: width of out)
-    float* out;            // STORE: [rows][ldo] fp32; RESID: residual h [rows][ldo] (+= D)
-    int ldo;
-    // SWIGLU: act planes [rows][ffn] bf16 hi / lo of silu(gate) * up
-    int ffn;
-    bf16* act_hi;
+    int stages;            // ring depth
+    int N;                 // output features (SWIGLU: ffn)
+    TcSched sched;
+    float* ws;             // [pairs][2][256][128] fp32 partial sums
+    unsigned* flags;       // [pairs][2][8] epoch of the partial sums a warp left
+    unsigned epoch;        // of this launch, never 0 or an earlier one
+    float* out;            // RESID: residual h [rows][N] (+= D)
+    bf16* act_hi;          // SWIGLU: planes [rows][ffn] of silu(gate) * up
     bf16* act_lo;
     // QKV: q (fp32, rotated) [rows][H*hd]; K / V cache of the layer
     // [Hkv][max_seq][hd] fp16; RoPE table [max_seq][hd/2] (cos, sin)
@@ -81,34 +104,67 @@ struct TcArgs {
     int* err;
 };
 
-// 128-row boxes of tile t: matrix index and first row of each half
-struct TcHalves {
-    int s0, r0, s1, r1;
+// One pair's work, segment by segment: k blocks [kb0, kb1) of a tile.
+struct TcWork {
+    long long U;
+    int cur, end, next_tile;
+    int tile, kb0, kb1;
+    int contributors;  // > 0: this segment ends the pair's range inside the tile; that many pairs follow
+    bool partial;      // the segment starts inside the tile: its sums go to the workspace
 };
-__device__ __forceinline__ TcHalves tc_halves(const TcArgs& a, int epi, int t) {
-    if (epi == TC_SWIGLU) return {0, t * 128, 1, t * 128};  // gate rows, up rows of features t*128..
-    if (epi == TC_QKV) {
-        // [Wq; Wk; Wv] in 128-row boxes (q and kv widths are multiples of 128)
-        const int qd = a.n_heads * a.head_dim, kvd = a.n_kv_heads * a.head_dim;
-        int b[2], s[2];
-        for (int h = 0; h < 2; ++h) {
-            int r = (2 * t + h) * 128;
-            if (r < qd) { s[h] = 0; b[h] = r; }
-            else if (r < qd + kvd) { s[h] = 1; b[h] = r - qd; }
-            else { s[h] = 2; b[h] = r - qd - kvd; }
-        }
-        return {s[0], b[0], s[1], b[1]};
+__host__ __device__ __forceinline__ void tc_work_init(TcWork& w, const TcSched& s, int n_kb, int pair) {
+    w.U = (long long)s.n_split * n_kb;
+    w.cur = w.end = 0;
+    if (pair < s.split_pairs) {
+        w.cur = (int)(pair * w.U / s.split_pairs);
+        w.end = (int)((pair + 1) * w.U / s.split_pairs);
     }
-    return {0, t * kBN, 0, t * kBN + 128};
+    w.next_tile = s.n_split + pair;
+}
+__host__ __device__ __forceinline__ bool tc_work_next(TcWork& w, const TcSched& s, int n_kb, int pair) {
+    w.contributors = 0;
+    w.partial = false;
+    if (w.cur < w.end) {
+        w.tile = w.cur / n_kb;
+        w.kb0 = w.cur - w.tile * n_kb;
+        w.kb1 = w.kb0 + w.end - w.cur < n_kb ? w.kb0 + w.end - w.cur : n_kb;
+        w.cur += w.kb1 - w.kb0;
+        w.partial = w.kb0 > 0;
+        if (!w.partial && w.kb1 < n_kb) {
+            const long long last = (long long)(w.tile + 1) * n_kb - 1;  // the pair holding the tile's last k block
+            w.contributors = (int)(((last + 1) * s.split_pairs + w.U - 1) / w.U - 1) - pair;
+        }
+        return true;
+    }
+    if (w.next_tile >= s.n_tiles) return false;
+    w.tile = w.next_tile;
+    w.kb0 = 0;
+    w.kb1 = n_kb;
+    w.next_tile += s.pairs;
+    return true;
 }
 
 // ---------------------------------------------------------------------------
-// PTX wrappers (tcgen05, TMA, mbarrier)
+// PTX wrappers (tcgen05, TMA, mbarrier, cluster)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned long long gtime() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// address of the same shared-memory object in the cluster's CTA `rank`
+__device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void mb_init(uint64_t* b, unsigned n) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(n) : "memory");
@@ -116,10 +172,15 @@ __device__ __forceinline__ void mb_init(uint64_t* b, unsigned n) {
 __device__ __forceinline__ void mb_arrive_tx(uint64_t* b, unsigned bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
 }
+// arrival on a barrier of either CTA of the pair (cluster address)
+__device__ __forceinline__ void mb_arrive_cluster(uint32_t addr) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
 __device__ __forceinline__ bool mb_try(uint64_t* b, unsigned parity) {
     unsigned ok;
     asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(ok)
         : "r"(smem_u32(b)), "r"(parity)
         : "memory");
@@ -140,11 +201,28 @@ __device__ __forceinline__ bool mb_wait(uint64_t* b, unsigned parity, int* err) 
     }
     return true;
 }
-// 2D tiled TMA load; x (the k coordinate) is always a multiple of 64 elements
-__device__ __forceinline__ void tma2d(void* dst, const void* map, int x, int y, uint64_t* b) {
+// tiled TMA loads into this CTA's shared memory, completing on a barrier of
+// either CTA of the pair (cluster address); x (the k coordinate) is always a
+// multiple of 64 elements
+__device__ __forceinline__ void tma2d(void* dst, const void* map, int x, int y, uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(smem_u32(b))
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
+        "l"(map), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
+__device__ __forceinline__ void tma3d(void* dst, const void* map, int x, int y, int z, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
+        "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
+__device__ __forceinline__ void tma5d_head(void* dst, const void* map, int x, int head, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%2, %3, %3, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
+        "l"(map), "r"(x), "r"(0), "r"(head), "r"(bar)
         : "memory");
 }
 
@@ -160,21 +238,25 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
     return d;
 }
 // instruction descriptor: kind::f16, A = B = bf16, D = fp32, both K-major,
-// N = 256, M = 128
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kBN >> 3) << 17) |
-                            ((uint32_t)(kBM >> 4) << 24);
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t ad, uint64_t bd, uint32_t accumulate) {
+// M = 256 over the pair, N = nt
+__device__ __forceinline__ uint32_t tc_idesc(int nt) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nt >> 3) << 17) | ((uint32_t)(kFeat >> 4) << 24);
+}
+__device__ __forceinline__ void mma_pair(uint32_t tmem_d, uint64_t ad, uint64_t bd, uint32_t idesc,
+                                         uint32_t accumulate) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-        ::"r"(tmem_d), "l"(ad), "l"(bd), "r"(kIdesc), "r"(accumulate)
+        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+        ::"r"(tmem_d), "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// the mbarrier completes once every tcgen05 op this thread issued so far is done
+// the barrier at this offset in both CTAs completes once every tcgen05 op this
+// thread issued so far is done
 __device__ __forceinline__ void mma_commit(uint64_t* b) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(b))
-                 : "memory");
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+        ::"r"(smem_u32(b)), "h"((uint16_t)3)
+        : "memory");
 }
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -195,183 +277,331 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// ---------------------------------------------------------------------------
-// epilogue helpers (one token row per thread, 32 columns at a time)
-// ---------------------------------------------------------------------------
 __device__ __forceinline__ void store_hilo(bf16* hi, bf16* lo, float x) {
     const bf16 h = __float2bfloat16_rn(x);
     *hi = h;
     *lo = __float2bfloat16_rn(x - __bfloat162float(h));
 }
 
+// The lanes of a warp hold features in two groups of 16: lane l < 16 one
+// member of a pair, lane l + 16 the other (gate / up, or the two halves of a
+// rotation).  Exchanges the columns of a chunk so that every lane has both
+// members for half of the tokens: on return lane l < 16 holds (a, b) of the
+// even columns, lane l + 16 of the odd columns, a = the lower lanes' feature.
+__device__ __forceinline__ void pair_up(const float (&v)[32], int upper, float (&a)[16], float (&b)[16]) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        const float recv = __shfl_xor_sync(0xffffffffu, upper ? v[2 * j] : v[2 * j + 1], 16);
+        a[j] = upper ? recv : v[2 * j];
+        b[j] = upper ? v[2 * j + 1] : recv;
+    }
+}
+
 // ---------------------------------------------------------------------------
-// the kernel: grid = (column tiles, row tiles)
+// the kernel: grid = 2 * pairs, clusters of 2
 // ---------------------------------------------------------------------------
 template <int EPI>
-__global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const TcArgs a) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm_kernel(const TcArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStage);
-    uint64_t* empty = full + kStages;
-    uint64_t* done = empty + kStages;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    __shared__ __align__(8) uint64_t full[kMaxStages];   // (even CTA) both CTAs' copies of a stage have landed
+    __shared__ __align__(8) uint64_t empty[kMaxStages];  // the pair's MMAs have read the stage
+    __shared__ __align__(8) uint64_t acc_full[2];        // accumulator complete
+    __shared__ __align__(8) uint64_t acc_empty[2];       // (even CTA) read by the epilogue warps of both CTAs
+    __shared__ uint32_t s_tmem;
     __shared__ int s_fail;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // row tiles fastest: the CTAs that share a weight tile run together, so
-    // each weight tile is read from DRAM once and from L2 by the other rows
-    const int tile = blockIdx.y, m0 = blockIdx.x * kBM;
+    const uint32_t rank = cluster_rank();
+    // the highest ranges start first: a pair only waits for partial sums of
+    // pairs with higher numbers, which were dispatched before it
+    const int pair = a.sched.pairs - 1 - (int)(blockIdx.x >> 1);
+    const int S = a.stages, stage_bytes = kATile + a.nt * 128;
     if (threadIdx.x == 0) {
         s_fail = 0;
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < S; ++s) {
             mb_init(full + s, 1);
             mb_init(empty + s, 1);
         }
-        mb_init(done, 1);
+        for (int b = 0; b < 2; ++b) {
+            mb_init(acc_full + b, 1);
+            mb_init(acc_empty + b, 2 * kEpiWarps);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (warp == 2) {  // TMEM: 256 fp32 columns x 128 lanes for the accumulator
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(kBN)
+    if (warp == kEpiWarps) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(kTmemCols)
                      : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     fence_before();
     __syncthreads();
+    cluster_sync();
     fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = s_tmem;
 
     bool ok = true;
-    if (warp == 0 && lane == 0) {
-        // producer: activations (may be written by the previous kernel:
-        // generic proxy) and weights through TMA
+    TcWork w;
+    tc_work_init(w, a.sched, a.n_kb, pair);
+    if (warp == kEpiWarps && lane == 0) {
+        // producer: weights, and activations that the previous kernel wrote
         asm volatile("fence.proxy.async.global;" ::: "memory");
-        const TcHalves hv = tc_halves(a, EPI, tile);
-        for (int kb = 0; kb < a.n_kb && ok; ++kb) {
-            const int s = kb % kStages;
-            if (kb >= kStages) ok = mb_wait(empty + s, ((kb / kStages) - 1) & 1u, a.err);
-            if (!ok) break;
-            unsigned char* st = smem + s * kStage;
-            mb_arrive_tx(full + s, (unsigned)kStage);
-            tma2d(st, a.tm_a_hi, kb * kBK, m0, full + s);
-            tma2d(st + kATile, a.tm_a_lo, kb * kBK, m0, full + s);
-            tma2d(st + 2 * kATile, a.tm_b[hv.s0], kb * kBK, hv.r0, full + s);
-            tma2d(st + 2 * kATile + kATile, a.tm_b[hv.s1], kb * kBK, hv.r1, full + s);
+        int s = 0;
+        unsigned ph = 1;  // parity of the next "empty" completion to wait for (the ring starts empty)
+        while (ok && tc_work_next(w, a.sched, a.n_kb, pair)) {
+            const int ft = w.tile / a.n_tt, tt = w.tile - ft * a.n_tt;
+            const int tok0 = tt * a.nt + (int)rank * (a.nt >> 1);
+            const int box = 2 * ft + (int)rank;  // this CTA's 128 TMEM lanes
+            const void* map = a.tm_w[0];
+            int row0 = box * 128;
+            if (EPI == TC_QKV) {  // [Wq; Wk; Wv] in 128-row boxes of whole heads (past the end: zeros)
+                const int qd = a.n_heads * a.head_dim, kvd = a.n_kv_heads * a.head_dim;
+                if (row0 >= qd + kvd) { map = a.tm_w[2]; row0 -= qd + kvd; }
+                else if (row0 >= qd) { map = a.tm_w[1]; row0 -= qd; }
+                row0 /= a.head_dim;
+            }
+            for (int kb = w.kb0; kb < w.kb1; ++kb) {
+                ok = mb_wait(empty + s, ph, a.err);
+                if (!ok) break;
+                unsigned char* st = smem + s * stage_bytes;
+                const uint32_t bar = map_rank(smem_u32(full + s), 0);
+                if (rank == 0) mb_arrive_tx(full + s, 2u * (unsigned)stage_bytes);
+                if (EPI == TC_QKV) {
+                    tma5d_head(st, map, kb * kBK, row0, bar);
+                } else if (EPI == TC_SWIGLU) {  // 16 gate rows, then 16 up rows of the same features, ...
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        tma2d(st + g * 4096, a.tm_w[0], kb * kBK, box * 64 + g * 16, bar);
+                        tma2d(st + g * 4096 + 2048, a.tm_w[1], kb * kBK, box * 64 + g * 16, bar);
+                    }
+                } else {
+                    tma2d(st, map, kb * kBK, row0, bar);
+                }
+                tma3d(st + kATile, a.tm_x, kb * kBK, tok0, 0, bar);
+                if (++s == S) { s = 0; ph ^= 1u; }
+            }
         }
-    } else if (warp == 1 && lane == 0) {
-        // MMA issuer
-        for (int kb = 0; kb < a.n_kb && ok; ++kb) {
-            const int s = kb % kStages;
-            ok = mb_wait(full + s, (kb / kStages) & 1u, a.err);
+        // the commits that release the last stages also arrive here: do not
+        // leave before them
+        for (int i = 0; i < S && ok; ++i) {
+            ok = mb_wait(empty + s, ph, a.err);
+            if (++s == S) { s = 0; ph ^= 1u; }
+        }
+    } else if (warp == kEpiWarps + 1 && lane == 0 && rank == 0) {
+        // MMA issuer of the pair
+        const uint32_t idesc = tc_idesc(a.nt);
+        int s = 0, b = 0;
+        unsigned ph = 0, aph = 3u;  // aph bit b: parity of the next release of accumulator b (both start free)
+        while (ok && tc_work_next(w, a.sched, a.n_kb, pair)) {
+            ok = mb_wait(acc_empty + b, (aph >> b) & 1u, a.err);
+            if (!ok) break;
+            aph ^= 1u << b;
+            fence_after();
+            const uint32_t d = tmem + (uint32_t)(b * kMaxTok);
+            for (int kb = w.kb0; kb < w.kb1; ++kb) {
+                ok = mb_wait(full + s, ph, a.err);
+                if (!ok) break;
+                fence_after();
+                const uint32_t st = smem_u32(smem + s * stage_bytes);
+                const uint32_t xh = st + kATile, xl = xh + (uint32_t)a.nt * 64;
+#pragma unroll
+                for (int kk = 0; kk < kBK / 16; ++kk) {
+                    const uint64_t ad = sdesc(st + kk * 32);
+                    mma_pair(d, ad, sdesc(xh + kk * 32), idesc, (kb != w.kb0 || kk) ? 1u : 0u);
+                    mma_pair(d, ad, sdesc(xl + kk * 32), idesc, 1u);
+                }
+                mma_commit(empty + s);  // the stage is free once these MMAs have read it
+                if (++s == S) { s = 0; ph ^= 1u; }
+            }
+            if (ok) mma_commit(acc_full + b);
+            b ^= 1;
+        }
+    } else if (warp < kEpiWarps) {
+        const int q4 = warp & 3, half = warp >> 2, upper = lane >> 4;
+        const int hc = a.nt >> 1;  // columns of this warp: half * hc .. + hc
+        const uint32_t empty0[2] = {map_rank(smem_u32(acc_empty), 0), map_rank(smem_u32(acc_empty + 1), 0)};
+        int b = 0;
+        unsigned fph = 0;  // bit b: parity of the next completion of accumulator b
+        while (ok && tc_work_next(w, a.sched, a.n_kb, pair)) {
+            const int ft = w.tile / a.n_tt, tt = w.tile - ft * a.n_tt;
+            const int box = 2 * ft + (int)rank;
+            const int tok0 = tt * a.nt + half * hc;
+            const int n_col = min(hc, a.rows - tok0);  // valid columns of this warp (may be <= 0)
+            ok = mb_wait(acc_full + b, (fph >> b) & 1u, a.err);
+            fph ^= 1u << b;
             if (!ok) break;
             fence_after();
-            const uint32_t st = smem_u32(smem + s * kStage);
-#pragma unroll
-            for (int kk = 0; kk < kBK / 16; ++kk) {
-                const uint64_t bd = sdesc(st + 2 * kATile + kk * 32);
-                mma_bf16(tmem, sdesc(st + kk * 32), bd, (kb | kk) != 0);
-                mma_bf16(tmem, sdesc(st + kATile + kk * 32), bd, 1u);
-            }
-            mma_commit(empty + s);  // the stage is free once these MMAs have read it
-        }
-        if (ok) mma_commit(done);
-    }
-    if (!ok) s_fail = 1;
-    __syncwarp();
-
-    // epilogue: wait for the accumulator (all threads)
-    if (ok) ok = mb_wait(done, 0, a.err);
-    if (!ok) s_fail = 1;
-    fence_after();
-    const int row = m0 + warp * 32 + lane;  // this thread's token row
-    const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
-    __syncthreads();
-    if (!s_fail) {
-        if (EPI == TC_STORE || EPI == TC_RESID) {
-            for (int c0 = 0; c0 < kBN; c0 += 32) {
-                float v[32];
-                tmem_ld32(tl + c0, v);
-                const int n0 = tile * kBN + c0;
-                if (row < a.rows) {
-                    float* o = a.out + (size_t)row * a.ldo + n0;
+            const uint32_t tl = tmem + (uint32_t)(b * kMaxTok + half * hc) + ((uint32_t)(q4 * 32) << 16);
+            // partial sums [pair][cta][column][lane], 128 bytes per warp and column
+            auto slot = [&](int p) {
+                return a.ws + (((size_t)p * 2 + rank) * kMaxTok + half * hc) * 128 + q4 * 32 + lane;
+            };
+            if (w.partial) {
+                float* o = slot(pair);
+                for (int c0 = 0; c0 < n_col; c0 += 32) {
+                    float v[32];
+                    tmem_ld32(tl + c0, v);
 #pragma unroll
                     for (int i = 0; i < 32; ++i)
-                        if (n0 + i < a.N) o[i] = EPI == TC_RESID ? o[i] + v[i] : v[i];
+                        if (c0 + i < n_col) __stcg(o + (size_t)(c0 + i) * 128, v[i]);
                 }
-            }
-        } else if (EPI == TC_SWIGLU) {
-            for (int c0 = 0; c0 < 128; c0 += 32) {
-                float g[32], u[32];
-                tmem_ld32(tl + c0, g);
-                tmem_ld32(tl + 128 + c0, u);
-                const int f0 = tile * 128 + c0;
-                if (row < a.rows) {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        if (f0 + i >= a.ffn) break;
-                        const float x = g[i] / (1.f + expf(-g[i])) * u[i];
-                        const size_t at = (size_t)row * a.ffn + f0 + i;
-                        store_hilo(a.act_hi + at, a.act_lo + at, x);
+                __threadfence();
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.flags + (pair * 2 + rank) * kEpiWarps + warp),
+                                 "r"(a.epoch)
+                                 : "memory");
+            } else {
+                for (int c = 1; c <= w.contributors && ok; ++c) {  // (bounded) until their partial sums are there
+                    const unsigned* f = a.flags + ((pair + c) * 2 + rank) * kEpiWarps + warp;
+                    const unsigned long long t0 = gtime();
+                    for (;;) {
+                        unsigned x;
+                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(f) : "memory");
+                        if (x == a.epoch) break;
+                        const unsigned long long dt = gtime() - t0;
+                        if ((dt > 20000ull && *(volatile int*)a.err) || dt > kWaitNs) {
+                            atomicCAS(a.err, 0, kErrTimeout);
+                            ok = false;
+                            break;
+                        }
                     }
                 }
-            }
-        } else {  // TC_QKV: two 128-row boxes, each whole heads of q, k or v
-            const int hd = a.head_dim, half = hd >> 1;
-            const int qd = a.n_heads * hd, kvd = a.n_kv_heads * hd;
-            const int pos = a.pos0 + row;
-            for (int h = 0; h < 2; ++h) {
-                const int f0 = (2 * tile + h) * 128;  // feature of column 0 of this box
-                if (f0 >= qd + 2 * kvd) break;
-                const int kind = f0 < qd ? 0 : (f0 < qd + kvd ? 1 : 2);
-                const int fb = kind == 0 ? f0 : (kind == 1 ? f0 - qd : f0 - qd - kvd);
-                for (int hb = 0; hb < 128; hb += hd) {       // heads in this box
-                    for (int c0 = 0; c0 < half; c0 += 32) {  // rotation pairs (i, i + half)
-                        float x1[32], x2[32];
-                        tmem_ld32(tl + h * 128 + hb + c0, x1);
-                        tmem_ld32(tl + h * 128 + hb + half + c0, x2);
-                        if (row >= a.rows) continue;
-                        const int head = (fb + hb) / hd;
+                ok = __all_sync(0xffffffffu, ok);
+                for (int c0 = 0; c0 < n_col && ok; c0 += 32) {
+                    float v[32];
+                    tmem_ld32(tl + c0, v);
+                    if (w.contributors) {
+                        float ps[32];
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) {
-                            const int ii = c0 + i;
-                            if (kind == 2) {
-                                f16* vrow = a.v_cache + ((size_t)head * a.max_seq + pos) * hd;
-                                vrow[ii] = __float2half_rn(x1[i]);
-                                vrow[ii + half] = __float2half_rn(x2[i]);
-                                continue;
+                        for (int i = 0; i < 32; ++i) ps[i] = 0.f;
+                        for (int c = 1; c <= w.contributors; ++c) {
+                            const float* p = slot(pair + c);
+                            float x[32];
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) x[i] = c0 + i < n_col ? __ldcg(p + (size_t)(c0 + i) * 128) : 0.f;
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) ps[i] += x[i];
+                        }
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) v[i] += ps[i];
+                    }
+                    const int tok = tok0 + c0;  // token row of v[0]
+                    if (EPI == TC_RESID) {
+                        const int n = box * 128 + q4 * 32 + lane;
+                        if (n < a.N) {
+                            float* o = a.out + (size_t)tok * a.N + n;
+                            float h[32];
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) h[i] = c0 + i < n_col ? o[(size_t)i * a.N] : 0.f;
+#pragma unroll
+                            for (int i = 0; i < 32; ++i)
+                                if (c0 + i < n_col) o[(size_t)i * a.N] = h[i] + v[i];
+                        }
+                    } else if (EPI == TC_SWIGLU) {
+                        float g[16], u[16];
+                        pair_up(v, upper, g, u);
+                        const int f = box * 64 + q4 * 16 + (lane & 15);
+                        if (f < a.N) {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) {
+                                const int c = 2 * j + upper;
+                                if (c0 + c >= n_col) continue;
+                                const float x = g[j] / (1.f + expf(-g[j])) * u[j];
+                                const size_t at = (size_t)(tok + c) * a.N + f;
+                                store_hilo(a.act_hi + at, a.act_lo + at, x);
                             }
-                            const float2 cs = a.rope[(size_t)pos * half + ii];
-                            const float y1 = x1[i] * cs.x - x2[i] * cs.y;
-                            const float y2 = x2[i] * cs.x + x1[i] * cs.y;
-                            if (kind == 0) {
-                                float* q = a.q + (size_t)row * qd + head * hd;
-                                q[ii] = y1;
-                                q[ii + half] = y2;
-                            } else {
-                                f16* krow = a.k_cache + ((size_t)head * a.max_seq + pos) * hd;
-                                krow[ii] = __float2half_rn(y1);
-                                krow[ii + half] = __float2half_rn(y2);
+                        }
+                    } else {  // TC_QKV: this CTA's box is whole heads of q, k or v
+                        const int hd = a.head_dim, half_d = hd >> 1;
+                        const int qd = a.n_heads * hd, kvd = a.n_kv_heads * hd;
+                        const int f0 = box * 128;
+                        const int kind = f0 < qd ? 0 : (f0 < qd + kvd ? 1 : 2);
+                        const int head = (f0 - (kind == 0 ? 0 : (kind == 1 ? qd : qd + kvd))) / hd + q4 / (hd / 32);
+                        const int ii = (q4 % (hd / 32)) * 16 + (lane & 15);  // rotation pair (ii, ii + hd / 2)
+                        if (f0 >= qd + 2 * kvd) continue;  // (uniform: past the last box)
+                        if (kind == 2) {
+                            f16* o = a.v_cache + ((size_t)head * a.max_seq + a.pos0 + tok) * hd + ii + upper * half_d;
+#pragma unroll
+                            for (int i = 0; i < 32; ++i)
+                                if (c0 + i < n_col) o[(size_t)i * hd] = __float2half_rn(v[i]);
+                        } else {
+                            float x1[16], x2[16];
+                            pair_up(v, upper, x1, x2);
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) {
+                                const int c = 2 * j + upper;
+                                if (c0 + c >= n_col) continue;
+                                const int pos = a.pos0 + tok + c;
+                                const float2 cs = a.rope[(size_t)pos * half_d + ii];
+                                const float y1 = x1[j] * cs.x - x2[j] * cs.y;
+                                const float y2 = x2[j] * cs.x + x1[j] * cs.y;
+                                if (kind == 0) {
+                                    float* q = a.q + (size_t)(tok + c) * qd + head * hd;
+                                    q[ii] = y1;
+                                    q[ii + half_d] = y2;
+                                } else {
+                                    f16* k = a.k_cache + ((size_t)head * a.max_seq + pos) * hd;
+                                    k[ii] = __float2half_rn(y1);
+                                    k[ii + half_d] = __float2half_rn(y2);
+                                }
                             }
                         }
                     }
                 }
             }
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mb_arrive_cluster(empty0[b]);  // this warp is done with the accumulator
+            b ^= 1;
         }
-    } else {
-        // a wait gave up: let copies and MMAs in flight finish before the
-        // shared memory and TMEM are released
-        if (threadIdx.x == 0) {
-            const unsigned long long t0 = gtime();
-            while (gtime() - t0 < 2000000ull) __nanosleep(1000);
-        }
+    }
+    if (!ok) s_fail = 1;
+    __syncwarp();
+    __syncthreads();
+    if (s_fail && threadIdx.x == 0) {
+        // a wait gave up: let copies and MMAs in flight finish before shared
+        // memory and TMEM are released
+        const unsigned long long t0 = gtime();
+        while (gtime() - t0 < 2000000ull) __nanosleep(1000);
     }
     fence_before();
     __syncthreads();
-    if (warp == 2) {
+    cluster_sync();  // the other CTA's MMAs, arrivals and commits are done with this CTA
+    if (warp == kEpiWarps) {
         fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kBN) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
     }
+}
+
+// Tile shape and schedule of a GEMM over `rows` tokens and n_ft feature tiles.
+// Tokens: as few tiles of at most 256 as hold the rows, of equal size rounded
+// up to 32.  Tiles that fill whole waves of pairs run whole; the rest is split
+// by k block over all pairs (with less than half a wave left, one more wave is
+// split with it, so that a tile is cut in two or three rather than many), in
+// pieces of at least kMinSplit k blocks.
+inline void tc_plan(TcArgs& a, int n_ft, int pairs) {
+    a.n_tt = (a.rows + kMaxTok - 1) / kMaxTok;
+    a.nt = ((a.rows + a.n_tt - 1) / a.n_tt + 31) / 32 * 32;
+    a.n_tt = (a.rows + a.nt - 1) / a.nt;
+    const int stage = kATile + a.nt * 128;
+    a.stages = kRingBytes / stage < kMaxStages ? kRingBytes / stage : kMaxStages;
+    TcSched& s = a.sched;
+    s.n_tiles = n_ft * a.n_tt;
+    const int waves = s.n_tiles / pairs, rest = s.n_tiles % pairs;
+    s.n_split = rest == 0 ? 0 : (waves > 0 && 2 * rest < pairs ? rest + pairs : rest);
+    long long p = (long long)s.n_split * a.n_kb / kMinSplit;
+    if (p > pairs) p = pairs;
+    if (p < rest) p = rest;  // (rest < pairs: at worst every tile is a range of its own)
+    if (p < 1) p = 1;
+    if (waves > 0 && s.n_split > rest && p < pairs) {  // too short to split: whole tiles only
+        s.n_split = 0;
+        p = 1;
+    }
+    s.split_pairs = (int)p;
+    s.pairs = s.n_tiles - s.n_split > 0 ? pairs : s.split_pairs;
 }
 
 template <int EPI>
@@ -381,8 +611,8 @@ inline int tc_configure() {
 }
 
 template <int EPI>
-inline int tc_launch(const TcArgs& a, int row_tiles, cudaStream_t s) {
-    tc_gemm_kernel<EPI><<<dim3(row_tiles, a.n_tiles), kThreads, kSmemBytes, s>>>(a);
+inline int tc_launch(const TcArgs& a, cudaStream_t s) {
+    tc_gemm_kernel<EPI><<<2 * a.sched.pairs, kThreads, kSmemBytes, s>>>(a);
     return (int)cudaGetLastError();
 }
 
