@@ -269,8 +269,12 @@ int build_tmaps(ssd_handle* h) {
 // 64 wide in k: layer l's wq wk wv wo w_gate w_up w_down at 7l + 0..6, then the
 // token planes x, attention output, SwiGLU output at 7L + 8 b + class.
 //   wo, w_down   {K, rows}, box of 128 rows
-//   w_gate, w_up {K, rows}, box of 16 rows: a tile's TMEM lanes alternate 16
-//                gate and 16 up rows, so that both are in one warp
+//   w_gate, w_up one map {K, 16, 2, rows / 16} whose third stride is the distance
+//                between the two matrices: one box is 128 rows, 16 of gate, 16 of
+//                up, ..., so that a TMEM lane quadrant holds both (at w_gate's
+//                place; the lower matrix comes first).  A tensor map's strides
+//                end at 2^40: matrices further apart get a map each, {K, rows},
+//                box of 16 rows, and eight copies per tile instead of one
 //   wq wk wv     {K, 16, 2, hd / 32, heads} with strides of 1 row, hd / 2 rows,
 //                16 rows and hd rows: one box is 128 rows, 16 of the first
 //                half of a head's dims, then their 16 rotation partners, ...
@@ -296,6 +300,22 @@ int build_prefill(ssd_handle* h) {
         cuuint32_t box[5] = {64, 16, 2, (cuuint32_t)(hd / 32), (cuuint32_t)(128 / hd)};
         return encode_map(enc, m, base, 5, dims, strides, box);
     };
+    auto far_apart = [](const bf16* g, const bf16* u) {
+        const uintptr_t x = (uintptr_t)g, y = (uintptr_t)u;
+        return (x < y ? y - x : x - y) >= ((uintptr_t)1 << 40);
+    };
+    auto pair4 = [&](CUtensorMap* m, const bf16* g, const bf16* u) {
+        if (far_apart(g, u)) {
+            const int r = rows2(m, g, d, c.ffn, 16);
+            return r ? r : rows2(m + 1, u, d, c.ffn, 16);
+        }
+        const bf16 *lo = g < u ? g : u, *hi = g < u ? u : g;
+        const cuuint64_t row = (cuuint64_t)d * 2;
+        cuuint64_t dims[4] = {(cuuint64_t)d, 16, 2, (cuuint64_t)(c.ffn / 16)};
+        cuuint64_t strides[3] = {row, (cuuint64_t)((uintptr_t)hi - (uintptr_t)lo), row * 16};
+        cuuint32_t box[4] = {64, 16, 2, 4};
+        return encode_map(enc, m, lo, 4, dims, strides, box);
+    };
     auto planes3 = [&](CUtensorMap* m, const void* base, int K, int tok) {
         cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)P.rows, 2};
         cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)K * 2 * P.rows};
@@ -309,8 +329,7 @@ int build_prefill(ssd_handle* h) {
         if (!rc) rc = heads5(m + 1, h->wk[l], c.n_kv_heads);
         if (!rc) rc = heads5(m + 2, h->wv[l], c.n_kv_heads);
         if (!rc) rc = rows2(m + 3, h->wo[l], qd, d, 128);
-        if (!rc) rc = rows2(m + 4, h->w_gate[l], d, c.ffn, 16);
-        if (!rc) rc = rows2(m + 5, h->w_up[l], d, c.ffn, 16);
+        if (!rc) rc = pair4(m + 4, h->w_gate[l], h->w_up[l]);
         if (!rc) rc = rows2(m + 6, h->w_down[l], c.ffn, d, 128);
     }
     const size_t a0 = (size_t)7 * L;
@@ -326,6 +345,9 @@ int build_prefill(ssd_handle* h) {
     for (int l = 0; l < L; ++l) {
         PrefillLayer& Ly = h->pf_layers[l];
         for (int i = 0; i < 7; ++i) Ly.tm_w[i] = h->pf_tmaps + 7 * l + i;
+        Ly.swapped = h->w_up[l] < h->w_gate[l];
+        if (far_apart(h->w_gate[l], h->w_up[l])) Ly.swapped = 0;
+        else Ly.tm_w[5] = nullptr;
         Ly.attn_norm = h->attn_norm[l];
         Ly.mlp_norm = h->mlp_norm[l];
         Ly.k_cache = h->kc + (size_t)l * h->kv_layer;

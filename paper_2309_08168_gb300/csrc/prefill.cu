@@ -356,6 +356,7 @@ int prefill_chunk(PrefillPlan& P, const int* toks, int n, int pos0, cudaStream_t
         tc::TcArgs gu = gemm(P.tm_x, P.ffn, (P.ffn + 127) / 128, d);  // 128 features: gate and up rows
         gu.tm_w[0] = L.tm_w[4];
         gu.tm_w[1] = L.tm_w[5];
+        gu.swapped = L.swapped;
         gu.act_hi = P.ac_hi;
         gu.act_lo = P.ac_lo;
         e = tc::tc_launch<tc::TC_SWIGLU>(gu, s);

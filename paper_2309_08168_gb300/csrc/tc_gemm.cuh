@@ -16,16 +16,16 @@
 // nt * 128 bytes of shared-memory traffic per CTA for 2 * 128 * nt * 64
 // multiply-adds (hi and lo), 25 % less L2 -> SM traffic than a CTA alone with a
 // 128 x 256 tile.  Per CTA:
-//   warp 8, one thread : TMA producer, a ring of S stages (as many as fit);
+//   warp 16            : TMA producer, a ring of S stages (as many as fit);
 //                        the copies of both CTAs complete on the even CTA's
 //                        barrier;
-//   warp 9, one thread : (even CTA) MMA issuer: tcgen05.mma kind::f16 (bf16 x
+//   warp 17            : (even CTA) MMA issuer: tcgen05.mma kind::f16 (bf16 x
 //                        bf16 -> fp32), M = 256, N = nt, K = 16, eight per k
 //                        block (four k steps x hi and lo), into one of two
 //                        TMEM accumulators of up to 256 columns;
-//   warps 0-7          : epilogue of a finished accumulator while the next one
+//   warps 0-15         : epilogue of a finished accumulator while the next one
 //                        fills.  Warp w reads TMEM lanes 32 (w mod 4) .. +31 and
-//                        the columns of half w / 4.
+//                        the columns of quarter w / 4, 16 at a time.
 // The grid is persistent, one CTA pair per two SMs.  Work = tiles (256 features
 // x nt tokens; token tiles fastest, so pairs that share weights run together)
 // x k blocks of 64.  A remainder that would leave a wave of tiles part empty
@@ -53,7 +53,7 @@ namespace tc {
 constexpr int kBK = 64;            // k per stage: 128 bytes of bf16 = one swizzle row
 constexpr int kFeat = 256;         // weight rows per tile (two CTAs x 128 TMEM lanes)
 constexpr int kMaxTok = 256;       // token columns per tile (TMEM columns of one accumulator)
-constexpr int kEpiWarps = 8;
+constexpr int kEpiWarps = 16;
 constexpr int kThreads = (kEpiWarps + 2) * 32;
 constexpr int kATile = 128 * kBK * 2;         // 16 KB: this CTA's weight rows of a k block
 constexpr int kRingBytes = 224 * 1024;
@@ -76,8 +76,10 @@ struct TcSched {
 };
 
 struct TcArgs {
-    // TMA maps.  Weights: RESID {K, N}, box {64, 128}; SWIGLU gate, up {K, N},
-    // box {64, 16}; QKV wq, wk, wv as {K, 16, 2, hd / 32, heads}, box = 128 rows.
+    // TMA maps.  Weights: RESID {K, N}, box {64, 128}; SWIGLU gate and up in one
+    // map {K, 16, 2, N / 16}, box {64, 16, 2, 4} (the lower matrix in memory
+    // first: swapped = 1 if that is up), or [1] != nullptr: gate, up {K, N}, box
+    // {64, 16} each; QKV wq, wk, wv as {K, 16, 2, hd / 32, heads}, box = 128 rows.
     // Tokens: planes as {K, rows, 2}, box {64, nt / 2, 2}.
     const void* tm_w[3];
     const void* tm_x;
@@ -87,9 +89,10 @@ struct TcArgs {
     int n_kb;              // ceil(K / 64)
     int stages;            // ring depth
     int N;                 // output features (SWIGLU: ffn)
+    int swapped;           // SWIGLU: lanes 0-15 hold up, 16-31 gate
     TcSched sched;
     float* ws;             // [pairs][2][256][128] fp32 partial sums
-    unsigned* flags;       // [pairs][2][8] epoch of the partial sums a warp left
+    unsigned* flags;       // [pairs][2][16] epoch of the partial sums a warp left
     unsigned epoch;        // of this launch, never 0 or an earlier one
     float* out;            // RESID: residual h [rows][N] (+= D)
     bf16* act_hi;          // SWIGLU: planes [rows][ffn] of silu(gate) * up
@@ -218,6 +221,13 @@ __device__ __forceinline__ void tma3d(void* dst, const void* map, int x, int y, 
         "l"(map), "r"(x), "r"(y), "r"(z), "r"(bar)
         : "memory");
 }
+__device__ __forceinline__ void tma4d_pair(void* dst, const void* map, int x, int group, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%2, %3, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
+        "l"(map), "r"(x), "r"(0), "r"(group), "r"(bar)
+        : "memory");
+}
 __device__ __forceinline__ void tma5d_head(void* dst, const void* map, int x, int head, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes "
@@ -261,20 +271,17 @@ __device__ __forceinline__ void mma_commit(uint64_t* b) {
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// 32 consecutive fp32 columns of this thread's TMEM lane
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-    uint32_t r[32];
+// 16 consecutive fp32 columns of this thread's TMEM lane
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 __device__ __forceinline__ void store_hilo(bf16* hi, bf16* lo, float x) {
@@ -288,9 +295,9 @@ __device__ __forceinline__ void store_hilo(bf16* hi, bf16* lo, float x) {
 // rotation).  Exchanges the columns of a chunk so that every lane has both
 // members for half of the tokens: on return lane l < 16 holds (a, b) of the
 // even columns, lane l + 16 of the odd columns, a = the lower lanes' feature.
-__device__ __forceinline__ void pair_up(const float (&v)[32], int upper, float (&a)[16], float (&b)[16]) {
+__device__ __forceinline__ void pair_up(const float (&v)[16], int upper, float (&a)[8], float (&b)[8]) {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
+    for (int j = 0; j < 8; ++j) {
         const float recv = __shfl_xor_sync(0xffffffffu, upper ? v[2 * j] : v[2 * j + 1], 16);
         a[j] = upper ? recv : v[2 * j];
         b[j] = upper ? v[2 * j + 1] : recv;
@@ -345,9 +352,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm
     bool ok = true;
     TcWork w;
     tc_work_init(w, a.sched, a.n_kb, pair);
-    if (warp == kEpiWarps && lane == 0) {
+    if (warp == kEpiWarps) {
         // producer: weights, and activations that the previous kernel wrote
         asm volatile("fence.proxy.async.global;" ::: "memory");
+        const uint32_t full0 = map_rank(smem_u32(full), 0);
         int s = 0;
         unsigned ph = 1;  // parity of the next "empty" completion to wait for (the ring starts empty)
         while (ok && tc_work_next(w, a.sched, a.n_kb, pair)) {
@@ -363,88 +371,99 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm
                 row0 /= a.head_dim;
             }
             for (int kb = w.kb0; kb < w.kb1; ++kb) {
-                ok = mb_wait(empty + s, ph, a.err);
+                ok = __all_sync(0xffffffffu, mb_wait(empty + s, ph, a.err));
                 if (!ok) break;
-                unsigned char* st = smem + s * stage_bytes;
-                const uint32_t bar = map_rank(smem_u32(full + s), 0);
-                if (rank == 0) mb_arrive_tx(full + s, 2u * (unsigned)stage_bytes);
-                if (EPI == TC_QKV) {
-                    tma5d_head(st, map, kb * kBK, row0, bar);
-                } else if (EPI == TC_SWIGLU) {  // 16 gate rows, then 16 up rows of the same features, ...
+                if (elect_one()) {
+                    unsigned char* st = smem + s * stage_bytes;
+                    const uint32_t bar = full0 + 8u * (uint32_t)s;
+                    if (rank == 0) mb_arrive_tx(full + s, 2u * (unsigned)stage_bytes);
+                    if (EPI == TC_QKV) {
+                        tma5d_head(st, map, kb * kBK, row0, bar);
+                    } else if (EPI == TC_SWIGLU) {
+                        if (a.tm_w[1] == nullptr) {
+                            tma4d_pair(st, map, kb * kBK, box * 4, bar);
+                        } else {
 #pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        tma2d(st + g * 4096, a.tm_w[0], kb * kBK, box * 64 + g * 16, bar);
-                        tma2d(st + g * 4096 + 2048, a.tm_w[1], kb * kBK, box * 64 + g * 16, bar);
+                            for (int g = 0; g < 4; ++g) {
+                                tma2d(st + g * 4096, map, kb * kBK, box * 64 + g * 16, bar);
+                                tma2d(st + g * 4096 + 2048, a.tm_w[1], kb * kBK, box * 64 + g * 16, bar);
+                            }
+                        }
+                    } else {
+                        tma2d(st, map, kb * kBK, row0, bar);
                     }
-                } else {
-                    tma2d(st, map, kb * kBK, row0, bar);
+                    tma3d(st + kATile, a.tm_x, kb * kBK, tok0, 0, bar);
                 }
-                tma3d(st + kATile, a.tm_x, kb * kBK, tok0, 0, bar);
+                __syncwarp();
                 if (++s == S) { s = 0; ph ^= 1u; }
             }
         }
         // the commits that release the last stages also arrive here: do not
         // leave before them
         for (int i = 0; i < S && ok; ++i) {
-            ok = mb_wait(empty + s, ph, a.err);
+            ok = __all_sync(0xffffffffu, mb_wait(empty + s, ph, a.err));
             if (++s == S) { s = 0; ph ^= 1u; }
         }
-    } else if (warp == kEpiWarps + 1 && lane == 0 && rank == 0) {
+    } else if (warp == kEpiWarps + 1 && rank == 0) {
         // MMA issuer of the pair
         const uint32_t idesc = tc_idesc(a.nt);
+        const uint64_t desc0 = sdesc(smem_u32(smem));
         int s = 0, b = 0;
         unsigned ph = 0, aph = 3u;  // aph bit b: parity of the next release of accumulator b (both start free)
         while (ok && tc_work_next(w, a.sched, a.n_kb, pair)) {
-            ok = mb_wait(acc_empty + b, (aph >> b) & 1u, a.err);
+            ok = __all_sync(0xffffffffu, mb_wait(acc_empty + b, (aph >> b) & 1u, a.err));
             if (!ok) break;
             aph ^= 1u << b;
             fence_after();
             const uint32_t d = tmem + (uint32_t)(b * kMaxTok);
             for (int kb = w.kb0; kb < w.kb1; ++kb) {
-                ok = mb_wait(full + s, ph, a.err);
+                ok = __all_sync(0xffffffffu, mb_wait(full + s, ph, a.err));
                 if (!ok) break;
                 fence_after();
-                const uint32_t st = smem_u32(smem + s * stage_bytes);
-                const uint32_t xh = st + kATile, xl = xh + (uint32_t)a.nt * 64;
+                if (elect_one()) {
+                    const uint64_t ad = desc0 + (uint64_t)((uint32_t)(s * stage_bytes) >> 4);
+                    const uint64_t xh = ad + (kATile >> 4), xl = xh + (uint64_t)(a.nt * 4);
 #pragma unroll
-                for (int kk = 0; kk < kBK / 16; ++kk) {
-                    const uint64_t ad = sdesc(st + kk * 32);
-                    mma_pair(d, ad, sdesc(xh + kk * 32), idesc, (kb != w.kb0 || kk) ? 1u : 0u);
-                    mma_pair(d, ad, sdesc(xl + kk * 32), idesc, 1u);
+                    for (int kk = 0; kk < kBK / 16; ++kk) {  // 16 k = 32 bytes
+                        mma_pair(d, ad + 2 * kk, xh + 2 * kk, idesc, (kb != w.kb0 || kk) ? 1u : 0u);
+                        mma_pair(d, ad + 2 * kk, xl + 2 * kk, idesc, 1u);
+                    }
+                    mma_commit(empty + s);  // the stage is free once these MMAs have read it
                 }
-                mma_commit(empty + s);  // the stage is free once these MMAs have read it
+                __syncwarp();
                 if (++s == S) { s = 0; ph ^= 1u; }
             }
-            if (ok) mma_commit(acc_full + b);
+            if (ok && elect_one()) mma_commit(acc_full + b);
+            __syncwarp();
             b ^= 1;
         }
     } else if (warp < kEpiWarps) {
-        const int q4 = warp & 3, half = warp >> 2, upper = lane >> 4;
-        const int hc = a.nt >> 1;  // columns of this warp: half * hc .. + hc
+        const int q4 = warp & 3, quarter = warp >> 2, upper = lane >> 4;
+        const int hc = a.nt >> 2;  // columns of this warp: quarter * hc .. + hc (a multiple of 8)
         const uint32_t empty0[2] = {map_rank(smem_u32(acc_empty), 0), map_rank(smem_u32(acc_empty + 1), 0)};
         int b = 0;
         unsigned fph = 0;  // bit b: parity of the next completion of accumulator b
         while (ok && tc_work_next(w, a.sched, a.n_kb, pair)) {
             const int ft = w.tile / a.n_tt, tt = w.tile - ft * a.n_tt;
             const int box = 2 * ft + (int)rank;
-            const int tok0 = tt * a.nt + half * hc;
+            const int tok0 = tt * a.nt + quarter * hc;
             const int n_col = min(hc, a.rows - tok0);  // valid columns of this warp (may be <= 0)
             ok = mb_wait(acc_full + b, (fph >> b) & 1u, a.err);
             fph ^= 1u << b;
             if (!ok) break;
             fence_after();
-            const uint32_t tl = tmem + (uint32_t)(b * kMaxTok + half * hc) + ((uint32_t)(q4 * 32) << 16);
+            const uint32_t tl = tmem + (uint32_t)(b * kMaxTok + quarter * hc) + ((uint32_t)(q4 * 32) << 16);
             // partial sums [pair][cta][column][lane], 128 bytes per warp and column
             auto slot = [&](int p) {
-                return a.ws + (((size_t)p * 2 + rank) * kMaxTok + half * hc) * 128 + q4 * 32 + lane;
+                return a.ws + (((size_t)p * 2 + rank) * kMaxTok + quarter * hc) * 128 + q4 * 32 + lane;
             };
             if (w.partial) {
                 float* o = slot(pair);
-                for (int c0 = 0; c0 < n_col; c0 += 32) {
-                    float v[32];
-                    tmem_ld32(tl + c0, v);
+                for (int c0 = 0; c0 < n_col; c0 += 16) {
+                    float v[16];
+                    tmem_ld16(tl + c0, v);
 #pragma unroll
-                    for (int i = 0; i < 32; ++i)
+                    for (int i = 0; i < 16; ++i)
                         if (c0 + i < n_col) __stcg(o + (size_t)(c0 + i) * 128, v[i]);
                 }
                 __threadfence();
@@ -470,80 +489,92 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm
                     }
                 }
                 ok = __all_sync(0xffffffffu, ok);
-                for (int c0 = 0; c0 < n_col && ok; c0 += 32) {
-                    float v[32];
-                    tmem_ld32(tl + c0, v);
-                    if (w.contributors) {
-                        float ps[32];
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) ps[i] = 0.f;
-                        for (int c = 1; c <= w.contributors; ++c) {
-                            const float* p = slot(pair + c);
-                            float x[32];
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) x[i] = c0 + i < n_col ? __ldcg(p + (size_t)(c0 + i) * 128) : 0.f;
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) ps[i] += x[i];
-                        }
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) v[i] += ps[i];
-                    }
+                // feature / rotation pair of this lane
+                const int hd = a.head_dim, half_d = hd >> 1;
+                const int ii = EPI == TC_QKV ? (q4 % (hd / 32)) * 16 + (lane & 15) : 0;
+                const int n = EPI == TC_SWIGLU ? box * 64 + q4 * 16 + (lane & 15) : box * 128 + q4 * 32 + lane;
+                for (int c0 = 0; c0 < n_col && ok; c0 += 16) {
                     const int tok = tok0 + c0;  // token row of v[0]
+                    // what the epilogue reads from memory is requested before the
+                    // accumulator and the partial sums are
+                    float h[EPI == TC_RESID ? 16 : 1];
+                    float2 cs[EPI == TC_QKV ? 8 : 1];
                     if (EPI == TC_RESID) {
-                        const int n = box * 128 + q4 * 32 + lane;
-                        if (n < a.N) {
-                            float* o = a.out + (size_t)tok * a.N + n;
-                            float h[32];
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) h[i] = c0 + i < n_col ? o[(size_t)i * a.N] : 0.f;
+                        for (int i = 0; i < 16; ++i)
+                            h[i] = c0 + i < n_col && n < a.N ? __ldcg(a.out + (size_t)(tok + i) * a.N + n) : 0.f;
+                    }
+                    if (EPI == TC_QKV) {
 #pragma unroll
-                            for (int i = 0; i < 32; ++i)
-                                if (c0 + i < n_col) o[(size_t)i * a.N] = h[i] + v[i];
+                        for (int j = 0; j < 8; ++j)
+                            cs[j] = c0 + 2 * j + upper < n_col
+                                        ? __ldg(a.rope + (size_t)(a.pos0 + tok + 2 * j + upper) * half_d + ii)
+                                        : make_float2(0.f, 0.f);
+                    }
+                    float ps[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) ps[i] = 0.f;
+                    for (int c = 1; c <= w.contributors; c += 2) {  // two ranges in flight, added in order
+                        const bool two = c < w.contributors;
+                        const float* p = slot(pair + c) + (size_t)c0 * 128;
+                        const float* p2 = slot(pair + (two ? c + 1 : c)) + (size_t)c0 * 128;
+                        float x[16], y[16];
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            x[i] = c0 + i < n_col ? __ldcg(p + i * 128) : 0.f;
+                            y[i] = c0 + i < n_col && two ? __ldcg(p2 + i * 128) : 0.f;
                         }
-                    } else if (EPI == TC_SWIGLU) {
-                        float g[16], u[16];
-                        pair_up(v, upper, g, u);
-                        const int f = box * 64 + q4 * 16 + (lane & 15);
-                        if (f < a.N) {
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) {
+                        for (int i = 0; i < 16; ++i) ps[i] = (ps[i] + x[i]) + y[i];
+                    }
+                    float v[16];
+                    tmem_ld16(tl + c0, v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[i] += ps[i];
+                    if (EPI == TC_RESID) {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            if (c0 + i < n_col && n < a.N) a.out[(size_t)(tok + i) * a.N + n] = h[i] + v[i];
+                    } else if (EPI == TC_SWIGLU) {
+                        float g[8], u[8];
+                        pair_up(v, upper, g, u);
+                        if (n < a.N) {
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
                                 const int c = 2 * j + upper;
                                 if (c0 + c >= n_col) continue;
-                                const float x = g[j] / (1.f + expf(-g[j])) * u[j];
-                                const size_t at = (size_t)(tok + c) * a.N + f;
+                                const float gt = a.swapped ? u[j] : g[j], up = a.swapped ? g[j] : u[j];
+                                const float x = gt / (1.f + expf(-gt)) * up;
+                                const size_t at = (size_t)(tok + c) * a.N + n;
                                 store_hilo(a.act_hi + at, a.act_lo + at, x);
                             }
                         }
                     } else {  // TC_QKV: this CTA's box is whole heads of q, k or v
-                        const int hd = a.head_dim, half_d = hd >> 1;
                         const int qd = a.n_heads * hd, kvd = a.n_kv_heads * hd;
                         const int f0 = box * 128;
                         const int kind = f0 < qd ? 0 : (f0 < qd + kvd ? 1 : 2);
                         const int head = (f0 - (kind == 0 ? 0 : (kind == 1 ? qd : qd + kvd))) / hd + q4 / (hd / 32);
-                        const int ii = (q4 % (hd / 32)) * 16 + (lane & 15);  // rotation pair (ii, ii + hd / 2)
                         if (f0 >= qd + 2 * kvd) continue;  // (uniform: past the last box)
                         if (kind == 2) {
                             f16* o = a.v_cache + ((size_t)head * a.max_seq + a.pos0 + tok) * hd + ii + upper * half_d;
 #pragma unroll
-                            for (int i = 0; i < 32; ++i)
+                            for (int i = 0; i < 16; ++i)
                                 if (c0 + i < n_col) o[(size_t)i * hd] = __float2half_rn(v[i]);
                         } else {
-                            float x1[16], x2[16];
+                            float x1[8], x2[8];
                             pair_up(v, upper, x1, x2);
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) {
+                            for (int j = 0; j < 8; ++j) {
                                 const int c = 2 * j + upper;
                                 if (c0 + c >= n_col) continue;
-                                const int pos = a.pos0 + tok + c;
-                                const float2 cs = a.rope[(size_t)pos * half_d + ii];
-                                const float y1 = x1[j] * cs.x - x2[j] * cs.y;
-                                const float y2 = x2[j] * cs.x + x1[j] * cs.y;
+                                const float y1 = x1[j] * cs[j].x - x2[j] * cs[j].y;
+                                const float y2 = x2[j] * cs[j].x + x1[j] * cs[j].y;
                                 if (kind == 0) {
                                     float* q = a.q + (size_t)(tok + c) * qd + head * hd;
                                     q[ii] = y1;
                                     q[ii + half_d] = y2;
                                 } else {
-                                    f16* k = a.k_cache + ((size_t)head * a.max_seq + pos) * hd;
+                                    f16* k = a.k_cache + ((size_t)head * a.max_seq + a.pos0 + tok + c) * hd;
                                     k[ii] = __float2half_rn(y1);
                                     k[ii + half_d] = __float2half_rn(y2);
                                 }
