@@ -287,7 +287,7 @@ int build_prefill(ssd_handle* h) {
     if (!fn || q != cudaDriverEntryPointSuccess) return fail(SSD_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
     auto enc = (PFN_cuTensorMapEncodeTiled_v12000)fn;
     const ssd_config& c = h->cfg;
-    const int L = c.n_layers, d = c.d_model, qd = c.n_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim;
+    const int L = c.n_layers, d = c.d_model, qd = c.n_heads * c.head_dim;
     PrefillPlan& P = h->pf;
     std::vector<CUtensorMap> maps((size_t)7 * L + 3 * kPfTokClasses);
     auto rows2 = [&](CUtensorMap* m, const void* base, int K, int rows, int box_rows) {

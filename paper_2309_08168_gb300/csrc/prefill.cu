@@ -304,7 +304,7 @@ int prefill_chunk(PrefillPlan& P, const int* toks, int n, int pos0, cudaStream_t
         a.rows = n;
         a.N = n_out;
         a.n_kb = (K + tc::kBK - 1) / tc::kBK;
-        tc::tc_plan(a, n_ft, P.pairs);
+        tc::tc_plan(a, n_ft, P.pairs, K);
         a.tm_x = tm_x[a.nt / 32 - 1];
         a.ws = P.ws;
         a.flags = P.flags;

@@ -607,32 +607,57 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm
     }
 }
 
-// Tile shape and schedule of a GEMM over `rows` tokens and n_ft feature tiles.
-// Tokens: as few tiles of at most 256 as hold the rows, of equal size rounded
-// up to 32.  Tiles that fill whole waves of pairs run whole; the rest is split
-// by k block over all pairs (with less than half a wave left, one more wave is
-// split with it, so that a tile is cut in two or three rather than many), in
-// pieces of at least kMinSplit k blocks.
-inline void tc_plan(TcArgs& a, int n_ft, int pairs) {
-    a.n_tt = (a.rows + kMaxTok - 1) / kMaxTok;
-    a.nt = ((a.rows + a.n_tt - 1) / a.n_tt + 31) / 32 * 32;
-    a.n_tt = (a.rows + a.nt - 1) / a.nt;
+// Tile shape and schedule of a GEMM over `rows` tokens and n_ft feature tiles
+// of K inputs: token tiles of equal size (a multiple of 32) and either whole
+// tiles only, pair by pair, or the tiles that do not fill a wave of pairs split
+// by k block over all of them (with less than half a wave left, one more wave
+// is split with it, so that a tile is cut in two or three rather than many), in
+// pieces of at least kMinSplit k blocks.  The choice with the least estimated
+// time, from times measured on GB300 at the 7B, 13B and 70B widths with 31 ..
+// 1535 rows (us):
+//   a k block of a tile     0.033 + 0.00222 nt, at least 0.24 (issue bound);
+//   the last tile's epilogue 5 nt / 256; of split tiles 13 nt / 256 + 4, the
+//                           partial sums' way through L2 included;
+//   split tiles walk K at offsets of their own: token planes of more than ~96
+//   MB do not stay in L2 and both operands come from HBM (6.8 TB/s).
+// Over those shapes the choice is within 1 % of the best measured one in the
+// sum (11034 of 10934 us; tiles of 256 tokens always split: 11.8 ms).
+inline void tc_plan(TcArgs& a, int n_ft, int pairs, int K) {
+    const int least = (a.rows + kMaxTok - 1) / kMaxTok;
+    double best = 1e30;
+    for (int n_tt = least; n_tt <= 4 * least; ++n_tt) {
+        const int nt = ((a.rows + n_tt - 1) / n_tt + 31) / 32 * 32;
+        if ((a.rows + nt - 1) / nt != n_tt) continue;
+        const int tiles = n_ft * n_tt, waves = tiles / pairs, rest = tiles % pairs;
+        const double t_kb = 0.033 + 0.00222 * nt > 0.24 ? 0.033 + 0.00222 * nt : 0.24;
+        for (int split = 0; split < 2; ++split) {
+            int n_split = 0, p = 1;
+            double us = (double)(waves + (rest ? 1 : 0)) * a.n_kb * t_kb + 5.0 * nt / 256;
+            if (split) {
+                if (rest == 0) continue;
+                n_split = waves > 0 && 2 * rest < pairs ? rest + pairs : rest;
+                const long long q = (long long)n_split * a.n_kb / kMinSplit;
+                p = q < pairs ? (int)q : pairs;
+                // too short for every pair: only useful if there is no whole wave
+                if (p < pairs && (waves > 0 || p <= rest)) continue;
+                double part = (double)n_split * a.n_kb / p * t_kb;
+                if (4e0 * a.rows * K > 96e6) {
+                    const double hbm = n_split * (512.0 * K + 4.0 * nt * K) / 6.8e6;
+                    if (hbm > part) part = hbm;
+                }
+                us = part + (double)((tiles - n_split) / pairs) * a.n_kb * t_kb + 13.0 * nt / 256 + 4;
+            }
+            if (us < best) {
+                best = us;
+                a.nt = nt;
+                a.n_tt = n_tt;
+                a.sched = {tiles, n_split, p, pairs};
+                if (tiles - n_split < pairs) a.sched.pairs = p > tiles - n_split ? p : tiles - n_split;
+            }
+        }
+    }
     const int stage = kATile + a.nt * 128;
     a.stages = kRingBytes / stage < kMaxStages ? kRingBytes / stage : kMaxStages;
-    TcSched& s = a.sched;
-    s.n_tiles = n_ft * a.n_tt;
-    const int waves = s.n_tiles / pairs, rest = s.n_tiles % pairs;
-    s.n_split = rest == 0 ? 0 : (waves > 0 && 2 * rest < pairs ? rest + pairs : rest);
-    long long p = (long long)s.n_split * a.n_kb / kMinSplit;
-    if (p > pairs) p = pairs;
-    if (p < rest) p = rest;  // (rest < pairs: at worst every tile is a range of its own)
-    if (p < 1) p = 1;
-    if (waves > 0 && s.n_split > rest && p < pairs) {  // too short to split: whole tiles only
-        s.n_split = 0;
-        p = 1;
-    }
-    s.split_pairs = (int)p;
-    s.pairs = s.n_tiles - s.n_split > 0 ? pairs : s.split_pairs;
 }
 
 template <int EPI>
