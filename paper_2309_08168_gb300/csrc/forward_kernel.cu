@@ -17,8 +17,8 @@
 // residual add, gate/up with SwiGLU, lm_head) run on the 5th-generation
 // tensor cores: work unit = 128-row tile x 128-wide k chunk (32 KB of
 // weights), each CTA owns an equal contiguous range of units in tile-major
-// order, streamed by TMA (128-byte swizzle) through a 5-stage ring; one
-// thread of the MMA warp issues tcgen05.mma kind::f16 per unit (M = 128 weight
+// order, streamed by TMA (128-byte swizzle) through a 5-stage ring; an
+// elected lane of the MMA warp issues tcgen05.mma kind::f16 per unit (M = 128 weight
 // rows, N = the activation rows as bf16 hi + lo planes, ~16 mantissa bits of
 // the fp32 activations) into a TMEM accumulator and releases the stage with
 // tcgen05.commit; the consumer warps read a finished tile segment from TMEM
@@ -392,7 +392,7 @@ __device__ __forceinline__ TileSrc tile_src(const GemmArgs& a, int epi, int tile
     return {0, tile * kFTile, -1, 0};
 }
 
-// weights of unit u into a stage (one thread): expect_tx without arriving.
+// weights of unit u into a stage (one lane): expect_tx without arriving.
 // Always a full 128 x 128 tile of bytes (rows / columns out of range are
 // delivered as zeros and counted).  Every x used here is a multiple of 64
 // elements (128 bytes), so the 16-byte rule for x * element size holds.
@@ -408,7 +408,7 @@ __device__ __forceinline__ void tma_weights(const GemmArgs& a, int epi, int u, u
     }
 }
 
-// input planes of unit u into a stage (one thread): arrive + expect_tx
+// input planes of unit u into a stage (one lane): arrive + expect_tx
 template <int R>
 __device__ __forceinline__ void tma_inputs(const GemmArgs& a, int u, unsigned char* st, uint64_t* bar) {
     using L = GemmSmem<R>;
@@ -449,7 +449,7 @@ __device__ __forceinline__ void advance_full(Pipe& pp, int n) {
         if (((n / S) + (s < n % S ? 1 : 0)) & 1) pp.cphase ^= 1u << s;
 }
 
-// Producer: requests the weights of this CTA's first S units of a projection
+// Producer warp: requests the weights of this CTA's first S units of a projection
 // before the grid barrier (they do not depend on the previous op).
 // n_pre: how many (at most the ring's depth) are requested.
 template <int R>
@@ -458,22 +458,22 @@ __device__ bool gemm_prefetch(const GemmArgs& a, int epi, unsigned char* smem, P
     int u_begin, n_my;
     my_units(a.n_units, &u_begin, &n_my);
     bool ok = true;
-    if (threadIdx.x == kConsumers) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        prefetch_tmap(a.tm_x[plane_cls(R)]);
-        for (int s = 0; s < S && s < n_pre && s < n_my && ok; ++s) {
-            ok = mbar_wait(pp.empty + s, (pp.pphase >> s) & 1u, err);
-            if (!ok) break;
-            pp.pphase ^= 1u << s;
-            tma_weights<R>(a, epi, u_begin + s, smem + s * GemmSmem<R>::STAGE, pp.full + s);
-        }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (elect_one()) prefetch_tmap(a.tm_x[plane_cls(R)]);
+    __syncwarp();
+    for (int s = 0; s < S && s < n_pre && s < n_my; ++s) {
+        ok = __all_sync(0xffffffffu, mbar_wait(pp.empty + s, (pp.pphase >> s) & 1u, err));
+        if (!ok) break;
+        pp.pphase ^= 1u << s;
+        if (elect_one()) tma_weights<R>(a, epi, u_begin + s, smem + s * GemmSmem<R>::STAGE, pp.full + s);
+        __syncwarp();
     }
     return ok;
 }
 
 // Returns false if a wait timed out (error recorded).  Three roles:
-//   producer (one thread of warp 8) streams this CTA's units through the ring;
-//   MMA issuer (one thread of warp 9) runs tcgen05.mma per unit into the
+//   producer (warp 8, one elected lane) streams this CTA's units through the ring;
+//   MMA issuer (warp 9, one elected lane) runs tcgen05.mma per unit into the
 //     accumulator of the unit's tile segment;
 //   consumers (warps 0-7), per finished segment: TMEM -> hi + lo summed ->
 //     split-K exchange -> epilogue (contributors and residual finalisers
@@ -496,27 +496,29 @@ __device__ bool gemm_op(const GemmArgs& a, int epi, int M, int pos0, int n_pre, 
     my_units(U, &u_begin, &n_my);
 
     if (threadIdx.x >= kConsumers && threadIdx.x < kConsumers + 32) {  // producer warp
-        if (threadIdx.x != kConsumers) return true;
         if (ut) ut[2] = globaltimer();
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("fence.proxy.async.global;" ::: "memory");  // inputs written by the previous op
         for (int i = 0; i < n_my; ++i) {
             const int s = i % S;
             unsigned char* st = smem + s * L::STAGE;
-            if (ut && i < 64) ut[i * 4 + 0] = globaltimer();
             if (i >= n_pre) {  // (the first n_pre units' weights were requested before the op)
-                if (!mbar_wait(pp.empty + s, (pp.pphase >> s) & 1u, err)) return false;
+                if (!__all_sync(0xffffffffu, mbar_wait(pp.empty + s, (pp.pphase >> s) & 1u, err))) return false;
                 pp.pphase ^= 1u << s;
-                tma_weights<R>(a, epi, u_begin + i, st, pp.full + s);
             }
-            tma_inputs<R>(a, u_begin + i, st, pp.full + s);
+            if (elect_one()) {
+                if (ut && i < 64) ut[i * 4 + 0] = globaltimer();
+                if (i >= n_pre) tma_weights<R>(a, epi, u_begin + i, st, pp.full + s);
+                tma_inputs<R>(a, u_begin + i, st, pp.full + s);
+            }
+            __syncwarp();
         }
         return true;
     }
 
-    if (threadIdx.x >= kConsumers + 32) {  // MMA warp: one elected thread issues
-        if (threadIdx.x != kConsumers + 32) return true;
+    if (threadIdx.x >= kConsumers + 32) {  // MMA warp: one elected lane issues
         constexpr uint32_t idesc = umma_idesc(NP);
+        const uint64_t desc0 = umma_desc(smem_u32(smem));  // (descriptors count 16-byte steps)
         for (int i = 0; i < n_my; ++i) {
             const int u = u_begin + i;
             const int chunk = u % a.n_chunks;
@@ -524,27 +526,28 @@ __device__ bool gemm_op(const GemmArgs& a, int epi, int M, int pos0, int n_pre, 
             const bool last = i == n_my - 1 || chunk == a.n_chunks - 1;
             const int ab = pp.ab;
             if (first) {  // the consumers have read this accumulator's previous segment
-                if (!mbar_wait(pp.acc_empty + ab, (pp.aempty >> ab) & 1u, err)) return false;
+                if (!__all_sync(0xffffffffu, mbar_wait(pp.acc_empty + ab, (pp.aempty >> ab) & 1u, err))) return false;
                 pp.aempty ^= 1u << ab;
             }
             const int s = i % S;
-            if (!mbar_wait(pp.full + s, (pp.cphase >> s) & 1u, err)) return false;
+            if (!__all_sync(0xffffffffu, mbar_wait(pp.full + s, (pp.cphase >> s) & 1u, err))) return false;
             pp.cphase ^= 1u << s;
             tc_fence_after();
-            const uint32_t st = smem_u32(smem + s * L::STAGE);
-            const uint32_t d = pp.tmem + (uint32_t)(ab * (kTmemCols / 2));
+            if (elect_one()) {
+                const uint64_t st = desc0 + (uint64_t)((uint32_t)(s * L::STAGE) >> 4);
+                const uint32_t d = pp.tmem + (uint32_t)(ab * (kTmemCols / 2));
 #pragma unroll
-            for (int kb = 0; kb < 2; ++kb)
+                for (int kb = 0; kb < 2; ++kb)
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks)
-                    umma(d, umma_desc(st + kb * 16384 + ks * 32), umma_desc(st + L::WB + kb * L::XKB + ks * 32),
-                         idesc, (first && kb == 0 && ks == 0) ? 0u : 1u);
-            umma_commit(pp.empty + s);  // the stage is free once these MMAs have read it
-            if (ut && i < 64) ut[i * 4 + 1] = globaltimer();
-            if (last) {
-                umma_commit(pp.acc_full + ab);
-                pp.ab ^= 1;
+                    for (int ks = 0; ks < 4; ++ks)
+                        umma(d, st + (kb * 16384 + ks * 32) / 16, st + (L::WB + kb * L::XKB + ks * 32) / 16, idesc,
+                             (first && kb == 0 && ks == 0) ? 0u : 1u);
+                umma_commit(pp.empty + s);  // the stage is free once these MMAs have read it
+                if (ut && i < 64) ut[i * 4 + 1] = globaltimer();
+                if (last) umma_commit(pp.acc_full + ab);
             }
+            __syncwarp();
+            if (last) pp.ab ^= 1;
         }
         return true;
     }
@@ -888,7 +891,7 @@ __device__ __forceinline__ AttnRange attn_range(const AttnArgs& a, int M, int po
     return r;
 }
 
-// Producer thread: requests K / V of this CTA's chunks at ring positions
+// Producer warp: requests K / V of this CTA's chunks at ring positions
 // [i_from, i_limit), in item order; with old_only it stops at the first chunk
 // holding rows this forward writes (those need the q/k/v op to be finished).
 // Returns the ring position reached, or -1 if a wait timed out.
@@ -905,14 +908,17 @@ __device__ int attn_produce(const AttnArgs& a, const AttnRange& ar, int pos0, un
             if (i >= i_limit || (old_only && (c + 1) * kAttnChunk > pos0)) return i;
             const int s = i % S;
             unsigned char* st = smem + s * L::STAGE;
-            if (!mbar_wait(pp.empty + s, (pp.pphase >> s) & 1u, err)) return -1;
+            if (!__all_sync(0xffffffffu, mbar_wait(pp.empty + s, (pp.pphase >> s) & 1u, err))) return -1;
             pp.pphase ^= 1u << s;
-            mbar_arrive_expect_tx(pp.full + s, 2u * (HD / 64) * 8192u);
+            if (elect_one()) {
+                mbar_arrive_expect_tx(pp.full + s, 2u * (HD / 64) * 8192u);
 #pragma unroll
-            for (int bx = 0; bx < HD / 64; ++bx) {
-                tma_load_3d(st + bx * 8192, a.tm_k, bx * 64, c * kAttnChunk, a.kv_z0 + kvh, pp.full + s);
-                tma_load_3d(st + 16384 + bx * 8192, a.tm_v, bx * 64, c * kAttnChunk, a.kv_z0 + kvh, pp.full + s);
+                for (int bx = 0; bx < HD / 64; ++bx) {
+                    tma_load_3d(st + bx * 8192, a.tm_k, bx * 64, c * kAttnChunk, a.kv_z0 + kvh, pp.full + s);
+                    tma_load_3d(st + 16384 + bx * 8192, a.tm_v, bx * 64, c * kAttnChunk, a.kv_z0 + kvh, pp.full + s);
+                }
             }
+            __syncwarp();
         }
     }
     return i;
@@ -920,15 +926,15 @@ __device__ int attn_produce(const AttnArgs& a, const AttnRange& ar, int pos0, un
 
 // Before the grid barrier ahead of an attention op: the producer requests the
 // K / V chunks of its first ring stages that hold only rows of earlier
-// forwards.  Returns how many (0 for other threads, -1 on a timeout).
+// forwards.  Returns how many (-1 on a timeout).
 template <int R, int HD>
 __device__ int attn_prefetch(const AttnArgs& a, int M, int pos0, unsigned char* smem, Pipe& pp, int* err) {
-    if (threadIdx.x != kConsumers) return 0;
     const AttnRange ar = attn_range(a, M, pos0);
-    if (ar.i_begin < ar.i_end) {
+    if (ar.i_begin < ar.i_end && elect_one()) {
         prefetch_tmap(a.tm_k);
         prefetch_tmap(a.tm_v);
     }
+    __syncwarp();
     return attn_produce<R, HD>(a, ar, pos0, smem, pp, err, 0, GemmSmem<R>::S, true);
 }
 
@@ -944,18 +950,15 @@ __device__ bool attn_op(const AttnArgs& a, int M, int pos0, unsigned char* smem,
     const AttnRange ar = attn_range(a, M, pos0);
 
     if (threadIdx.x >= kConsumers + 32) {  // MMA warp: only keeps its copy of the ring parities
-        if (threadIdx.x == kConsumers + 32) {
-            int n = 0;
-            for (int it = ar.i_begin; it < ar.i_end; ++it) {
-                const int sg = it % ar.n_seg;
-                n += min(SC, ar.n_ch - sg * SC);
-            }
-            advance_full<S>(pp, n);
+        int n = 0;
+        for (int it = ar.i_begin; it < ar.i_end; ++it) {
+            const int sg = it % ar.n_seg;
+            n += min(SC, ar.n_ch - sg * SC);
         }
+        advance_full<S>(pp, n);
         return true;
     }
-    if (threadIdx.x >= kConsumers) {  // producer warp: one elected thread requests K / V
-        if (threadIdx.x != kConsumers) return true;
+    if (threadIdx.x >= kConsumers) {  // producer warp: one elected lane requests K / V
         // K / V rows of this forward were stored by other CTAs (generic proxy)
         if (ar.i_begin < ar.i_end) asm volatile("fence.proxy.async.global;" ::: "memory");
         return attn_produce<R, HD>(a, ar, pos0, smem, pp, err, pre, 1 << 30, false) >= 0;
@@ -1433,7 +1436,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams
                 asm volatile("cp.async.wait_all;" ::: "memory");
                 __syncwarp();
             }
-            if (plane == 0 && nx && is_gemm(nx->type)) {
+            if (plane >= 0 && nx && is_gemm(nx->type)) {
                 ok = gemm_prefetch<R>(nx->g, epi_of(nx->type), smem, pp, p.err, GemmSmem<R>::S);
                 early = true;
             }
@@ -1465,7 +1468,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams
         }
         n_pre = 0;
         attn_pre = 0;
-        if (plane == 0 && nx) {
+        if (plane >= 0 && nx) {
             if (is_gemm(nx->type)) {
                 n_pre = (early || kBoundaryPrefetch > GemmSmem<R>::S) ? GemmSmem<R>::S : kBoundaryPrefetch;
                 if (!early) ok = gemm_prefetch<R>(nx->g, epi_of(nx->type), smem, pp, p.err, n_pre);
