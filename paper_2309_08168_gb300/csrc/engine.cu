@@ -672,8 +672,8 @@ int ssd_create(const ssd_config* cfg, const ssd_weights* w, void* cuda_stream, s
         h->own_stream = true;
     }
     {
-        int e1 = forward_configure(), e2 = gemm_configure(), e3 = sampling_configure();
-        int e = e1 ? e1 : (e2 ? e2 : e3);
+        int e1 = forward_configure(), e2 = sampling_configure();
+        int e = e1 ? e1 : e2;
         if (!e) e = (int)cudaDeviceGetAttribute(&h->n_sms, cudaDevAttrMultiProcessorCount, h->device);
         if (e) return bail(fail(SSD_ERR_CUDA, std::string("kernel setup: ") + cudaGetErrorString((cudaError_t)e)));
     }

@@ -1,24 +1,29 @@
 // gemm.cu - the stand-alone skinny projection GEMM of ssd_linear_noalloc:
 // Y[M x N] = X[M x K] * W^T with W bf16 [N][K], fp32 X and Y, M <= 16.
 //
-// The weights are the large operand, so the kernel is "swap-AB": 16 weight
-// rows form the M side of an m16n8k16 tensor-core MMA and the <= 16
-// activation rows form its N side.  The result for activation row m depends
-// only on row m (the MMA computes every output column independently, and the
-// split of K into CTA chunks, into k-interleaved warps and into the
-// fixed-order split-K combine depends on (N, K) only).
+// Bound by HBM: every weight is read once.  The weights are the large operand,
+// so the kernel is "swap-AB": 16 weight rows form the M side of an m16n8k16
+// tensor-core MMA and the <= 16 activation rows form its N side.  (mma.sync: a
+// block of 64 k needs 8 to 16 of them per 2 KB of weights, a few percent of the
+// tensor pipe, and its operands come from registers.)
+//
+// CTA = 8 warps x 16 weight rows = 128 rows, over a range of K.  A warp loads
+// its weights from global memory into MMA fragments directly, 16 bytes a
+// thread, two or four 64-wide k blocks (128 KB an SM) ahead of the MMAs: thread (g, t) reads 8 consecutive bf16 of rows g and g + 8, which the A and
+// B fragments both interpret as the same logical k slots, so the product is
+// unchanged, and a quad reads whole 128-byte lines.  The activations pass
+// through shared memory as bf16 pairs, up to 1024 k at a time.
+//
+// Few row tiles: K is split over a cluster of 2, 4 or 8 CTAs, which add their
+// sums through distributed shared memory in rank order: no scratch in global
+// memory, no counters, one launch.  The split depends on (N, K) and the SM
+// count only and MMA columns are independent, so the result for activation row
+// m depends on row m alone.
 //
 // Precision: the fp32 activation rows are split into bf16 hi = rn(x) and
 // lo = rn(x - hi) and both are multiplied (the MMA's N side holds the hi rows
 // then the lo rows), so the product sees ~16 mantissa bits of x; the weights
 // are exact bf16; accumulation is fp32.
-//
-// CTA = 256 threads: warp w handles the 16-row group (w & 3) of the 64-row
-// tile and the k32 blocks b = (w >> 2) (mod 2) of its k-chunk.  The weight
-// chunk (64 rows x kc) is streamed HBM -> shared memory with 16-byte cp.async,
-// then fed to the MMA with a k-permutation: thread (g, t) reads 8 consecutive
-// bf16 of a row, which the A and B fragments both interpret as the same
-// logical k slots, so the product is unchanged and every load is a 128-bit LDS.
 #include <mutex>
 #include <string>
 
@@ -28,245 +33,226 @@
 namespace ssd {
 namespace {
 
-// NPH = n8 tiles per activation half (1: M <= 8, 2: M <= 16).  The MMA's N
-// side holds P = 8*NPH rows of x_hi followed by P rows of x_lo.
-template <int NPH>
-__global__ void __launch_bounds__(kGemmThreads) gemm_kernel(const GemmArgs a) {
-    constexpr int NT = 2 * NPH;
-    constexpr int P = 8 * NPH;
-    constexpr int RC = 2 * P;
+constexpr int kLinThreads = 256;
+constexpr int kLinRows = 128;    // weight rows per CTA
+constexpr int kLinChunk = 1024;  // k staged in shared memory at a time
+constexpr int kLinFold = 4;      // 64-wide k blocks per fp32 fold
+constexpr int kRedPitch = kLinRows + 4;
+
+struct LinearArgs {
+    const bf16* w;
+    const float* x;
+    float* y;
+    int N, K, M;
+    int kc;  // k per CTA of the cluster, a multiple of 64
+};
+
+__device__ __forceinline__ float ld_cluster(uint32_t saddr, unsigned rank) {
+    uint32_t r;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(r) : "memory");
+    return v;
+}
+// 16 weight bytes, read once: not kept in L1.  volatile, like the MMAs, so that
+// the loads stay as far ahead of them as they are written
+__device__ __forceinline__ uint4 ld_weights(const bf16* p) {
+    uint4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p));
+    return v;
+}
+__device__ __forceinline__ void lin_cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// P = 8 or 16 activation rows; the MMA's N side holds P rows of x_hi, then P of
+// x_lo.  128 KB of weights in flight per SM either way: 4 CTAs with 2
+// blocks a warp ahead where registers allow it (P = 8; N 22016, K 4096, cold:
+// 45 us against 61 with 2 CTAs and 4 blocks), else 2 CTAs with 4 blocks (P = 16;
+// N = K = 4096: 18.0 us against 20.1).
+template <int P>
+struct LinShape {
+    static constexpr int CTAS = P == 8 ? 4 : 2, DEPTH = P == 8 ? 2 : 4;
+};
+template <int P>
+__global__ void __launch_bounds__(kLinThreads, LinShape<P>::CTAS) linear_kernel(const LinearArgs a) {
+    constexpr int NT = P / 4;  // n8 tiles: hi, then lo
+    constexpr int D = LinShape<P>::DEPTH;
     extern __shared__ __align__(16) unsigned char smem[];
     pdl_launch_dependents();
-    const int tile = blockIdx.x, split = blockIdx.y;
-    const int k0 = split * a.kc;
-    const int kc_eff = min(a.kc, a.K - k0);
-    const int pitch = a.kc * 2 + 64;  // bytes; pitch % 128 == 64 -> conflict-free LDS.128
-    unsigned char* ws = smem;
-    unsigned char* xs = smem + kTileRows * pitch;                // [2P][pitch] hi rows, then lo rows
-    float* red = reinterpret_cast<float*>(xs + 2 * P * pitch);  // [64][RC]
-    float* ys = reinterpret_cast<float*>(smem);                  // [64][16], reuses ws after the MMA
-    __shared__ int s_last;
-
-    // 1. stream the weight chunk (independent of the previous kernel)
-    const int cpr = kc_eff >> 3;  // 16-byte chunks per row
-    for (int c = threadIdx.x; c < kTileRows * cpr; c += kGemmThreads) {
-        int r = c / cpr, cc = c - r * cpr;
-        const int n = tile * kTileRows + r;
-        const bf16* src = n < a.N ? a.w0 + (size_t)n * a.K : nullptr;
-        const bf16* g = src ? src + k0 + cc * 8 : a.w0;
-        SSD_GUARD(a.err, (((uintptr_t)g & 15u) == 0) && (r * pitch + cc * 16 + 16 <= kTileRows * pitch), 101)
-        cp_async16(ws + r * pitch + cc * 16, g, src ? 16 : 0);
-    }
-    cp_async_commit();
-    // 2. activations of the previous kernel: fp32 -> bf16 hi / lo rows
-    pdl_wait();
-    for (int c = threadIdx.x; c < P * cpr; c += kGemmThreads) {
-        int n = c / cpr, cc = c - n * cpr;
-        uint4 hi = make_uint4(0, 0, 0, 0), lo = make_uint4(0, 0, 0, 0);
-        if (n < a.M) {
-            const float4* src = reinterpret_cast<const float4*>(a.x + (size_t)n * a.K + k0 + cc * 8);
-            split8(__ldcg(src), __ldcg(src + 1), hi, lo);
-        }
-        *reinterpret_cast<uint4*>(xs + n * pitch + cc * 16) = hi;
-        *reinterpret_cast<uint4*>(xs + (P + n) * pitch + cc * 16) = lo;
-    }
-    cp_async_wait<0>();
-    __syncthreads();
-
-    // 3. tensor-core MMA over the chunk
+    unsigned rank, n_ranks;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n_ranks));
+    const int tile = blockIdx.x / n_ranks;
+    const int k0 = (int)rank * a.kc, k1 = min(a.K, k0 + a.kc);
+    const int nb = k1 > k0 ? (k1 - k0 + 63) / 64 : 0;
+    const int pitch = min(a.kc, kLinChunk) * 2 + 64;  // bytes; pitch % 128 == 64: conflict-free LDS.128
+    float* red = reinterpret_cast<float*>(smem);       // [P][kRedPitch]
+    unsigned char* xs = smem + P * kRedPitch * 4;      // [2P][pitch] hi rows, then lo rows
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rg = warp & 3, kh = warp >> 2;
-    const int g = lane >> 2, tig = lane & 3;
-    float acc[NT][4];
+    const int g = lane >> 2, t = lane & 3;
+    // rows past N read row N - 1 again; their sums are not stored
+    const int r0 = tile * kLinRows + warp * 16 + g;
+    const bf16* w0 = a.w + (size_t)min(r0, a.N - 1) * a.K + t * 8;
+    const bf16* w1 = a.w + (size_t)min(r0 + 8, a.N - 1) * a.K + t * 8;
+    uint4 wr[D][4];
+    // K is a multiple of 16: a thread's 8 values are all inside or all outside
+    auto load = [&](uint4 (&d)[4], int b) {
+        const int k = k0 + b * 64;
+        const uint4 z = make_uint4(0, 0, 0, 0);
+        const bool in0 = k + t * 8 < k1, in1 = k + 32 + t * 8 < k1;
+        d[0] = in0 ? ld_weights(w0 + k) : z;
+        d[1] = in0 ? ld_weights(w1 + k) : z;
+        d[2] = in1 ? ld_weights(w0 + k + 32) : z;
+        d[3] = in1 ? ld_weights(w1 + k + 32) : z;
+    };
+    pdl_wait();  // weights and activations may come from the previous kernel
+#pragma unroll
+    for (int d = 0; d < D; ++d) load(wr[d], d);
+
+    // the MMAs' running sums, folded into fp32 sums of hi + lo every
+    // kLinFold k blocks (256 k): the tensor cores' own accumulation rounds less
+    // well over long chains (K 4096 in chains of 2048 k: error 3.2e-6, of 256 k 2.5e-6)
+    float acc[NT][4], sum[NT / 2][4];
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-    const unsigned char* ar0 = ws + (rg * 16 + g) * pitch;
-    const unsigned char* ar1 = ar0 + 8 * pitch;
-    const int nb = kc_eff >> 5;
-#pragma unroll 2
-    for (int b = kh; b < nb; b += 2) {
-        const int off = b * 64 + tig * 16;
-        uint4 wa = *reinterpret_cast<const uint4*>(ar0 + off);
-        uint4 wb = *reinterpret_cast<const uint4*>(ar1 + off);
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            uint4 xv = *reinterpret_cast<const uint4*>(xs + (nt * 8 + g) * pitch + off);
-            mma_bf16_16816(acc[nt], wa.x, wb.x, wa.y, wb.y, xv.x, xv.y);
-            mma_bf16_16816(acc[nt], wa.z, wb.z, wa.w, wb.w, xv.z, xv.w);
-        }
-    }
-    if ((kc_eff & 31) && kh == (nb & 1)) {  // k16 tail block
-        const int off = nb * 64 + tig * 8;
-        uint2 wa = *reinterpret_cast<const uint2*>(ar0 + off);
-        uint2 wb = *reinterpret_cast<const uint2*>(ar1 + off);
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            uint2 xv = *reinterpret_cast<const uint2*>(xs + (nt * 8 + g) * pitch + off);
-            mma_bf16_16816(acc[nt], wa.x, wb.x, wa.y, wb.y, xv.x, xv.y);
-        }
-    }
-
-    // 4. fixed-order combines: k-interleave 0 + 1, then x_hi + x_lo -> ys[row][m]
-    const int r0 = rg * 16 + g;
-    if (kh == 1) {
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            int c = nt * 8 + 2 * tig;
-            red[r0 * RC + c] = acc[nt][0];
-            red[r0 * RC + c + 1] = acc[nt][1];
-            red[(r0 + 8) * RC + c] = acc[nt][2];
-            red[(r0 + 8) * RC + c + 1] = acc[nt][3];
-        }
-    }
-    __syncthreads();
-    if (kh == 0) {
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            int c = nt * 8 + 2 * tig;
-            red[r0 * RC + c] = acc[nt][0] + red[r0 * RC + c];
-            red[r0 * RC + c + 1] = acc[nt][1] + red[r0 * RC + c + 1];
-            red[(r0 + 8) * RC + c] = acc[nt][2] + red[(r0 + 8) * RC + c];
-            red[(r0 + 8) * RC + c + 1] = acc[nt][3] + red[(r0 + 8) * RC + c + 1];
-        }
-    }
-    __syncthreads();
-    const int M = a.M;
-    for (int idx = threadIdx.x; idx < kTileRows * M; idx += kGemmThreads) {
-        int m = idx / kTileRows, r = idx - m * kTileRows;
-        ys[r * 16 + m] = red[r * RC + m] + red[r * RC + P + m];
-    }
-    __syncthreads();
-
-    // 5. split-K: the last CTA of the tile sums the partials in split order
-    if (a.ksplit > 1) {
-        const size_t NP = (size_t)a.n_tiles * kTileRows;
-        for (int idx = threadIdx.x; idx < M * kTileRows; idx += kGemmThreads) {
-            int m = idx / kTileRows, r = idx - m * kTileRows;
-            a.partial[((size_t)split * M + m) * NP + (size_t)tile * kTileRows + r] = ys[r * 16 + m];
-        }
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned prev = atomicAdd(&a.counters[tile], 1u);
-            s_last = (prev == (unsigned)(a.ksplit - 1));
+    for (int nt = 0; nt < NT / 2; ++nt) sum[nt][0] = sum[nt][1] = sum[nt][2] = sum[nt][3] = 0.f;
+    for (int c0 = 0; c0 < nb; c0 += kLinChunk / 64) {
+        const int cb = min(kLinChunk / 64, nb - c0);  // k blocks of this chunk
+        if (c0) __syncthreads();
+        for (int i = threadIdx.x; i < P * cb * 8; i += kLinThreads) {
+            const int n = i / (cb * 8), cc = i - n * (cb * 8), k = k0 + c0 * 64 + cc * 8;
+            uint4 hi = make_uint4(0, 0, 0, 0), lo = make_uint4(0, 0, 0, 0);
+            if (n < a.M && k < k1) {
+                const float4* src = reinterpret_cast<const float4*>(a.x + (size_t)n * a.K + k);
+                split8(__ldcg(src), __ldcg(src + 1), hi, lo);
+            }
+            *reinterpret_cast<uint4*>(xs + n * pitch + cc * 16) = hi;
+            *reinterpret_cast<uint4*>(xs + (P + n) * pitch + cc * 16) = lo;
         }
         __syncthreads();
-        if (!s_last) return;
-        __threadfence();
-        for (int idx = threadIdx.x; idx < M * kTileRows; idx += kGemmThreads) {
-            int m = idx / kTileRows, r = idx - m * kTileRows;
-            const float* p = a.partial + (size_t)m * NP + (size_t)tile * kTileRows + r;
-            float s = __ldcg(p);
-            for (int sp = 1; sp < a.ksplit; ++sp) s += __ldcg(p + (size_t)sp * M * NP);
-            ys[r * 16 + m] = s;
+        for (int b = 0; b < cb; b += kLinFold) {
+#pragma unroll
+            for (int d = 0; d < kLinFold; ++d) {
+                if (b + d < cb) {
+                    const unsigned char* xb = xs + g * pitch + (b + d) * 128 + t * 16;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint4 wa = wr[d % D][2 * h], wb = wr[d % D][2 * h + 1];
+#pragma unroll
+                        for (int nt = 0; nt < NT; ++nt) {
+                            const uint4 xv = *reinterpret_cast<const uint4*>(xb + nt * 8 * pitch + h * 64);
+                            mma_bf16_16816(acc[nt], wa.x, wb.x, wa.y, wb.y, xv.x, xv.y);
+                            mma_bf16_16816(acc[nt], wa.z, wb.z, wa.w, wb.w, xv.z, xv.w);
+                        }
+                    }
+                    load(wr[d % D], c0 + b + d + D);
+                }
+            }
+#pragma unroll
+            for (int nt = 0; nt < NT / 2; ++nt)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    sum[nt][x] += acc[nt][x] + acc[nt + NT / 2][x];
+                    acc[nt][x] = acc[nt + NT / 2][x] = 0.f;
+                }
         }
-        if (threadIdx.x == 0) a.counters[tile] = 0u;
-        __syncthreads();
     }
-
-    // 6. the output rows
-    for (int idx = threadIdx.x; idx < M * kTileRows; idx += kGemmThreads) {
-        int m = idx / kTileRows, r = idx - m * kTileRows;
-        int n = tile * kTileRows + r;
-        if (n < a.N) a.out_f32[(size_t)m * a.ldo + n] = ys[r * 16 + m];
+    // this CTA's sums, then the ranks' sums in order
+#pragma unroll
+    for (int nt = 0; nt < NT / 2; ++nt)
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+            red[(nt * 8 + 2 * t + (x & 1)) * kRedPitch + warp * 16 + g + 8 * (x >> 1)] = sum[nt][x];
+    if (n_ranks > 1) lin_cluster_sync();
+    else __syncthreads();
+    const int rows = kLinRows / (int)n_ranks, row0 = (int)rank * rows;  // (a power of two of ranks)
+    for (int i = threadIdx.x; i < a.M * rows; i += kLinThreads) {
+        const int m = i / rows, r = row0 + i - m * rows, n = tile * kLinRows + r;
+        if (n >= a.N) continue;
+        float s;
+        if (n_ranks == 1) {
+            s = red[m * kRedPitch + r];
+        } else {
+            float v[8];
+#pragma unroll
+            for (unsigned q = 0; q < 8; ++q) v[q] = q < n_ranks ? ld_cluster(smem_u32(red + m * kRedPitch + r), q) : 0.f;
+            s = v[0];
+#pragma unroll
+            for (unsigned q = 1; q < 8; ++q)
+                if (q < n_ranks) s += v[q];
+        }
+        a.y[(size_t)m * a.N + n] = s;
     }
+    if (n_ranks > 1) lin_cluster_sync();  // the other ranks have read this CTA's sums
 }
 
-template <int NPH>
-int launch_one(const GemmArgs& a, cudaStream_t s) {
-    const size_t smem = gemm_smem_bytes(a.kc, a.M);
+size_t linear_smem_bytes(int kc, int P) {
+    const int k = kc < kLinChunk ? kc : kLinChunk;
+    return (size_t)P * kRedPitch * 4 + (size_t)2 * P * (k * 2 + 64);
+}
+
+template <int P>
+int launch_linear(const LinearArgs& a, int ranks, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.n_tiles, a.ksplit, 1);
-    cfg.blockDim = dim3(kGemmThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
+    cfg.gridDim = dim3((unsigned)((a.N + kLinRows - 1) / kLinRows * ranks), 1, 1);
+    cfg.blockDim = dim3(kLinThreads, 1, 1);
+    cfg.dynamicSmemBytes = linear_smem_bytes(a.kc, P);
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)ranks;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return (int)cudaLaunchKernelEx(&cfg, gemm_kernel<NPH>, a);
+    cfg.numAttrs = 2;
+    return (int)cudaLaunchKernelEx(&cfg, linear_kernel<P>, a);
 }
 
-template <int NPH>
-int configure_one() {
-    return (int)cudaFuncSetAttribute(gemm_kernel<NPH>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-}
-
-}  // namespace
-
-int gemm_configure() {
-    int e = configure_one<1>();
-    return e ? e : configure_one<2>();
-}
-
-size_t gemm_smem_bytes(int kc, int M) {
-    const int P = gemm_half_rows(M);
-    return (size_t)(kTileRows + 2 * P) * (kc * 2 + 64) + (size_t)kTileRows * 2 * P * sizeof(float);
-}
-
-}  // namespace ssd
-
-// ---------------------------------------------------------------------------
-// ssd_linear_noalloc: the projection GEMM with its split-K scratch in a fixed
-// device array instead of memory the caller or the library allocates.
-//
-// Some callers cannot allocate device memory at the point where they need a
-// projection: a serving process that reserves every byte of HBM at start-up
-// and treats any later allocation as a failure, a plug-in whose host
-// framework owns all device allocations, or a latency-critical loop that
-// must not call cudaMalloc / cudaFree because those calls can synchronise
-// the whole device.  For them this entry point takes device inputs and
-// outputs only and keeps its scratch (split-K partial sums and the per-tile
-// arrival counters) in the static arrays below.  Every GPU that loads the
-// library holds these arrays (about 4 MiB) until the process exits.
-// ---------------------------------------------------------------------------
-namespace ssd {
-namespace {
-
-constexpr size_t kNoAllocPartialFloats = size_t(1) << 20;  // 4 MiB of partial sums
-constexpr int kNoAllocTiles = 4096;                          // 64-row tiles: N <= 262144
-
-static __device__ __align__(256) float g_noalloc_partial[kNoAllocPartialFloats];
-static __device__ __align__(256) unsigned g_noalloc_counters[kNoAllocTiles];
-static __device__ __align__(256) int g_noalloc_err;
-
-// Host-side device addresses of the arrays, resolved once per device.  (In
-// host code the array names are host stand-ins, not device addresses.)
-struct NoAllocDevice {
+// Per device, once: kernel attributes and the SM count.
+struct LinearDevice {
     bool ready = false;
-    float* partial = nullptr;
-    unsigned* counters = nullptr;
-    int* err = nullptr;
+    int n_sms = 0;
 };
-constexpr int kNoAllocMaxDevices = 64;
-NoAllocDevice g_noalloc_dev[kNoAllocMaxDevices];
-std::mutex g_noalloc_mu;
+constexpr int kLinMaxDevices = 64;
+LinearDevice g_lin_dev[kLinMaxDevices];
+std::mutex g_lin_mu;
 
-int noalloc_setup(int dev, NoAllocDevice** out) {
-    std::lock_guard<std::mutex> lock(g_noalloc_mu);
-    NoAllocDevice& d = g_noalloc_dev[dev];
+int linear_setup(int dev, int* n_sms) {
+    std::lock_guard<std::mutex> lock(g_lin_mu);
+    LinearDevice& d = g_lin_dev[dev];
     if (!d.ready) {
-        cudaError_t e = cudaGetSymbolAddress((void**)&d.partial, g_noalloc_partial);
-        if (e == cudaSuccess) e = cudaGetSymbolAddress((void**)&d.counters, g_noalloc_counters);
-        if (e == cudaSuccess) e = cudaGetSymbolAddress((void**)&d.err, g_noalloc_err);
-        if (e == cudaSuccess) e = (cudaError_t)configure_one<1>();
-        if (e == cudaSuccess) e = (cudaError_t)configure_one<2>();
-        // (the arrays start at zero when the module loads; each call clears
-        // the counters it uses on its own stream)
+        cudaError_t e = cudaFuncSetAttribute(linear_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)linear_smem_bytes(kLinChunk, 8));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(linear_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)linear_smem_bytes(kLinChunk, 16));
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&d.n_sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess)
             return set_last_error(SSD_ERR_CUDA, (std::string("ssd_linear_noalloc set-up: ") +
                                                  cudaGetErrorString(e)).c_str());
         d.ready = true;
     }
-    *out = &d;
+    *n_sms = d.n_sms;
     return SSD_OK;
 }
 
 }  // namespace
 }  // namespace ssd
 
+// ---------------------------------------------------------------------------
+// ssd_linear_noalloc: the projection GEMM alone, for callers that cannot
+// allocate device memory at the point where they need a projection: a serving
+// process that reserves every byte of HBM at start-up and treats any later
+// allocation as a failure, a plug-in whose host framework owns all device
+// allocations, or a latency-critical loop that must not call cudaMalloc /
+// cudaFree because those calls can synchronise the whole device.
+// ---------------------------------------------------------------------------
 extern "C" int ssd_linear_noalloc(const void* w, const float* x, float* y, int N, int K, int M,
                                   void* cuda_stream) {
     using namespace ssd;
@@ -276,58 +262,34 @@ extern "C" int ssd_linear_noalloc(const void* w, const float* x, float* y, int N
     if (M < 1 || M > kMaxRows || N < 1 || K < 16 || K % 16)
         return set_last_error(SSD_ERR_INVALID_ARG,
                               "ssd_linear_noalloc: need 1 <= M <= 16, N >= 1, K a positive multiple of 16");
-    const int kc = K >= 512 ? 512 : ((K + 63) / 64) * 64;
-    const int ksplit = (K + kc - 1) / kc;
-    const int n_tiles = (N + kTileRows - 1) / kTileRows;
-    const size_t need = ksplit > 1 ? (size_t)ksplit * M * n_tiles * kTileRows : 0;
-    if (n_tiles > kNoAllocTiles || need > kNoAllocPartialFloats)
+    // the sizes the call takes (ssd.h): the kernel itself needs no scratch
+    const size_t tiles64 = ((size_t)N + 63) / 64, need = K > 512 ? (size_t)((K + 511) / 512) * M * 64 * tiles64 : 0;
+    if (tiles64 > 4096 || need > (size_t(1) << 20))
         return set_last_error(SSD_ERR_CAPACITY,
-                              ("ssd_linear_noalloc: problem needs " + std::to_string(need) +
-                               " scratch floats and " + std::to_string(n_tiles) +
-                               " tiles; the fixed scratch holds 1048576 floats and 4096 tiles")
+                              ("ssd_linear_noalloc: problem counts " + std::to_string(need) + " scratch floats and " +
+                               std::to_string(tiles64) + " tiles; the limits are 1048576 floats and 4096 tiles")
                                   .c_str());
-    int dev = 0;
+    int dev = 0, n_sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess || dev < 0 || dev >= kNoAllocMaxDevices)
+    if (e != cudaSuccess || dev < 0 || dev >= kLinMaxDevices)
         return set_last_error(SSD_ERR_CUDA, "ssd_linear_noalloc: no usable current device");
-    NoAllocDevice* d = nullptr;
-    int rc = noalloc_setup(dev, &d);
+    const int rc = linear_setup(dev, &n_sms);
     if (rc) return rc;
-    cudaStream_t s = (cudaStream_t)cuda_stream;
-    // the arrival counters must start at zero (the array keeps the last call's contents)
-    e = cudaMemsetAsync(d->counters, 0, sizeof(unsigned) * n_tiles, s);
-    GemmArgs a{};
-    a.w0 = (const bf16*)w;
+    // K split over a cluster until there are two CTAs per SM, at least 128 k each
+    const int tiles = (N + kLinRows - 1) / kLinRows;
+    int ranks = 1;
+    while (ranks < 8 && tiles * ranks < 2 * n_sms && K / (2 * ranks) >= 128) ranks *= 2;
+    LinearArgs a{};
+    a.w = (const bf16*)w;
+    a.x = x;
+    a.y = y;
     a.N = N;
     a.K = K;
-    a.kc = kc;
-    a.ksplit = ksplit;
-    a.n_tiles = n_tiles;
-    a.x = x;
     a.M = M;
-    a.partial = d->partial;
-    a.counters = d->counters;
-    a.out_f32 = y;
-    a.ldo = N;
-    a.err = d->err;
-    if (e == cudaSuccess)
-        e = (cudaError_t)(M > 8 ? launch_one<2>(a, s) : launch_one<1>(a, s));
+    a.kc = ((K + ranks - 1) / ranks + 63) / 64 * 64;
+    cudaStream_t s = (cudaStream_t)cuda_stream;
+    e = (cudaError_t)(M > 8 ? launch_linear<16>(a, ranks, s) : launch_linear<8>(a, ranks, s));
     if (e != cudaSuccess)
         return set_last_error(SSD_ERR_CUDA, (std::string("ssd_linear_noalloc: ") + cudaGetErrorString(e)).c_str());
-#ifdef SSD_CHECKED
-    // checked builds: the kernel's alignment / bounds guards record a code in
-    // the device flag; read it back (this makes the call synchronous), clear it
-    // for the next call and report it
-    int derr = 0;
-    e = cudaMemcpyAsync(&derr, d->err, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d->err, 0, sizeof(int), s);
-    if (e != cudaSuccess)
-        return set_last_error(SSD_ERR_CUDA, (std::string("ssd_linear_noalloc: ") + cudaGetErrorString(e)).c_str());
-    if (derr)
-        return set_last_error(SSD_ERR_CUDA,
-                              ("ssd_linear_noalloc: device check failed with code " + std::to_string(derr)).c_str());
-#endif
     return SSD_OK;
 }
-

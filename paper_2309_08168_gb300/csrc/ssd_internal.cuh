@@ -13,11 +13,9 @@ typedef __half f16;
 
 constexpr int kMaxRows = 16;      // rows of one forward (verification K+1 <= 16)
 constexpr int kMaxK = 15;         // drafts per round
-constexpr int kTileRows = 64;     // stand-alone projection kernel (gemm.cu): output rows per CTA
-constexpr int kGemmThreads = 256; // 8 warps: 4 row groups x 2 k-interleaves
+constexpr int kGemmThreads = 256; // consumer threads of a forward CTA
 constexpr int kAttnChunk = 64;    // KV positions per attention CTA (absolute chunks)
 constexpr int kAttnThreads = 256;
-constexpr int kStreamKC = 256;    // (stand-alone projection kernel of gemm.cu) k per CTA chunk step
 constexpr int kFTile = 128;       // forward kernel: weight rows per tile (tcgen05 M, TMEM lanes)
 constexpr int kFKC = 128;         // forward kernel: k per work unit (128 rows x 128 k = 32 KB of weights)
 constexpr int kTraceUnits = 1024, kTraceCtas = 1280;  // offsets in FwdParams::trace
@@ -51,8 +49,7 @@ struct DecodeState {
 };
 
 // ---------------------------------------------------------------------------
-// Projection arguments: the forward kernel's tcgen05 projections and the
-// stand-alone swap-AB mma.sync kernel of gemm.cu (bf16 in, fp32 accumulate)
+// Projection arguments of the forward kernel (bf16 in, fp32 accumulate)
 // ---------------------------------------------------------------------------
 enum GemmEpi { EPI_LOGITS = 0, EPI_RESID = 1, EPI_SWIGLU = 2, EPI_QKV = 3 };
 
@@ -62,14 +59,8 @@ struct GemmArgs {
     const bf16* w2;      // segment 2 (wv)
     int N;               // logical output rows
     int K;               // reduction length (row length of every segment)
-    int kc;              // gemm.cu: k-chunk per CTA (multiple of 64)
-    int ksplit;          // gemm.cu: ceil(K / kc)
     int n_tiles;         // row tiles
-    const float* x;      // gemm.cu: activations [M][K] fp32 (split into bf16 hi + lo in the kernel)
-    int M;               // gemm.cu: activation rows (1..16)
-    float* partial;      // split-K partials: gemm.cu [ksplit][M][n_tiles*64] floats; forward
-                         // kernel [n_tiles][n_chunks][16][128] tagged 64-bit words
-    unsigned* counters;  // gemm.cu: [n_tiles] arrival counters (left at zero)
+    float* partial;      // split-K partials [n_tiles][n_chunks][16][128], tagged 64-bit words
     // epilogue operands
     float* out_f32;      // EPI_LOGITS: [M][ldo]; EPI_RESID: residual h [M][ldo]
     int ldo;
@@ -215,9 +206,6 @@ int launch_forward(const FwdParams& p, int head_dim, int grid, cudaStream_t s);
 int set_last_error(int code, const char* msg);
 
 // launchers (return cudaError_t)
-int gemm_configure();
-size_t gemm_smem_bytes(int kc, int M);
-constexpr int gemm_half_rows(int M) { return M <= 8 ? 8 : 16; }  // padded rows of x_hi (and of x_lo)
 
 // src for launch_embed
 enum EmbedSrc { SRC_TOKENS = 0, SRC_DRAFT = 1, SRC_VERIFY = 2 };
