@@ -711,7 +711,7 @@ int ssd_create(const ssd_config* cfg, const ssd_weights* w, void* cuda_stream, s
     h->mask.assign(2 * L, 0);
 
     // plans
-    // split-K slots of the forward kernel: [tile][segment <= chunks][16][128] tagged words
+    // split-K slots of the forward kernel: [tile][segment <= chunks][kPartWords] tagged 128-bit words
     size_t part = 0;
     {
         const int Ks[5] = {d, qd, d, c.ffn, d};
@@ -719,7 +719,7 @@ int ssd_create(const ssd_config* cfg, const ssd_weights* w, void* cuda_stream, s
                               (c.vocab + kFTile - 1) / kFTile};
         for (int i = 0; i < 5; ++i) {
             const size_t chunks = (size_t)(Ks[i] + kFKC - 1) / kFKC;
-            part = std::max(part, chunks * kMaxRows * (size_t)tiles[i] * kFTile);
+            part = std::max(part, chunks * kPartWords * (size_t)tiles[i]);
         }
     }
     h->n_chunks = (c.max_seq + kAttnChunk - 1) / kAttnChunk;
@@ -739,7 +739,7 @@ int ssd_create(const ssd_config* cfg, const ssd_weights* w, void* cuda_stream, s
         (rc = dalloc(h, &h->logits, (size_t)kMaxRows * V, &B)) ||
         (rc = dalloc(h, &h->p_rows, (size_t)kMaxRows * V, &B)) ||
         (rc = dalloc(h, &h->q_rows, (size_t)kMaxRows * V, &B)) ||
-        (rc = dalloc(h, &h->partial, 2 * part, &B)) ||  // tagged 64-bit words in the forward kernel
+        (rc = dalloc(h, &h->partial, 4 * part, &B)) ||
         (rc = dalloc(h, &h->counters, (size_t)4, &B)) ||
         (rc = dalloc(h, &h->attn_part, (size_t)c.n_kv_heads * h->n_chunks * G * kMaxRows * attn_part_floats((int)HD), &B)) ||
         (rc = dalloc(h, &h->rope, (size_t)c.max_seq * (HD / 2), &B)) ||
@@ -780,7 +780,7 @@ int ssd_create(const ssd_config* cfg, const ssd_weights* w, void* cuda_stream, s
     // barrier counter and forward sequence number; split-K slots hold no
     // valid tag (a tag is never 0: GEMM ops have an op index >= 1)
     if (e == cudaSuccess) e = cudaMemsetAsync(h->bar, 0, 4 * sizeof(unsigned), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->partial, 0, 2 * part * sizeof(float), h->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->partial, 0, 4 * part * sizeof(float), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->kc, 0, h->kv_layer * L * sizeof(f16), h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->vc, 0, h->kv_layer * L * sizeof(f16), h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);

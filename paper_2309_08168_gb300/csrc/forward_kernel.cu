@@ -7,10 +7,12 @@
 // the step.  Instead one CTA per SM walks the forward's op list
 //     embed -> [QKV -> attention -> O] -> [gate/up -> down] -> ... -> lm_head
 // (sublayers in the skip set z are simply absent from the draft's list,
-// Sec. 3.2 / 3.3) with a grid barrier between dependent ops.  Once a CTA has
-// arrived at a barrier it requests the weights of its first units of the next
-// projection (they do not depend on the previous op), so the barrier's
-// latency overlaps HBM streaming.  Every wait is bounded: a barrier that does
+// Sec. 3.2 / 3.3) with a grid barrier between dependent ops.  The CTA's roles
+// (consumer warps, TMA producer, MMA issuer) walk the list on their own: once
+// the consumers have arrived at a barrier the producer requests the weights of
+// the CTA's first units of the next projection (they do not depend on the
+// previous op), so the barrier's latency overlaps HBM streaming, and it is told
+// by thread 0, not by a CTA barrier, that the inputs may be requested.  Every wait is bounded: a barrier that does
 // not complete within ~2 s records an error code and the CTAs return.
 //
 // Projections (all of them: q/k/v + RoPE + KV write, output and down with the
@@ -25,8 +27,12 @@
 // (tcgen05.ld) while the next segment accumulates in the other accumulator.
 // A tile split over several CTAs is summed in segment order by the CTA
 // holding its first chunks; the others store their partials tagged with the
-// op (value and tag in one 64-bit word), so they neither fence nor signal,
-// and the finaliser polls the words themselves.
+// op (three input rows' sums and the tag in one 128-bit word), so they neither
+// fence nor signal, and the finaliser polls the words themselves.  That exchange
+// is what an op's end waits for (weights of the next op in flight slow every L2
+// round trip to ~1.5 us), so it takes as few words and round trips as it can:
+// with a word per sum a 13-row verification of 4 layers at 13B widths took 640 us,
+// with a word per three rows 597 us.
 // RMSNorm is folded in: the producer of the residual stream writes the planes
 // of h * g_next and per-128-column sums of h^2, the consumer scales row m by
 // rsqrt(mean(h^2) + eps) in its epilogue (W (h g r) = r W (h g)).
@@ -61,8 +67,18 @@ constexpr unsigned long long kErrPollAfterNs = 20000ull;
 constexpr int kConsumers = 256;
 constexpr int kFwdThreads = kConsumers + 64;
 
-// barrier among the consumer warps only (the producer keeps streaming)
+// barrier among the consumer warps only (the producer and MMA warps go on)
 __device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// the same; true in every consumer thread if any of them passed true
+__device__ __forceinline__ bool consumer_or(bool x) {
+    unsigned r;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, 256, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+        : "=r"(r)
+        : "r"((unsigned)x)
+        : "memory");
+    return r != 0;
+}
 
 
 __device__ __forceinline__ unsigned long long globaltimer() {
@@ -107,21 +123,30 @@ __device__ bool grid_wait(unsigned* bar, unsigned target, int* err, unsigned lon
     return true;
 }
 
-// Split-K partials: a float and the tag of the op that wrote it (forward
-// sequence number << 10 | op index) in one 64-bit word, written and read as
-// single 64-bit accesses.
-__device__ __forceinline__ unsigned long long tagged(unsigned tag, float v) {
-    return ((unsigned long long)tag << 32) | __float_as_uint(v);
+// Split-K partials: up to three input rows' sums of a tile row and the tag of
+// the op that wrote them (forward sequence number << 10 | op index) in one
+// 128-bit word, written and read as single 128-bit accesses.
+struct PartWord {
+    unsigned long long lo, hi;  // rows 0, 1; row 2, tag
+};
+__device__ __forceinline__ unsigned tag_of(const PartWord& w) { return (unsigned)(w.hi >> 32); }
+__device__ __forceinline__ float value_of(const PartWord& w, int j) {
+    return __uint_as_float((unsigned)(j == 0 ? w.lo : j == 1 ? w.lo >> 32 : w.hi));
 }
-__device__ __forceinline__ unsigned tag_of(unsigned long long w) { return (unsigned)(w >> 32); }
-__device__ __forceinline__ float value_of(unsigned long long w) { return __uint_as_float((unsigned)w); }
-__device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+__device__ __forceinline__ void st_relaxed(PartWord* p, unsigned tag, float v0, float v1, float v2) {
+    const unsigned long long lo = (unsigned long long)__float_as_uint(v1) << 32 | __float_as_uint(v0);
+    const unsigned long long hi = (unsigned long long)tag << 32 | __float_as_uint(v2);
+    asm volatile("{\n .reg .b128 t;\n mov.b128 t, {%1, %2};\n st.relaxed.gpu.global.b128 [%0], t;\n}\n" ::"l"(p),
+                 "l"(lo), "l"(hi)
+                 : "memory");
 }
-__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
+__device__ __forceinline__ PartWord ld_relaxed(const PartWord* p) {
+    PartWord w;
+    asm volatile("{\n .reg .b128 t;\n ld.relaxed.gpu.global.b128 t, [%2];\n mov.b128 {%0, %1}, t;\n}\n"
+                 : "=l"(w.lo), "=l"(w.hi)
+                 : "l"(p)
+                 : "memory");
+    return w;
 }
 __device__ __forceinline__ int unit_owner(long long u, long long U, long long G) {
     return (int)(((u + 1) * G + U - 1) / U - 1);
@@ -428,6 +453,8 @@ __device__ __forceinline__ void tma_inputs(const GemmArgs& a, int u, unsigned ch
 //   afull bit b  : parity of the next completion of accumulator b (consumers)
 //   aempty bit b : parity of the next release of accumulator b (MMA thread)
 //   ab           : accumulator of the next tile segment
+//   rb           : ring stage of the op's first unit (the ring runs on from op
+//                  to op, so a stage is reused in the order it was released)
 struct Pipe {
     uint64_t* full;     // [stages] TMA completion (count 1: the producer's arrive)
     uint64_t* empty;    // [stages] stage released (count 1: tcgen05.commit, or consumer thread 0)
@@ -439,52 +466,129 @@ struct Pipe {
     unsigned afull;
     unsigned aempty;
     int ab;
+    int rb;
 };
 
-// flips the full-barrier parity bits of n consecutive ring positions from 0
+// ring stage of the op's unit i
+template <int S>
+__device__ __forceinline__ int ring_stage(const Pipe& pp, int i) {
+    return (pp.rb + i) % S;
+}
+// the op's n ring positions are used up
+template <int S>
+__device__ __forceinline__ void ring_advance(Pipe& pp, int n) {
+    pp.rb = (pp.rb + n) % S;
+}
+// flips the full-barrier parity bits of the op's n ring positions, whose waits
+// another role took
 template <int S>
 __device__ __forceinline__ void advance_full(Pipe& pp, int n) {
 #pragma unroll
-    for (int s = 0; s < S; ++s)
-        if (((n / S) + (s < n % S ? 1 : 0)) & 1) pp.cphase ^= 1u << s;
+    for (int k = 0; k < S; ++k)
+        if (((n / S) + (k < n % S ? 1 : 0)) & 1) pp.cphase ^= 1u << ring_stage<S>(pp, k);
 }
 
-// Producer warp: requests the weights of this CTA's first S units of a projection
-// before the grid barrier (they do not depend on the previous op).
-// n_pre: how many (at most the ring's depth) are requested.
-template <int R>
-__device__ bool gemm_prefetch(const GemmArgs& a, int epi, unsigned char* smem, Pipe& pp, int* err, int n_pre) {
-    constexpr int S = GemmSmem<R>::S;
-    int u_begin, n_my;
-    my_units(a.n_units, &u_begin, &n_my);
-    bool ok = true;
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    if (elect_one()) prefetch_tmap(a.tm_x[plane_cls(R)]);
-    __syncwarp();
-    for (int s = 0; s < S && s < n_pre && s < n_my; ++s) {
-        ok = __all_sync(0xffffffffu, mbar_wait(pp.empty + s, (pp.pphase >> s) & 1u, err));
-        if (!ok) break;
-        pp.pphase ^= 1u << s;
-        if (elect_one()) tma_weights<R>(a, epi, u_begin + s, smem + s * GemmSmem<R>::STAGE, pp.full + s);
-        __syncwarp();
-    }
-    return ok;
-}
-
-// Returns false if a wait timed out (error recorded).  Three roles:
+// A projection op in a CTA has three roles:
 //   producer (warp 8, one elected lane) streams this CTA's units through the ring;
 //   MMA issuer (warp 9, one elected lane) runs tcgen05.mma per unit into the
 //     accumulator of the unit's tile segment;
 //   consumers (warps 0-7), per finished segment: TMEM -> hi + lo summed ->
 //     split-K exchange -> epilogue (contributors and residual finalisers
 //     per warp from registers, the other finalisers through shared memory).
-// ut: nullptr, or [64][4] timestamps of this CTA's first units (producer
-// issue, MMAs issued, 0, segment flush done); ct: nullptr, or this CTA's op
-// stamps (FwdParams::trace) - profiling aids.
+// Each returns false if a wait timed out (error recorded).  ut: nullptr, or
+// [64][4] timestamps of this CTA's first units (producer issue, MMAs issued, 0,
+// segment flush done); ct: nullptr, or this CTA's op stamps (FwdParams::trace) -
+// profiling aids.
+
+// Producer warp, once the consumers have left the previous op: the weights of
+// the first S units, which depend on nothing, while the grid gathers; then the
+// inputs, once `go` says that the grid barrier has passed.
 template <int R>
-__device__ bool gemm_op(const GemmArgs& a, int epi, int M, int pos0, int n_pre, unsigned char* smem,
-                        float* r_s, Pipe& pp, unsigned tag, int* err, unsigned long long* ut,
-                        unsigned long long* ct) {
+__device__ bool gemm_produce(const GemmArgs& a, int epi, unsigned char* smem, Pipe& pp, uint64_t* go, unsigned go_parity,
+                             int* err, unsigned long long* ut) {
+    using L = GemmSmem<R>;
+    constexpr int S = L::S;
+    int u_begin, n_my;
+    my_units(a.n_units, &u_begin, &n_my);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (n_my > 0 && elect_one()) prefetch_tmap(a.tm_x[plane_cls(R)]);
+    __syncwarp();
+    const int n_pre = min(S, n_my);
+    for (int i = 0; i < n_pre; ++i) {
+        const int s = ring_stage<S>(pp, i);
+        if (!__all_sync(0xffffffffu, mbar_wait(pp.empty + s, (pp.pphase >> s) & 1u, err))) return false;
+        pp.pphase ^= 1u << s;
+        if (elect_one()) tma_weights<R>(a, epi, u_begin + i, smem + s * L::STAGE, pp.full + s);
+        __syncwarp();
+    }
+    if (!__all_sync(0xffffffffu, mbar_wait(go, go_parity, err))) return false;
+    if (ut) ut[2] = globaltimer();
+    asm volatile("fence.proxy.async.global;" ::: "memory");  // inputs written by the previous op
+    for (int i = 0; i < n_my; ++i) {
+        const int s = ring_stage<S>(pp, i);
+        unsigned char* st = smem + s * L::STAGE;
+        if (i >= n_pre) {
+            if (!__all_sync(0xffffffffu, mbar_wait(pp.empty + s, (pp.pphase >> s) & 1u, err))) return false;
+            pp.pphase ^= 1u << s;
+        }
+        if (elect_one()) {
+            if (ut && i < 64) ut[i * 4 + 0] = globaltimer();
+            if (i >= n_pre) tma_weights<R>(a, epi, u_begin + i, st, pp.full + s);
+            tma_inputs<R>(a, u_begin + i, st, pp.full + s);
+        }
+        __syncwarp();
+    }
+    ring_advance<S>(pp, n_my);
+    return true;
+}
+
+// MMA warp: n_units, n_chunks of the op
+template <int R>
+__device__ bool gemm_mma(int n_units, int n_chunks, unsigned char* smem, Pipe& pp, int* err, unsigned long long* ut) {
+    using L = GemmSmem<R>;
+    constexpr int S = L::S, NP = L::NP;
+    int u_begin, n_my;
+    my_units(n_units, &u_begin, &n_my);
+    constexpr uint32_t idesc = umma_idesc(NP);
+    const uint64_t desc0 = umma_desc(smem_u32(smem));  // (descriptors count 16-byte steps)
+    int chunk = u_begin % n_chunks;
+    for (int i = 0; i < n_my; ++i) {
+        const bool first = i == 0 || chunk == 0;
+        const bool last = i == n_my - 1 || chunk == n_chunks - 1;
+        chunk = chunk == n_chunks - 1 ? 0 : chunk + 1;
+        const int ab = pp.ab;
+        if (first) {  // the consumers have read this accumulator's previous segment
+            if (!__all_sync(0xffffffffu, mbar_wait(pp.acc_empty + ab, (pp.aempty >> ab) & 1u, err))) return false;
+            pp.aempty ^= 1u << ab;
+        }
+        const int s = ring_stage<S>(pp, i);
+        if (!__all_sync(0xffffffffu, mbar_wait(pp.full + s, (pp.cphase >> s) & 1u, err))) return false;
+        pp.cphase ^= 1u << s;
+        tc_fence_after();
+        if (elect_one()) {
+            const uint64_t st = desc0 + (uint64_t)((uint32_t)(s * L::STAGE) >> 4);
+            const uint32_t d = pp.tmem + (uint32_t)(ab * (kTmemCols / 2));
+#pragma unroll
+            for (int kb = 0; kb < 2; ++kb)
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks)
+                    umma(d, st + (kb * 16384 + ks * 32) / 16, st + (L::WB + kb * L::XKB + ks * 32) / 16, idesc,
+                         (first && kb == 0 && ks == 0) ? 0u : 1u);
+            umma_commit(pp.empty + s);  // the stage is free once these MMAs have read it
+            if (ut && i < 64) ut[i * 4 + 1] = globaltimer();
+            if (last) umma_commit(pp.acc_full + ab);
+        }
+        __syncwarp();
+        if (last) pp.ab ^= 1;
+    }
+    ring_advance<S>(pp, n_my);
+    return true;
+}
+
+// Consumer warps
+template <int R>
+__device__ bool gemm_consume(const GemmArgs& a, int epi, int M, int pos0, unsigned char* smem, float* r_s, Pipe& pp,
+                             unsigned tag, int* err, unsigned long long* ut, unsigned long long* ct) {
     using L = GemmSmem<R>;
     constexpr int S = L::S, NP = L::NP;
     float* ys = reinterpret_cast<float*>(smem + L::YS);  // [128][16]
@@ -494,63 +598,6 @@ __device__ bool gemm_op(const GemmArgs& a, int epi, int M, int pos0, int n_pre, 
     const int b = blockIdx.x;
     int u_begin, n_my;
     my_units(U, &u_begin, &n_my);
-
-    if (threadIdx.x >= kConsumers && threadIdx.x < kConsumers + 32) {  // producer warp
-        if (ut) ut[2] = globaltimer();
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("fence.proxy.async.global;" ::: "memory");  // inputs written by the previous op
-        for (int i = 0; i < n_my; ++i) {
-            const int s = i % S;
-            unsigned char* st = smem + s * L::STAGE;
-            if (i >= n_pre) {  // (the first n_pre units' weights were requested before the op)
-                if (!__all_sync(0xffffffffu, mbar_wait(pp.empty + s, (pp.pphase >> s) & 1u, err))) return false;
-                pp.pphase ^= 1u << s;
-            }
-            if (elect_one()) {
-                if (ut && i < 64) ut[i * 4 + 0] = globaltimer();
-                if (i >= n_pre) tma_weights<R>(a, epi, u_begin + i, st, pp.full + s);
-                tma_inputs<R>(a, u_begin + i, st, pp.full + s);
-            }
-            __syncwarp();
-        }
-        return true;
-    }
-
-    if (threadIdx.x >= kConsumers + 32) {  // MMA warp: one elected lane issues
-        constexpr uint32_t idesc = umma_idesc(NP);
-        const uint64_t desc0 = umma_desc(smem_u32(smem));  // (descriptors count 16-byte steps)
-        for (int i = 0; i < n_my; ++i) {
-            const int u = u_begin + i;
-            const int chunk = u % a.n_chunks;
-            const bool first = i == 0 || chunk == 0;
-            const bool last = i == n_my - 1 || chunk == a.n_chunks - 1;
-            const int ab = pp.ab;
-            if (first) {  // the consumers have read this accumulator's previous segment
-                if (!__all_sync(0xffffffffu, mbar_wait(pp.acc_empty + ab, (pp.aempty >> ab) & 1u, err))) return false;
-                pp.aempty ^= 1u << ab;
-            }
-            const int s = i % S;
-            if (!__all_sync(0xffffffffu, mbar_wait(pp.full + s, (pp.cphase >> s) & 1u, err))) return false;
-            pp.cphase ^= 1u << s;
-            tc_fence_after();
-            if (elect_one()) {
-                const uint64_t st = desc0 + (uint64_t)((uint32_t)(s * L::STAGE) >> 4);
-                const uint32_t d = pp.tmem + (uint32_t)(ab * (kTmemCols / 2));
-#pragma unroll
-                for (int kb = 0; kb < 2; ++kb)
-#pragma unroll
-                    for (int ks = 0; ks < 4; ++ks)
-                        umma(d, st + (kb * 16384 + ks * 32) / 16, st + (L::WB + kb * L::XKB + ks * 32) / 16, idesc,
-                             (first && kb == 0 && ks == 0) ? 0u : 1u);
-                umma_commit(pp.empty + s);  // the stage is free once these MMAs have read it
-                if (ut && i < 64) ut[i * 4 + 1] = globaltimer();
-                if (last) umma_commit(pp.acc_full + ab);
-            }
-            __syncwarp();
-            if (last) pp.ab ^= 1;
-        }
-        return true;
-    }
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // 1 / rms of each input row from the previous op's per-tile sums of
@@ -565,8 +612,9 @@ __device__ bool gemm_op(const GemmArgs& a, int epi, int M, int pos0, int n_pre, 
         }
         if (lane == 0) r_s[m] = r;
     }
-    // the MMA thread took the full-barrier waits of these ring positions
+    // the MMA warp took the full-barrier waits of these ring positions
     advance_full<S>(pp, n_my);
+    ring_advance<S>(pp, n_my);
 
     for (int i = 0; i < n_my; ++i) {
         const int u = u_begin + i;
@@ -578,110 +626,112 @@ __device__ bool gemm_op(const GemmArgs& a, int epi, int M, int pos0, int n_pre, 
         // accumulator holds W x_hi in columns 0..R-1 and W x_lo in columns
         // R..2R-1.  Split-K: the CTA holding the tile's first chunks (its
         // segment ends last, at the end of that CTA's range) finalises; the
-        // others store their partial and move on.  Each value travels with the
-        // op's tag in one 64-bit word, so the finaliser needs no flag and no
+        // others store their partial and move on.  The sums travel with the
+        // op's tag in 128-bit words, so the finaliser needs no flag and no
         // fence: it reads each word until the tag is this op's.
+        //
+        // Every consumer warp reads its own TMEM rows - warp w holds tile row
+        // rr = 32 (w % 4) + lane for the input rows m = w / 4, w / 4 + 2, ... -
+        // so no CTA barrier precedes the contributors' stores.  A finaliser
+        // first fetches the other segments' partials (and a residual one the
+        // residual rows and the gains) while its own accumulator completes; its
+        // sum is own + (p_1 + p_2 + ...), the partials added in segment order.
         const int ab = pp.ab;
         const long long u_first = (long long)tile * a.n_chunks;
         const int seg0 = unit_owner(u_first, U, G);
         const int nseg = unit_owner(u_first + a.n_chunks - 1, U, G) - seg0 + 1;
-        constexpr size_t kSlot = (size_t)kMaxRows * kFTile;
-        unsigned long long* slots =
-            reinterpret_cast<unsigned long long*>(a.partial) + (size_t)tile * a.n_chunks * kSlot;
         const bool contributor = nseg > 1 && b != seg0;
-
-        if (contributor || epi == EPI_RESID) {
-            // Direct path: every consumer warp reads its own TMEM rows - warp w
-            // holds tile row rr = 32 (w % 4) + lane for the input rows m = w / 4,
-            // w / 4 + 2, ... - so nothing goes through shared memory and no CTA
-            // barrier precedes the stores.  A residual finaliser first fetches
-            // the residual rows, the gains and the other segments' partials
-            // while its own accumulator completes; its sum is own + (p_1 + p_2
-            // + ...), the partials added in segment order.
-            constexpr int HM = (R + 1) / 2;
-            const int q4 = warp & 3, par = warp >> 2, rr = q4 * 32 + lane;
-            const int n = tile * kFTile + rr;
-            float hp[HM], ps[HM];
-            const float gp = (!contributor && n < a.N && a.g_next) ? __bfloat162float(a.g_next[n]) : 0.f;
+        const bool resid = epi == EPI_RESID && !contributor;
+        constexpr int HM = (R + 1) / 2;     // input rows per thread
+        constexpr int NW = (HM + 2) / 3;    // words they take
+        const int q4 = warp & 3, par = warp >> 2, rr = q4 * 32 + lane;
+        const int n = tile * kFTile + rr;
+        // words [tile][segment][par][word][tile row]
+        PartWord* slots = reinterpret_cast<PartWord*>(a.partial) + (size_t)tile * a.n_chunks * kPartWords + par * 3 * kFTile + rr;
+        float hp[HM], ps[HM];
+        const float gp = (resid && n < a.N && a.g_next) ? __bfloat162float(a.g_next[n]) : 0.f;
 #pragma unroll
-            for (int k = 0; k < HM; ++k) {
-                const int m = par + 2 * k;
-                hp[k] = (!contributor && m < M && n < a.N) ? __ldcg(a.out_f32 + (size_t)m * a.ldo + n) : 0.f;
-                ps[k] = 0.f;
-            }
-            if (!contributor && nseg > 1) {
-                constexpr int QB = R <= 8 ? 4 : R <= 12 ? 2 : 1;  // segments per batch (registers: QB * HM words)
-                for (int sg0 = 1; sg0 < nseg; sg0 += QB) {
-                    unsigned long long w[QB][HM];
+        for (int k = 0; k < HM; ++k) {
+            const int m = par + 2 * k;
+            hp[k] = (resid && m < M && n < a.N) ? __ldcg(a.out_f32 + (size_t)m * a.ldo + n) : 0.f;
+            ps[k] = 0.f;
+        }
+        if (!contributor && nseg > 1 && par < M) {
+            constexpr int QB = R <= 4 ? 5 : R <= 12 ? 3 : 2;  // segments per batch (registers: 4 QB NW)
+            for (int sg0 = 1; sg0 < nseg; sg0 += QB) {
+                PartWord w[QB][NW];
+#pragma unroll
+                for (int q = 0; q < QB; ++q)
+#pragma unroll
+                    for (int k = 0; k < NW; ++k)
+                        if (sg0 + q < nseg && par + 6 * k < M)
+                            w[q][k] = ld_relaxed(slots + (size_t)(sg0 + q) * kPartWords + k * kFTile);
+                // words that do not carry this op's tag yet (their CTA has
+                // not published) are re-read together, not one at a time
+                unsigned long long t_wait = 0;
+                for (;;) {
+                    bool ready = true;
 #pragma unroll
                     for (int q = 0; q < QB; ++q)
 #pragma unroll
-                        for (int k = 0; k < HM; ++k)
-                            if (sg0 + q < nseg && par + 2 * k < M)
-                                w[q][k] = ld_relaxed_u64(slots + (size_t)(sg0 + q) * kSlot + (par + 2 * k) * kFTile + rr);
-                    // words that do not carry this op's tag yet (their CTA has
-                    // not published) are re-read together, not one at a time
-                    unsigned long long t_wait = 0;
-                    for (;;) {
-                        bool ready = true;
-#pragma unroll
-                        for (int q = 0; q < QB; ++q)
-#pragma unroll
-                            for (int k = 0; k < HM; ++k)
-                                if (sg0 + q < nseg && par + 2 * k < M && tag_of(w[q][k]) != tag) ready = false;
-                        if (ready) break;
-                        const unsigned long long now = globaltimer();
-                        if (t_wait == 0) t_wait = now;
-                        if (now - t_wait > kErrPollAfterNs) {
-                            if (*(volatile int*)err) { ok = false; break; }
-                            if (now - t_wait > kBarrierTimeoutNs) {
-                                atomicCAS(err, 0, kDevErrTimeout);
-                                ok = false;
-                                break;
-                            }
+                        for (int k = 0; k < NW; ++k)
+                            if (sg0 + q < nseg && par + 6 * k < M && tag_of(w[q][k]) != tag) ready = false;
+                    if (ready) break;
+                    const unsigned long long now = globaltimer();
+                    if (t_wait == 0) t_wait = now;
+                    if (now - t_wait > kErrPollAfterNs) {
+                        if (*(volatile int*)err) { ok = false; break; }
+                        if (now - t_wait > kBarrierTimeoutNs) {
+                            atomicCAS(err, 0, kDevErrTimeout);
+                            ok = false;
+                            break;
                         }
-#pragma unroll
-                        for (int q = 0; q < QB; ++q)
-#pragma unroll
-                            for (int k = 0; k < HM; ++k)
-                                if (sg0 + q < nseg && par + 2 * k < M && tag_of(w[q][k]) != tag)
-                                    w[q][k] = ld_relaxed_u64(slots + (size_t)(sg0 + q) * kSlot + (par + 2 * k) * kFTile + rr);
                     }
 #pragma unroll
                     for (int q = 0; q < QB; ++q)
 #pragma unroll
-                        for (int k = 0; k < HM; ++k)
-                            if (sg0 + q < nseg && par + 2 * k < M) ps[k] += value_of(w[q][k]);
+                        for (int k = 0; k < NW; ++k)
+                            if (sg0 + q < nseg && par + 6 * k < M && tag_of(w[q][k]) != tag)
+                                w[q][k] = ld_relaxed(slots + (size_t)(sg0 + q) * kPartWords + k * kFTile);
                 }
-            }
-            ok = mbar_wait(pp.acc_full + ab, (pp.afull >> ab) & 1u, err) && ok;
-            pp.afull ^= 1u << ab;
-            pp.ab ^= 1;
-            tc_fence_after();
-            if (threadIdx.x == 0 && ct) ct[2] = globaltimer();
-            constexpr int NC = R == 12 ? 24 : NP;  // the 2R accumulator columns, rounded up
-            float v[NC];
-            tmem_ld<NC>(pp.tmem + (uint32_t)(ab * (kTmemCols / 2)) + ((uint32_t)(q4 * 32) << 16), v);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(pp.acc_empty + ab);  // this warp is done with the accumulator
-            float own[HM];
 #pragma unroll
-            for (int k = 0; k < HM; ++k) {  // input row m = par + 2k: columns m (hi) and R + m (lo)
-                const float hi = par ? v[(2 * k + 1) < NC ? 2 * k + 1 : 0] : v[2 * k];
-                const float lo = par ? v[(R + 2 * k + 1) < NC ? R + 2 * k + 1 : 0] : v[(R + 2 * k) < NC ? R + 2 * k : 0];
-                own[k] = hi + lo;
-            }
-            if (contributor) {
-                unsigned long long* mine = slots + (size_t)(b - seg0) * kSlot;
+                for (int q = 0; q < QB; ++q)
 #pragma unroll
-                for (int k = 0; k < HM; ++k)
-                    if (par + 2 * k < M) st_relaxed_u64(mine + (par + 2 * k) * kFTile + rr, tagged(tag, own[k]));
-                continue;
+                    for (int k = 0; k < HM; ++k)
+                        if (sg0 + q < nseg && par + 2 * k < M) ps[k] += value_of(w[q][k / 3], k % 3);
             }
-            // residual finaliser: h += sum, the next norm's input planes of
-            // h * g_next and the per-tile sums of h^2 (per quadrant of 32 rows,
-            // then the 4 quadrants in order)
+        }
+        ok = mbar_wait(pp.acc_full + ab, (pp.afull >> ab) & 1u, err) && ok;
+        pp.afull ^= 1u << ab;
+        pp.ab ^= 1;
+        tc_fence_after();
+        if (threadIdx.x == 0 && ct) ct[2] = globaltimer();
+        constexpr int NC = R == 12 ? 24 : NP;  // the 2R accumulator columns, rounded up
+        float v[NC];
+        tmem_ld<NC>(pp.tmem + (uint32_t)(ab * (kTmemCols / 2)) + ((uint32_t)(q4 * 32) << 16), v);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(pp.acc_empty + ab);  // this warp is done with the accumulator
+        float own[HM];
+#pragma unroll
+        for (int k = 0; k < HM; ++k) {  // input row m = par + 2k: columns m (hi) and R + m (lo)
+            const float hi = par ? v[(2 * k + 1) < NC ? 2 * k + 1 : 0] : v[2 * k];
+            const float lo = par ? v[(R + 2 * k + 1) < NC ? R + 2 * k + 1 : 0] : v[(R + 2 * k) < NC ? R + 2 * k : 0];
+            own[k] = hi + lo;
+        }
+        if (contributor) {
+#pragma unroll
+            for (int k = 0; k < NW; ++k)
+                if (par + 6 * k < M)
+                    st_relaxed(slots + (size_t)(b - seg0) * kPartWords + k * kFTile, tag, own[3 * k],
+                               3 * k + 1 < HM ? own[3 * k + 1 < HM ? 3 * k + 1 : 0] : 0.f,
+                               3 * k + 2 < HM ? own[3 * k + 2 < HM ? 3 * k + 2 : 0] : 0.f);
+            continue;
+        }
+        if (resid) {
+            // h += sum, the next norm's input planes of h * g_next and the
+            // per-tile sums of h^2 (per quadrant of 32 rows, then the 4
+            // quadrants in order)
             float* ssq = ys;  // [16][4]
 #pragma unroll
             for (int k = 0; k < HM; ++k) {
@@ -713,91 +763,11 @@ __device__ bool gemm_op(const GemmArgs& a, int epi, int M, int pos0, int n_pre, 
             if (ut && i < 64 && threadIdx.x == 0) ut[i * 4 + 3] = globaltimer();
             continue;
         }
-
-        // finalisers of the other epilogues: TMEM -> ys (warps 0-3), then the
-        // other segments' partials and the epilogue over ys
-        ok = mbar_wait(pp.acc_full + ab, (pp.afull >> ab) & 1u, err) && ok;
-        pp.afull ^= 1u << ab;
-        pp.ab ^= 1;
-        tc_fence_after();
-        if (threadIdx.x == 0 && ct) ct[2] = globaltimer();
-        if (warp < 4) {  // warp w reads TMEM lanes (tile rows) 32w .. 32w + 31
-            float v[NP];
-            tmem_ld<NP>(pp.tmem + (uint32_t)(ab * (kTmemCols / 2)) + ((uint32_t)(warp * 32) << 16), v);
-            const int r = warp * 32 + lane;
+        // the other epilogues combine rows of the tile: through ys
 #pragma unroll
-            for (int m = 0; m < R; ++m) ys[r * 16 + m] = v[m] + v[R + m];
-        }
-        tc_fence_before();
+        for (int k = 0; k < HM; ++k)
+            if (par + 2 * k < M) ys[rr * 16 + par + 2 * k] = own[k] + ps[k];
         consumer_sync();
-        if (lane == 0) mbar_arrive(pp.acc_empty + ab);  // the accumulator may be refilled
-
-        constexpr int HJ = (R * kFTile + kGemmThreads - 1) / kGemmThreads;  // elements per thread (M <= R)
-
-        if (nseg > 1) {
-            // the other segments come from later CTAs, which never wait on this
-            // one.  Each thread issues the words of all its elements for a batch
-            // of segments before using any (one L2 round trip per batch), then
-            // adds them in segment order.
-            float acc[HJ];
-            int at[HJ];
-#pragma unroll
-            for (int j = 0; j < HJ; ++j) {
-                const int idx = threadIdx.x + j * kGemmThreads;
-                const int m = idx / kFTile, r = idx - m * kFTile;
-                at[j] = idx < M * kFTile ? m * kFTile + r : -1;
-                acc[j] = at[j] >= 0 ? ys[r * 16 + m] : 0.f;
-            }
-            constexpr int QB = R <= 8 ? 4 : 2;  // segments per batch (registers: QB * HJ words)
-            for (int sg0 = 1; sg0 < nseg; sg0 += QB) {
-                unsigned long long w[QB][HJ];
-#pragma unroll
-                for (int q = 0; q < QB; ++q)
-#pragma unroll
-                    for (int j = 0; j < HJ; ++j)
-                        if (sg0 + q < nseg && at[j] >= 0) w[q][j] = ld_relaxed_u64(slots + (size_t)(sg0 + q) * kSlot + at[j]);
-                // words that do not carry this op's tag yet (their segment's CTA
-                // has not published) are re-read together, not one at a time
-                unsigned long long t_wait = 0;
-                for (;;) {
-                    bool ready = true;
-#pragma unroll
-                    for (int q = 0; q < QB; ++q)
-#pragma unroll
-                        for (int j = 0; j < HJ; ++j)
-                            if (sg0 + q < nseg && at[j] >= 0 && tag_of(w[q][j]) != tag) ready = false;
-                    if (ready) break;
-                    const unsigned long long now = globaltimer();
-                    if (t_wait == 0) t_wait = now;
-                    if (now - t_wait > kErrPollAfterNs) {
-                        if (*(volatile int*)err) { ok = false; break; }
-                        if (now - t_wait > kBarrierTimeoutNs) {
-                            atomicCAS(err, 0, kDevErrTimeout);
-                            ok = false;
-                            break;
-                        }
-                    }
-#pragma unroll
-                    for (int q = 0; q < QB; ++q)
-#pragma unroll
-                        for (int j = 0; j < HJ; ++j)
-                            if (sg0 + q < nseg && at[j] >= 0 && tag_of(w[q][j]) != tag)
-                                w[q][j] = ld_relaxed_u64(slots + (size_t)(sg0 + q) * kSlot + at[j]);
-                }
-#pragma unroll
-                for (int q = 0; q < QB; ++q)
-#pragma unroll
-                    for (int j = 0; j < HJ; ++j)
-                        if (sg0 + q < nseg && at[j] >= 0) acc[j] += value_of(w[q][j]);
-            }
-#pragma unroll
-            for (int j = 0; j < HJ; ++j)
-                if (at[j] >= 0) {
-                    const int m = at[j] / kFTile, r = at[j] - m * kFTile;
-                    ys[r * 16 + m] = acc[j];
-                }
-            consumer_sync();
-        }
 
         // epilogue of the finished tile (row m scaled by its RMSNorm factor)
         if (epi == EPI_LOGITS) {
@@ -896,7 +866,7 @@ __device__ __forceinline__ AttnRange attn_range(const AttnArgs& a, int M, int po
 // holding rows this forward writes (those need the q/k/v op to be finished).
 // Returns the ring position reached, or -1 if a wait timed out.
 template <int R, int HD>
-__device__ int attn_produce(const AttnArgs& a, const AttnRange& ar, int pos0, unsigned char* smem, Pipe& pp,
+__device__ int attn_request(const AttnArgs& a, const AttnRange& ar, int pos0, unsigned char* smem, Pipe& pp,
                             int* err, int i_from, int i_limit, bool old_only) {
     using L = GemmSmem<R>;
     constexpr int S = L::S, SC = kAttnSegChunks;
@@ -906,7 +876,7 @@ __device__ int attn_produce(const AttnArgs& a, const AttnRange& ar, int pos0, un
         for (int c = c0; c < min(c0 + SC, ar.n_ch); ++c, ++i) {
             if (i < i_from) continue;
             if (i >= i_limit || (old_only && (c + 1) * kAttnChunk > pos0)) return i;
-            const int s = i % S;
+            const int s = ring_stage<S>(pp, i);
             unsigned char* st = smem + s * L::STAGE;
             if (!__all_sync(0xffffffffu, mbar_wait(pp.empty + s, (pp.pphase >> s) & 1u, err))) return -1;
             pp.pphase ^= 1u << s;
@@ -924,45 +894,47 @@ __device__ int attn_produce(const AttnArgs& a, const AttnRange& ar, int pos0, un
     return i;
 }
 
-// Before the grid barrier ahead of an attention op: the producer requests the
-// K / V chunks of its first ring stages that hold only rows of earlier
-// forwards.  Returns how many (-1 on a timeout).
+// Producer warp of an attention op: the chunks that hold only rows of earlier
+// forwards as soon as stages are free, the others once `go` says that the
+// q/k/v op has finished everywhere.
 template <int R, int HD>
-__device__ int attn_prefetch(const AttnArgs& a, int M, int pos0, unsigned char* smem, Pipe& pp, int* err) {
+__device__ bool attn_produce(const AttnArgs& a, int M, int pos0, unsigned char* smem, Pipe& pp, uint64_t* go,
+                             unsigned go_parity, int* err) {
+    constexpr int S = GemmSmem<R>::S;
     const AttnRange ar = attn_range(a, M, pos0);
     if (ar.i_begin < ar.i_end && elect_one()) {
         prefetch_tmap(a.tm_k);
         prefetch_tmap(a.tm_v);
     }
     __syncwarp();
-    return attn_produce<R, HD>(a, ar, pos0, smem, pp, err, 0, GemmSmem<R>::S, true);
+    int n = attn_request<R, HD>(a, ar, pos0, smem, pp, err, 0, S, true);
+    if (n < 0 || !__all_sync(0xffffffffu, mbar_wait(go, go_parity, err))) return false;
+    // K / V rows of this forward were stored by other CTAs (generic proxy)
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    n = attn_request<R, HD>(a, ar, pos0, smem, pp, err, n, 1 << 30, false);
+    if (n < 0) return false;
+    ring_advance<S>(pp, n);
+    return true;
 }
 
-// Returns false if a wait timed out (error recorded).  pre: ring positions the
-// producer already filled before the grid barrier (attn_prefetch).
+// ring positions (K / V chunks) this CTA's items take
+__device__ __forceinline__ int attn_positions(const AttnRange& ar) {
+    constexpr int SC = kAttnSegChunks;
+    int n = 0;
+    for (int it = ar.i_begin; it < ar.i_end; ++it) n += min(SC, ar.n_ch - (it % ar.n_seg) * SC);
+    return n;
+}
+
+// Consumer warps: the items' segment partials.  Returns false if a wait timed
+// out (error recorded).
 template <int R, int HD>
-__device__ bool attn_op(const AttnArgs& a, int M, int pos0, unsigned char* smem, Pipe& pp, int* err,
-                        unsigned long long* ct, int pre, unsigned long long* ut) {
+__device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* smem, Pipe& pp, int* err,
+                             unsigned long long* ct, unsigned long long* ut) {
     using L = GemmSmem<R>;
     constexpr int S = L::S, VG = L::VG, SC = kAttnSegChunks, SP = SC * kAttnChunk;  // positions per segment
     static_assert(SC <= S, "a segment's chunks are held in the ring at once");
     const int G = a.n_heads / a.n_kv_heads, NV = G * M;
     const AttnRange ar = attn_range(a, M, pos0);
-
-    if (threadIdx.x >= kConsumers + 32) {  // MMA warp: only keeps its copy of the ring parities
-        int n = 0;
-        for (int it = ar.i_begin; it < ar.i_end; ++it) {
-            const int sg = it % ar.n_seg;
-            n += min(SC, ar.n_ch - sg * SC);
-        }
-        advance_full<S>(pp, n);
-        return true;
-    }
-    if (threadIdx.x >= kConsumers) {  // producer warp: one elected lane requests K / V
-        // K / V rows of this forward were stored by other CTAs (generic proxy)
-        if (ar.i_begin < ar.i_end) asm volatile("fence.proxy.async.global;" ::: "memory");
-        return attn_produce<R, HD>(a, ar, pos0, smem, pp, err, pre, 1 << 30, false) >= 0;
-    }
 
     constexpr int QST = L::QST, PST = L::PST;
     __half* qh = reinterpret_cast<__half*>(smem + L::ATT);  // [VG][QST] q hi, then lo
@@ -1023,7 +995,7 @@ __device__ bool attn_op(const AttnArgs& a, int M, int pos0, unsigned char* smem,
         q_key = key;
         stamp(it, 1);
         for (int j = 0; j < n_u; ++j) {
-            const int s = (i + j) % S;
+            const int s = ring_stage<S>(pp, i + j);
             ok = mbar_wait(pp.full + s, (pp.cphase >> s) & 1u, err) && ok;
             pp.cphase ^= 1u << s;
         }
@@ -1047,7 +1019,7 @@ __device__ bool attn_op(const AttnArgs& a, int M, int pos0, unsigned char* smem,
                 // K q_hi and K q_lo in separate accumulators (two short
                 // dependency chains instead of one long one), added at the end
                 float cl[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-                const unsigned char* kst = smem + ((i + j) % S) * L::STAGE;
+                const unsigned char* kst = smem + ring_stage<S>(pp, i + j) * L::STAGE;
                 const int t = (p0 % kAttnChunk) + (lane & 7) + 8 * ((lane >> 3) & 1);
                 const int qv = (lane & 7) + 8 * (lane >> 4), qk = ((lane >> 3) & 1) * 8;
 #pragma unroll
@@ -1146,7 +1118,7 @@ __device__ bool attn_op(const AttnArgs& a, int M, int pos0, unsigned char* smem,
                 const int p = ks * 16 + (lane & 7) + 8 * ((lane >> 3) & 1), j = p / kAttnChunk, tt = p % kAttnChunk;
                 ldsm_x4(ah, ph + pv * PST + ks * 16 + pk);
                 ldsm_x4(al, pl + pv * PST + ks * 16 + pk);
-                ldsm_x4_t(bv, smem + ((i + j) % S) * L::STAGE + 16384 + bx * 8192 + tt * 128 + ((cc ^ (tt & 7)) << 4));
+                ldsm_x4_t(bv, smem + ring_stage<S>(pp, i + j) * L::STAGE + 16384 + bx * 8192 + tt * 128 + ((cc ^ (tt & 7)) << 4));
                 mma_f16_16816(c[0], ah[0], ah[1], ah[2], ah[3], bv[0], bv[1]);
                 mma_f16_16816(c[1], ah[0], ah[1], ah[2], ah[3], bv[2], bv[3]);
                 mma_f16_16816(cl[0], al[0], al[1], al[2], al[3], bv[0], bv[1]);
@@ -1170,10 +1142,11 @@ __device__ bool attn_op(const AttnArgs& a, int M, int pos0, unsigned char* smem,
         consumer_sync();  // q / scores / weights are free for the next item
         stamp(it, 6);
         if (tid == 0)
-            for (int j = 0; j < n_u; ++j) mbar_arrive(pp.empty + (i + j) % S);  // the stages are free
+            for (int j = 0; j < n_u; ++j) mbar_arrive(pp.empty + ring_stage<S>(pp, i + j));  // the stages are free
         i += n_u;
     }
     if (ct && tid == 0) ct[6] = (unsigned long long)(ar.i_end - ar.i_begin);
+    ring_advance<S>(pp, i);
     return ok;
 }
 
@@ -1191,7 +1164,6 @@ __device__ bool attn_op(const AttnArgs& a, int M, int pos0, unsigned char* smem,
 constexpr int kCombineBatch = 16;
 template <int HD>
 __device__ void attn_combine(const AttnArgs& a, int M, int pos0) {
-    if (threadIdx.x >= kConsumers) return;
     constexpr int SP = kAttnSegChunks * kAttnChunk, HALVES = HD / 64, B = kCombineBatch;
     static_assert(B <= 32, "one lane per segment of a batch");
     const int G = a.n_heads / a.n_kv_heads, NV = G * M;
@@ -1258,7 +1230,6 @@ __device__ void attn_combine(const AttnArgs& a, int M, int pos0) {
 // embedding op: h = E[token], planes of h * g (first RMSNorm), sums of h^2
 // ---------------------------------------------------------------------------
 __device__ void embed_op(const FwdParams& p, int pos0) {
-    if (threadIdx.x >= kConsumers) return;
     const int d = p.d, n_tiles = d / kFTile;  // sums of squares per 128 columns
     const int lane = threadIdx.x & 31;
     const int gw = blockIdx.x * (kGemmThreads / 32) + (threadIdx.x >> 5);
@@ -1288,15 +1259,6 @@ __device__ void embed_op(const FwdParams& p, int pos0) {
     }
 }
 
-// Block-cooperative copy of an op descriptor into shared memory.
-__device__ __forceinline__ void copy_op(const FwdOp* src, FwdOp* dst) {
-    static_assert(sizeof(FwdOp) % 4 == 0, "FwdOp is copied in 4-byte words");
-    const unsigned* s = reinterpret_cast<const unsigned*>(src);
-    unsigned* d = reinterpret_cast<unsigned*>(dst);
-    for (int i = threadIdx.x; i < (int)(sizeof(FwdOp) / 4); i += blockDim.x) d[i] = s[i];
-    __syncthreads();
-}
-
 // After a timed-out wait: give copies still in flight a bounded time to land
 // before the CTA exits (the error is already recorded).
 __device__ void drain_before_exit() {
@@ -1307,9 +1269,9 @@ __device__ void drain_before_exit() {
     __syncthreads();
 }
 
-// Units of the next projection whose weights the producer requests between
-// its CTA's arrival at an op boundary's grid barrier and the barrier's end.
-constexpr int kBoundaryPrefetch = 5;
+// The producer reads op o + 1's arguments while the consumers may still be in
+// op o, and fetches those of op o + 2: three slots.
+constexpr int kOpSlots = 3;
 
 template <int R, int HD>
 __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams p) {
@@ -1323,7 +1285,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams
     __shared__ __align__(8) uint64_t empty[S];      // stage released (tcgen05.commit, or one consumer thread)
     __shared__ __align__(8) uint64_t acc_full[2];   // TMEM accumulator complete (tcgen05.commit)
     __shared__ __align__(8) uint64_t acc_empty[2];  // TMEM accumulator read by the consumers
-    __shared__ FwdOp s_op[2];                       // current and next op's arguments
+    __shared__ __align__(8) uint64_t desc[kOpSlots];  // producer and MMA warp are at op o; its arguments are in shared memory
+    __shared__ __align__(8) uint64_t left;            // this CTA's work of an op is done (consumer thread 0)
+    __shared__ __align__(8) uint64_t go;              // the grid barrier before an op has passed (consumer thread 0)
+    __shared__ FwdOp s_op[kOpSlots];                // arguments of op o at o % kOpSlots
     // 128-byte TMA swizzle needs 1 KB aligned boxes
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const bool mma_warp = threadIdx.x >= kConsumers + 32;
@@ -1344,6 +1309,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams
             mbar_init(acc_full + b, 1);
             mbar_init(acc_empty + b, kConsumers / 32);  // one arrival per consumer warp
         }
+        for (int o = 0; o < kOpSlots; ++o) mbar_init(desc + o, 2);
+        mbar_init(&left, 1);
+        mbar_init(&go, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         if (p.trace && blockIdx.x == 0) p.trace[0] = globaltimer();
@@ -1367,127 +1335,159 @@ __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams
     __syncthreads();
     tc_fence_after();
     const int pos0 = s_pos0;
-    unsigned target = 0;
-    int n_barrier = 0;
-    // Grid barriers of this launch, each split in two: thread 0 arrives right
-    // after a CTA barrier that ends the work before it, and waits for the
-    // others later, so the producer's requests for the next op (the issue of
-    // which can take microseconds while HBM is busy) overlap the wait instead
-    // of delaying the arrival.  The profiling hook p.stall_barrier (0: none)
-    // makes barrier number n unreachable, so that its bounded wait runs out
-    // and the launch ends with the timeout recorded.
-    __shared__ int s_ok;
-    auto barrier_arrive = [&]() {
-        target += gridDim.x;
-        ++n_barrier;
-        if (threadIdx.x == 0) grid_arrive(p.bar);
-    };
-    auto barrier_wait = [&]() {  // thread 0: result in s_ok
-        const unsigned extra = n_barrier == p.stall_barrier ? 1u : 0u;
-        s_ok = grid_wait(p.bar, target + extra, p.err, p.wait_ns) ? 1 : 0;
-        // every CTA has read the sequence number before the first barrier
-        if (s_ok && n_barrier == 1 && blockIdx.x == 0) *p.seq = s_seq + 1u;
-    };
-    Pipe pp{full, empty, acc_full, acc_empty, s_tmem, 0u, 0u, 0u, 0u, 0};
-    int n_pre = 0;  // producer: units of the op whose weights were requested before it
+    Pipe pp{full, empty, acc_full, acc_empty, s_tmem, 0u, 0u, 0u, 0u, 0, 0};
     bool failed = false;
-    int attn_pre = 0;  // producer: K / V chunks of the next attention op requested early
-    copy_op(p.ops, s_op);
-    for (int o = 0; o < p.n_ops; ++o) {
-        const FwdOp& op = s_op[o & 1];
-        const int type = op.type;
-        bool ok = true;
-        unsigned long long* ct = (p.trace && o == (p.trace_op & 0xffff)) ? p.trace + kTraceCtas + blockIdx.x * 8 : nullptr;
-        const bool ut_cta = ct && (int)blockIdx.x == (p.trace_op >> 16);  // the CTA whose units are stamped
-        if (ct && threadIdx.x == 0) ct[0] = globaltimer();
-        // the next op's arguments: the producer warp copies them (16 bytes a
-        // lane, asynchronously) into their slot, which held op o-1, while op
-        // o runs; the producer uses them as soon as it has issued op o
-        constexpr int kOpChunks = (int)(sizeof(FwdOp) / 16);
-        static_assert(sizeof(FwdOp) % 16 == 0 && kOpChunks <= 32, "an op is copied in 16-byte pieces by one warp");
-        const bool has_nx = o + 1 < p.n_ops;
-        const int plane = mma_warp ? -1 : (int)threadIdx.x - kConsumers;  // lane in the producer warp
-        if (has_nx && plane >= 0 && plane < kOpChunks)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                             smem_u32(reinterpret_cast<unsigned char*>(s_op + ((o + 1) & 1)) + 16 * plane)),
-                         "l"(reinterpret_cast<const unsigned char*>(p.ops + o + 1) + 16 * plane)
-                         : "memory");
-        const FwdOp* nx = has_nx ? s_op + ((o + 1) & 1) : nullptr;
-        bool early = false;  // producer: the next projection's weights already requested
-        if (is_gemm(type)) {
-            ok = gemm_op<R>(op.g, epi_of(type), p.M, pos0, n_pre, smem, r_s, pp, (s_seq << 10) | (unsigned)o, p.err,
-                            ut_cta ? p.trace + kTraceUnits : nullptr, ct);
-        } else if (type == OP_EMBED) {
-            embed_op(p, pos0);
-        } else {
-            // attention: segment partials; a grid barrier; then every CTA
-            // combines a share of the partials.  Between arriving and passing,
-            // the producer requests the next projection's first weights (the
-            // ring is free again); the consumers do not wait for that.
-            ok = attn_op<R, HD>(op.at, p.M, pos0, smem, pp, p.err, ct, attn_pre,
-                                ut_cta ? p.trace + kTraceUnits : nullptr);
-            if (__syncthreads_or(!ok)) {  // (uniform)
+    // The roles walk the op list on their own.  The consumers run op o, arrive at
+    // the grid barrier and wait for it; the producer requests what depends on no op
+    // (weights, old K / V rows) as soon as they have left the previous op, and waits
+    // for `go` before it requests anything an op of this forward has written, as does
+    // the MMA warp before each op.
+    auto stamps = [&](int o) -> unsigned long long* {  // op stamps of this CTA if op o is traced
+        return (p.trace && o == (p.trace_op & 0xffff)) ? p.trace + kTraceCtas + blockIdx.x * 8 : nullptr;
+    };
+    auto unit_stamps = [&](int o) -> unsigned long long* {  // the CTA whose units are stamped
+        return (stamps(o) && (int)blockIdx.x == (p.trace_op >> 16)) ? p.trace + kTraceUnits : nullptr;
+    };
+    if (threadIdx.x >= kConsumers + 32) {  // MMA warp
+        const bool lane0 = threadIdx.x == kConsumers + 32;
+        if (lane0) mbar_arrive(desc);  // op 0: the embedding
+        for (int o = 1; o < p.n_ops && !failed; ++o) {
+            // It waits for `go` like the producer: attention's chunks complete ring
+            // stages that it does not wait for, so it must not reach the next
+            // projection while any of them is still to come.
+            if (lane0) mbar_arrive(desc + o % kOpSlots);
+            if (!__all_sync(0xffffffffu, mbar_wait(&go, (unsigned)(o - 1) & 1u, p.err))) {
                 failed = true;
                 break;
             }
-            if (ct && threadIdx.x == 0) ct[2] = globaltimer();
-            barrier_arrive();
-            if (plane >= 0) {
-                asm volatile("cp.async.wait_all;" ::: "memory");
-                __syncwarp();
-            }
-            if (plane >= 0 && nx && is_gemm(nx->type)) {
-                ok = gemm_prefetch<R>(nx->g, epi_of(nx->type), smem, pp, p.err, GemmSmem<R>::S);
-                early = true;
-            }
-            if (threadIdx.x < kConsumers) {  // (the producer and MMA warps go on to the op's end)
-                if (threadIdx.x == 0) {
-                    barrier_wait();
-                    if (ct) ct[7] = globaltimer();
-                }
-                consumer_sync();
-                if (s_ok) attn_combine<HD>(op.at, p.M, pos0);
-                else ok = false;
+            const FwdOp& op = s_op[o % kOpSlots];
+            if (is_gemm(op.type)) {
+                failed = !gemm_mma<R>(op.g.n_units, op.g.n_chunks, smem, pp, p.err, unit_stamps(o));
+            } else if (op.type == OP_ATTN) {  // the consumers wait for these ring positions
+                const int n = attn_positions(attn_range(op.at, p.M, pos0));
+                advance_full<S>(pp, n);
+                ring_advance<S>(pp, n);
             }
         }
-        if (ct && threadIdx.x == 0) ct[3] = globaltimer();
-        // the end of op o in this CTA (its stores ordered before thread 0's
-        // arrival); the last op needs no grid barrier
-        if (__syncthreads_or(!ok)) {
-            failed = true;
-            break;
-        }
-        if (ct && threadIdx.x == 0) ct[4] = globaltimer();
-        if (has_nx) barrier_arrive();
-        // next op: visible to the producer warp now, to every thread after
-        // the CTA barrier below; the producer requests its first inputs that
-        // do not depend on op o while the grid gathers
-        if (plane >= 0) {
+    } else if (threadIdx.x >= kConsumers) {  // producer warp
+        const int lane = threadIdx.x & 31;
+        constexpr int kOpChunks = (int)(sizeof(FwdOp) / 16);
+        static_assert(sizeof(FwdOp) % 16 == 0 && kOpChunks <= 32, "an op is copied in 16-byte pieces by one warp");
+        auto fetch = [&](int o) {  // arguments of op o, 16 bytes a lane, asynchronously
+            if (lane < kOpChunks)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                 smem_u32(reinterpret_cast<unsigned char*>(s_op + o % kOpSlots) + 16 * lane)),
+                             "l"(reinterpret_cast<const unsigned char*>(p.ops + o) + 16 * lane)
+                             : "memory");
+        };
+        fetch(0);
+        for (int o = 0; o < p.n_ops && !failed; ++o) {
+            // Nothing is requested before this CTA's consumers are done with the
+            // previous op (with attention's items): their partial sums and
+            // arrivals would queue in L2 behind 25 MB of weights (7B widths, a
+            // decode step of 4 layers: 384 us; requested as stages fall free: 397).
+            if (o > 0 && !__all_sync(0xffffffffu, mbar_wait(&left, (unsigned)(o - 1) & 1u, p.err))) {
+                failed = true;
+                break;
+            }
             asm volatile("cp.async.wait_all;" ::: "memory");
             __syncwarp();
+            if (lane == 0) mbar_arrive(desc + o % kOpSlots);
+            // its slot held op o - 2, which the consumers left before `go` for op o - 1
+            if (o + 1 < p.n_ops) fetch(o + 1);
+            const FwdOp& op = s_op[o % kOpSlots];
+            const unsigned go_parity = (unsigned)(o - 1) & 1u;
+            if (is_gemm(op.type))
+                failed = !gemm_produce<R>(op.g, epi_of(op.type), smem, pp, &go, go_parity, p.err, unit_stamps(o));
+            else if (op.type == OP_ATTN)
+                failed = !attn_produce<R, HD>(op.at, p.M, pos0, smem, pp, &go, go_parity, p.err);
         }
-        n_pre = 0;
-        attn_pre = 0;
-        if (plane >= 0 && nx) {
-            if (is_gemm(nx->type)) {
-                n_pre = (early || kBoundaryPrefetch > GemmSmem<R>::S) ? GemmSmem<R>::S : kBoundaryPrefetch;
-                if (!early) ok = gemm_prefetch<R>(nx->g, epi_of(nx->type), smem, pp, p.err, n_pre);
-            } else if (nx->type == OP_ATTN) {
-                attn_pre = attn_prefetch<R, HD>(nx->at, p.M, pos0, smem, pp, p.err);
-                ok = attn_pre >= 0;
+    } else {  // consumer warps
+        // Grid barriers of this launch: thread 0 arrives after a consumer barrier
+        // that orders the CTA's stores before it, and waits for the others.  The
+        // profiling hook p.stall_barrier (0: none) makes barrier number n
+        // unreachable, so that its bounded wait runs out and the launch ends with
+        // the timeout recorded.
+        unsigned target = 0;
+        int n_barrier = 0;
+        auto barrier_arrive = [&]() {
+            target += gridDim.x;
+            ++n_barrier;
+            if (threadIdx.x == 0) grid_arrive(p.bar);
+        };
+        auto barrier_wait = [&]() {  // thread 0
+            const unsigned extra = n_barrier == p.stall_barrier ? 1u : 0u;
+            const bool passed = grid_wait(p.bar, target + extra, p.err, p.wait_ns);
+            // every CTA has read the sequence number before the first barrier
+            if (passed && n_barrier == 1 && blockIdx.x == 0) *p.seq = s_seq + 1u;
+            return passed;
+        };
+        for (int o = 0; o < p.n_ops; ++o) {
+            unsigned long long* ct = stamps(o);
+            if (ct && threadIdx.x == 0) ct[0] = globaltimer();
+            bool ok = mbar_wait(desc + o % kOpSlots, (unsigned)(o / kOpSlots) & 1u, p.err);
+            if (consumer_or(!ok)) {
+                failed = true;
+                break;
             }
+            const FwdOp& op = s_op[o % kOpSlots];
+            const int type = op.type;
+            if (is_gemm(type)) {
+                ok = gemm_consume<R>(op.g, epi_of(type), p.M, pos0, smem, r_s, pp, (s_seq << 10) | (unsigned)o, p.err,
+                                     unit_stamps(o), ct);
+            } else if (type == OP_EMBED) {
+                embed_op(p, pos0);
+            } else {
+                // attention: segment partials; a grid barrier; then every CTA
+                // combines a share of the partials
+                ok = attn_consume<R, HD>(op.at, p.M, pos0, smem, pp, p.err, ct, unit_stamps(o));
+                if (consumer_or(!ok)) {
+                    failed = true;
+                    break;
+                }
+                if (ct && threadIdx.x == 0) ct[2] = globaltimer();
+                barrier_arrive();
+                if (threadIdx.x == 0) {
+                    mbar_arrive(&left);
+                    ok = barrier_wait();
+                    if (ct) ct[7] = globaltimer();
+                }
+                if (consumer_or(!ok)) {
+                    failed = true;
+                    break;
+                }
+                attn_combine<HD>(op.at, p.M, pos0);
+            }
+            if (ct && threadIdx.x == 0) ct[3] = globaltimer();
+            // the end of op o in this CTA (its stores ordered before thread 0's
+            // arrival); the last op needs no grid barrier
+            if (consumer_or(!ok)) {
+                failed = true;
+                break;
+            }
+            if (ct && threadIdx.x == 0) ct[4] = globaltimer();
+            if (o + 1 < p.n_ops) {
+                barrier_arrive();
+                if (threadIdx.x == 0) {
+                    if (type != OP_ATTN) mbar_arrive(&left);
+                    ok = barrier_wait();
+                    // producer and MMA warp have left op o, i.e. seen `go` for
+                    // it: no completion of `go` is ever two ahead of a waiter
+                    ok = ok && mbar_wait(desc + (o + 1) % kOpSlots, (unsigned)((o + 1) / kOpSlots) & 1u, p.err);
+                    if (ok) mbar_arrive(&go);
+                    if (ct && is_gemm(type)) ct[7] = globaltimer();
+                }
+                if (consumer_or(!ok)) {
+                    failed = true;
+                    break;
+                }
+            }
+            if (ct && threadIdx.x == 0) ct[5] = globaltimer();
+            if (p.trace && blockIdx.x == 0 && threadIdx.x == 0) p.trace[o + 1] = globaltimer();
         }
-        if (has_nx && threadIdx.x == 0) {
-            barrier_wait();
-            if (ct && is_gemm(type)) ct[7] = globaltimer();
-        }
-        if (__syncthreads_or(!ok || (has_nx && threadIdx.x == 0 && !s_ok))) {
-            failed = true;
-            break;
-        }
-        if (ct && threadIdx.x == 0) ct[5] = globaltimer();
-        if (p.trace && blockIdx.x == 0 && threadIdx.x == 0) p.trace[o + 1] = globaltimer();
     }
+    __syncwarp();
+    failed = __syncthreads_or(failed);
     // After a failed wait, copies and MMAs still in flight get a bounded time
     // to land; otherwise every MMA this CTA issued has completed (the
     // consumers waited for each accumulator).  Then TMEM is freed.

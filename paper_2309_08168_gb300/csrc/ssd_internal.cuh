@@ -18,6 +18,7 @@ constexpr int kAttnChunk = 64;    // KV positions per attention CTA (absolute ch
 constexpr int kAttnThreads = 256;
 constexpr int kFTile = 128;       // forward kernel: weight rows per tile (tcgen05 M, TMEM lanes)
 constexpr int kFKC = 128;         // forward kernel: k per work unit (128 rows x 128 k = 32 KB of weights)
+constexpr int kPartWords = 6 * 128;  // 128-bit words of a segment's partial: [2][3][128], three input rows each
 constexpr int kTraceUnits = 1024, kTraceCtas = 1280;  // offsets in FwdParams::trace
 // rows per input plane of a forward of M rows (the plane classes)
 constexpr int fwd_plane_rows(int M) { return M == 1 ? 1 : (M <= 4 ? 4 : (M <= 8 ? 8 : (M <= 12 ? 12 : 16))); }
@@ -60,7 +61,7 @@ struct GemmArgs {
     int N;               // logical output rows
     int K;               // reduction length (row length of every segment)
     int n_tiles;         // row tiles
-    float* partial;      // split-K partials [n_tiles][n_chunks][16][128], tagged 64-bit words
+    void* partial;       // split-K partials [n_tiles][n_chunks][kPartWords], tagged 128-bit words
     // epilogue operands
     float* out_f32;      // EPI_LOGITS: [M][ldo]; EPI_RESID: residual h [M][ldo]
     int ldo;
