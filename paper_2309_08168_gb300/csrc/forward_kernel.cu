@@ -155,10 +155,18 @@ __device__ __forceinline__ int unit_owner(long long u, long long U, long long G)
 // An op's units are split over the first min(U, grid) CTAs, so every CTA that
 // takes part owns at least one unit and the owners of consecutive units are
 // consecutive CTAs (the segment arithmetic of the projection op relies on it).
-__device__ __forceinline__ long long op_ctas(long long U) { return U < gridDim.x ? U : (long long)gridDim.x; }
+// A tile of at most kWholeChunks chunks is one CTA's if there is a CTA for every
+// tile: two or three units one after the other take 0.35 us each, the split-K
+// exchange ~1 us (tiny model, a forward of 5 rows: 100.4 us, split 101.0).
+constexpr int kWholeChunks = 3;
+__device__ __forceinline__ long long op_ctas(long long U, int n_chunks) {
+    const long long G = gridDim.x;
+    if (n_chunks <= kWholeChunks && U <= G * n_chunks) return U / n_chunks;
+    return U < G ? U : G;
+}
 
-__device__ __forceinline__ void my_units(long long U, int* u_begin, int* n_my) {
-    const long long G = op_ctas(U), b = blockIdx.x;
+__device__ __forceinline__ void my_units(long long U, int n_chunks, int* u_begin, int* n_my) {
+    const long long G = op_ctas(U, n_chunks), b = blockIdx.x;
     if (b >= G) { *u_begin = 0; *n_my = 0; return; }
     *u_begin = (int)(b * U / G);
     *n_my = (int)((b + 1) * U / G) - *u_begin;
@@ -509,7 +517,7 @@ __device__ bool gemm_produce(const GemmArgs& a, int epi, unsigned char* smem, Pi
     using L = GemmSmem<R>;
     constexpr int S = L::S;
     int u_begin, n_my;
-    my_units(a.n_units, &u_begin, &n_my);
+    my_units(a.n_units, a.n_chunks, &u_begin, &n_my);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (n_my > 0 && elect_one()) prefetch_tmap(a.tm_x[plane_cls(R)]);
     __syncwarp();
@@ -548,7 +556,7 @@ __device__ bool gemm_mma(int n_units, int n_chunks, unsigned char* smem, Pipe& p
     using L = GemmSmem<R>;
     constexpr int S = L::S, NP = L::NP;
     int u_begin, n_my;
-    my_units(n_units, &u_begin, &n_my);
+    my_units(n_units, n_chunks, &u_begin, &n_my);
     constexpr uint32_t idesc = umma_idesc(NP);
     const uint64_t desc0 = umma_desc(smem_u32(smem));  // (descriptors count 16-byte steps)
     int chunk = u_begin % n_chunks;
@@ -594,10 +602,10 @@ __device__ bool gemm_consume(const GemmArgs& a, int epi, int M, int pos0, unsign
     float* ys = reinterpret_cast<float*>(smem + L::YS);  // [128][16]
     bool ok = true;
 
-    const long long U = a.n_units, G = op_ctas(U);
+    const long long U = a.n_units, G = op_ctas(U, a.n_chunks);
     const int b = blockIdx.x;
     int u_begin, n_my;
-    my_units(U, &u_begin, &n_my);
+    my_units(U, a.n_chunks, &u_begin, &n_my);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // 1 / rms of each input row from the previous op's per-tile sums of
@@ -742,14 +750,14 @@ __device__ bool gemm_consume(const GemmArgs& a, int epi, int M, int pos0, unsign
                     hv = hp[k] + (own[k] + ps[k]);
                     a.out_f32[(size_t)m * a.ldo + n] = hv;
                     if (a.g_next) {
-                        const float z = hv * gp;
+                        const float z = __fmul_rn(hv, gp);
                         const bf16 zh = __float2bfloat16_rn(z);
                         a.xo_hi[(size_t)m * a.N + n] = zh;
                         a.xo_lo[(size_t)m * a.N + n] = __float2bfloat16_rn(z - __bfloat162float(zh));
                     }
                 }
                 if (a.g_next) {
-                    const float sq = warp_sum(hv * hv);
+                    const float sq = warp_sum(__fmul_rn(hv, hv));
                     if (lane == 0) ssq[m * 4 + q4] = sq;
                 }
             }
@@ -800,8 +808,9 @@ __device__ bool gemm_consume(const GemmArgs& a, int epi, int M, int pos0, unsign
                     const int head = tt * (kFTile / hd) + hl, pos = pos0 + m;
                     const float x1 = ys[r1 * 16 + m] * r_s[m], x2 = ys[r2 * 16 + m] * r_s[m];
                     const float2 cs = a.rope[(size_t)pos * half + ii];
-                    const float y1 = x1 * cs.x - x2 * cs.y;
-                    const float y2 = x2 * cs.x + x1 * cs.y;
+                    // (rounded the same in every row class: no contraction of the compiler's choice)
+                    const float y1 = __fmaf_rn(x1, cs.x, -__fmul_rn(x2, cs.y));
+                    const float y2 = __fmaf_rn(x2, cs.x, __fmul_rn(x1, cs.y));
                     if (is_q) {
                         float* q = a.q_out + (size_t)m * a.n_heads * hd + head * hd;
                         q[ii] = y1;
@@ -828,6 +837,18 @@ __device__ bool gemm_consume(const GemmArgs& a, int epi, int M, int pos0, unsign
     }
     consumer_sync();
     return ok;
+}
+
+// two neighbouring values into the hi / lo planes (at: even)
+__device__ __forceinline__ void store_pair(bf16* hi_at, bf16* lo_at, float v0, float v1) {
+    const bf16 h0 = __float2bfloat16_rn(v0), h1 = __float2bfloat16_rn(v1);
+    __nv_bfloat162 hi, lo;
+    hi.x = h0;
+    hi.y = h1;
+    lo.x = __float2bfloat16_rn(v0 - __bfloat162float(h0));
+    lo.y = __float2bfloat16_rn(v1 - __bfloat162float(h1));
+    *reinterpret_cast<__nv_bfloat162*>(hi_at) = hi;
+    *reinterpret_cast<__nv_bfloat162*>(lo_at) = lo;
 }
 
 // ---------------------------------------------------------------------------
@@ -948,6 +969,12 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
     bool ok = true;
     int i = 0;       // ring position within the op
     int q_key = -1;  // (KV head, vector group) whose q is in shared memory
+    int n_held = 0;  // stages of the previous item, not yet released
+    auto release = [&]() {
+        if (tid == 0)
+            for (int j = 1; j <= n_held; ++j) mbar_arrive(pp.empty + ring_stage<S>(pp, i - j));
+        n_held = 0;
+    };
 
     // profiling aid: ut (CTA 0 of a traced forward) gets per-item phase stamps
     auto stamp = [&](int it, int k) {
@@ -994,6 +1021,9 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
         }
         q_key = key;
         stamp(it, 1);
+        const unsigned char* stage[SC];
+#pragma unroll
+        for (int j = 0; j < SC; ++j) stage[j] = smem + ring_stage<S>(pp, i + j) * L::STAGE;
         for (int j = 0; j < n_u; ++j) {
             const int s = ring_stage<S>(pp, i + j);
             ok = mbar_wait(pp.full + s, (pp.cphase >> s) & 1u, err) && ok;
@@ -1003,6 +1033,8 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
         stamp(it, 2);
         consumer_sync();
         stamp(it, 3);
+        // every warp has left the previous item: its stages are free
+        release();
 
         // scores S = K q^T on tensor cores: warp w takes positions 16w..16w+15
         // (A = K rows, 128-byte swizzled), all 16 vectors (B = q hi, then lo);
@@ -1019,7 +1051,7 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
                 // K q_hi and K q_lo in separate accumulators (two short
                 // dependency chains instead of one long one), added at the end
                 float cl[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-                const unsigned char* kst = smem + ring_stage<S>(pp, i + j) * L::STAGE;
+                const unsigned char* kst = j ? stage[1] : stage[0];
                 const int t = (p0 % kAttnChunk) + (lane & 7) + 8 * ((lane >> 3) & 1);
                 const int qv = (lane & 7) + 8 * (lane >> 4), qk = ((lane >> 3) & 1) * 8;
 #pragma unroll
@@ -1091,7 +1123,7 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
         consumer_sync();
         stamp(it, 5);
         // the segment's (max, sum) of each vector; -inf: nothing visible
-        if (tid < nv) {
+        if (tid < nv && ar.n_seg > 1) {
             const int v = v0 + tid, m = v / G;
             float mx = -INFINITY, l = 0.f;
 #pragma unroll
@@ -1113,37 +1145,64 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
             float cl[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
             const int d = warp * 16 + 8 * (lane >> 4), bx = d >> 6, cc = (d & 63) >> 3;
             const int pv = (lane & 7) + 8 * ((lane >> 3) & 1), pk = (lane >> 4) * 8;
-            for (int ks = 0; ks < n_u * (kAttnChunk / 16); ++ks) {
-                uint32_t ah[4], al[4], bv[4];
-                const int p = ks * 16 + (lane & 7) + 8 * ((lane >> 3) & 1), j = p / kAttnChunk, tt = p % kAttnChunk;
-                ldsm_x4(ah, ph + pv * PST + ks * 16 + pk);
-                ldsm_x4(al, pl + pv * PST + ks * 16 + pk);
-                ldsm_x4_t(bv, smem + ring_stage<S>(pp, i + j) * L::STAGE + 16384 + bx * 8192 + tt * 128 + ((cc ^ (tt & 7)) << 4));
-                mma_f16_16816(c[0], ah[0], ah[1], ah[2], ah[3], bv[0], bv[1]);
-                mma_f16_16816(c[1], ah[0], ah[1], ah[2], ah[3], bv[2], bv[3]);
-                mma_f16_16816(cl[0], al[0], al[1], al[2], al[3], bv[0], bv[1]);
-                mma_f16_16816(cl[1], al[0], al[1], al[2], al[3], bv[2], bv[3]);
+#pragma unroll
+            for (int j = 0; j < SC; ++j) {
+                if (j >= n_u) break;
+                const unsigned char* vst = stage[j] + 16384 + bx * 8192;
+#pragma unroll
+                for (int ks = 0; ks < kAttnChunk / 16; ++ks) {
+                    uint32_t ah[4], al[4], bv[4];
+                    const int tt = ks * 16 + (lane & 7) + 8 * ((lane >> 3) & 1), pc = j * kAttnChunk + ks * 16 + pk;
+                    ldsm_x4(ah, ph + pv * PST + pc);
+                    ldsm_x4(al, pl + pv * PST + pc);
+                    ldsm_x4_t(bv, vst + tt * 128 + ((cc ^ (tt & 7)) << 4));
+                    mma_f16_16816(c[0], ah[0], ah[1], ah[2], ah[3], bv[0], bv[1]);
+                    mma_f16_16816(c[1], ah[0], ah[1], ah[2], ah[3], bv[2], bv[3]);
+                    mma_f16_16816(cl[0], al[0], al[1], al[2], al[3], bv[0], bv[1]);
+                    mma_f16_16816(cl[1], al[0], al[1], al[2], al[3], bv[2], bv[3]);
+                }
             }
 #pragma unroll
             for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
                 for (int x = 0; x < 4; ++x) c[nt][x] += cl[nt][x];
             // C: rows = vectors g (+8), columns = dims 16w + 8 nt + 2 tg (+1)
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
+            if (ar.n_seg == 1) {
+                // the only segment: what the combine would make of it (weight
+                // exp(0) = 1), written at once
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int vl = g + 8 * h;
-                    if (vl < nv)
-                        *reinterpret_cast<float2*>(part + (size_t)(v0 + vl) * part_v + warp * 16 + nt * 8 + 2 * tg) =
-                            make_float2(c[nt][2 * h], c[nt][2 * h + 1]);
+                    if (vl >= nv) continue;
+                    float l = 0.f;
+#pragma unroll
+                    for (int w2 = 0; w2 < kConsumers / 32; ++w2) l += wsum[w2 * VG + vl];
+                    const float inv = 1.f / l;
+                    const int v = v0 + vl, m = v / G, gi = v - m * G;
+                    const size_t at = (size_t)m * a.n_heads * HD + (size_t)(kvh * G + gi) * HD + warp * 16 + 2 * tg;
+#pragma unroll
+                    for (int nt = 0; nt < 2; ++nt)
+                        store_pair(a.out_hi + at + nt * 8, a.out_lo + at + nt * 8, c[nt][2 * h] * inv, c[nt][2 * h + 1] * inv);
                 }
+            } else {
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int vl = g + 8 * h;
+                        if (vl < nv)
+                            *reinterpret_cast<float2*>(part + (size_t)(v0 + vl) * part_v + warp * 16 + nt * 8 + 2 * tg) =
+                                make_float2(c[nt][2 * h], c[nt][2 * h + 1]);
+                    }
+            }
         }
-        consumer_sync();  // q / scores / weights are free for the next item
         stamp(it, 6);
-        if (tid == 0)
-            for (int j = 0; j < n_u; ++j) mbar_arrive(pp.empty + ring_stage<S>(pp, i + j));  // the stages are free
         i += n_u;
+        n_held = n_u;  // released once every warp is past this item
+    }
+    if (n_held) {
+        consumer_sync();
+        release();
     }
     if (ct && tid == 0) ct[6] = (unsigned long long)(ar.i_end - ar.i_begin);
     ring_advance<S>(pp, i);
@@ -1214,15 +1273,7 @@ __device__ void attn_combine(const AttnArgs& a, int M, int pos0) {
         }
         const float inv = 1.f / l;
         const size_t at = (size_t)m * a.n_heads * HD + (size_t)(kvh * G + gi) * HD + e;
-        const float v0 = o0 * inv, v1 = o1 * inv;
-        const bf16 h0 = __float2bfloat16_rn(v0), h1 = __float2bfloat16_rn(v1);
-        __nv_bfloat162 hi, lo;
-        hi.x = h0;
-        hi.y = h1;
-        lo.x = __float2bfloat16_rn(v0 - __bfloat162float(h0));
-        lo.y = __float2bfloat16_rn(v1 - __bfloat162float(h1));
-        *reinterpret_cast<__nv_bfloat162*>(a.out_hi + at) = hi;
-        *reinterpret_cast<__nv_bfloat162*>(a.out_lo + at) = lo;
+        store_pair(a.out_hi + at, a.out_lo + at, o0 * inv, o1 * inv);
     }
 }
 
@@ -1241,18 +1292,25 @@ __device__ void embed_op(const FwdParams& p, int pos0) {
         if (p.src == SRC_TOKENS) tok = p.toks[m];
         else if (p.src == SRC_DRAFT) tok = p.st->j == 0 ? p.st->x_last : p.st->drafts[p.st->j - 1];
         else tok = m == 0 ? p.st->x_last : p.st->drafts[m - 1];
-        const bf16* row = p.embed + (size_t)tok * d;
+        // (all loads before the stores: they come from HBM, one round trip)
+        constexpr int J = kFTile / 32;
+        float v[J], g[J];
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const int i = t * kFTile + j * 32 + lane;
+            v[j] = __bfloat162float(p.embed[(size_t)tok * d + i]);
+            g[j] = __bfloat162float(p.g0[i]);
+        }
         float sq = 0.f;
 #pragma unroll
-        for (int j = 0; j < kFTile / 32; ++j) {
+        for (int j = 0; j < J; ++j) {
             const int i = t * kFTile + j * 32 + lane;
-            const float v = __bfloat162float(row[i]);
-            p.h[(size_t)m * d + i] = v;
-            const float z = v * __bfloat162float(p.g0[i]);
+            p.h[(size_t)m * d + i] = v[j];
+            const float z = v[j] * g[j];
             const bf16 zh = __float2bfloat16_rn(z);
             p.xn_hi[(size_t)m * d + i] = zh;
             p.xn_lo[(size_t)m * d + i] = __float2bfloat16_rn(z - __bfloat162float(zh));
-            sq += v * v;
+            sq += v[j] * v[j];
         }
         sq = warp_sum(sq);
         if (lane == 0) p.ss[m * n_tiles + t] = sq;
@@ -1422,6 +1480,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams
             if (passed && n_barrier == 1 && blockIdx.x == 0) *p.seq = s_seq + 1u;
             return passed;
         };
+        // every row's attention within the first segment: no partials to combine
+        const bool one_segment = pos0 + p.M <= kAttnSegChunks * kAttnChunk;
         for (int o = 0; o < p.n_ops; ++o) {
             unsigned long long* ct = stamps(o);
             if (ct && threadIdx.x == 0) ct[0] = globaltimer();
@@ -1439,24 +1499,27 @@ __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams
                 embed_op(p, pos0);
             } else {
                 // attention: segment partials; a grid barrier; then every CTA
-                // combines a share of the partials
+                // combines a share of the partials (tiny model at contexts up to
+                // 128, one segment: 6.8 us per layer with both, 4.8 without)
                 ok = attn_consume<R, HD>(op.at, p.M, pos0, smem, pp, p.err, ct, unit_stamps(o));
-                if (consumer_or(!ok)) {
-                    failed = true;
-                    break;
+                if (!one_segment) {
+                    if (consumer_or(!ok)) {
+                        failed = true;
+                        break;
+                    }
+                    if (ct && threadIdx.x == 0) ct[2] = globaltimer();
+                    barrier_arrive();
+                    if (threadIdx.x == 0) {
+                        mbar_arrive(&left);
+                        ok = barrier_wait();
+                        if (ct) ct[7] = globaltimer();
+                    }
+                    if (consumer_or(!ok)) {
+                        failed = true;
+                        break;
+                    }
+                    attn_combine<HD>(op.at, p.M, pos0);
                 }
-                if (ct && threadIdx.x == 0) ct[2] = globaltimer();
-                barrier_arrive();
-                if (threadIdx.x == 0) {
-                    mbar_arrive(&left);
-                    ok = barrier_wait();
-                    if (ct) ct[7] = globaltimer();
-                }
-                if (consumer_or(!ok)) {
-                    failed = true;
-                    break;
-                }
-                attn_combine<HD>(op.at, p.M, pos0);
             }
             if (ct && threadIdx.x == 0) ct[3] = globaltimer();
             // the end of op o in this CTA (its stores ordered before thread 0's
@@ -1469,7 +1532,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams
             if (o + 1 < p.n_ops) {
                 barrier_arrive();
                 if (threadIdx.x == 0) {
-                    if (type != OP_ATTN) mbar_arrive(&left);
+                    if (type != OP_ATTN || one_segment) mbar_arrive(&left);
                     ok = barrier_wait();
                     // producer and MMA warp have left op o, i.e. seen `go` for
                     // it: no completion of `go` is ever two ahead of a waiter
