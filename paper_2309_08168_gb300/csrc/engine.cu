@@ -813,6 +813,8 @@ int ssd_create(const ssd_config* cfg, const ssd_weights* w, void* cuda_stream, s
             (rc = dalloc(h, &h->pf_tmaps, (size_t)7 * L + 3 * kPfTokClasses, &B)))
             return bail(rc);
         P.pairs = h->n_sms / 2;
+        P.tm_k = h->tmaps + tmap_kv(h, 0);
+        P.tm_v = h->tmaps + tmap_kv(h, 1);
         cudaError_t ef = cudaMemset(P.flags, 0, prefill_flag_words(P.pairs) * sizeof(unsigned));
         if (ef != cudaSuccess) return bail(fail(SSD_ERR_CUDA, std::string("prefill flags: ") + cudaGetErrorString(ef)));
         P.x_lo = P.x_hi + R * d;

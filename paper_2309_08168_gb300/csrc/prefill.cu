@@ -10,7 +10,7 @@
 //   QKV GEMM   tcgen05 (tc_gemm.cuh), epilogue: RoPE, q (fp32) and the fp16
 //              K / V cache rows of the chunk's positions
 //   attention  causal flash attention of the chunk's rows over the cache
-//              [0, position] (mma.sync fp16, online softmax), output as bf16
+//              [0, position] (tcgen05, fp16, online softmax), output as bf16
 //              hi / lo planes
 //   O GEMM     tcgen05, epilogue: h += D
 //   norm, gate/up GEMM (epilogue: SwiGLU as bf16 hi / lo planes), down GEMM
@@ -66,35 +66,88 @@ __global__ void __launch_bounds__(kNormThreads) pf_norm_kernel(const float* __re
 }
 
 // ---------------------------------------------------------------------------
-// causal attention of the chunk's rows (flash attention, fp16 tensor cores)
+// causal attention of the chunk's rows (flash attention on tcgen05)
 // ---------------------------------------------------------------------------
-// CTA = 4 warps x 16 query rows of one query head; key blocks of 64
-// positions from the fp16 cache, double-buffered with cp.async; S = q K^T
-// with q as fp16 hi + lo, online softmax in fp32, O += P V with P as fp16
-// hi + lo.  Rows r < n_rows sit at positions pos0 + r and see keys
-// [0, pos0 + r].
-constexpr int kAttQ = 64, kAttKB = 64, kAttThreads = 128;
+// CTA = 128 query rows of one query head (the TMEM lanes), key blocks of 64
+// positions from the fp16 cache by TMA.  Rows r < n_rows sit at positions pos0 +
+// r and see keys [0, pos0 + r].
+//   warp 4      : TMA producer, kAttStages blocks of K and V;
+//   warp 5      : MMA issuer: S_j = q K_j^T (q as fp16 hi + lo in shared memory,
+//                 16 MMAs 128 x 64 x 16) one block ahead of O += P_j V_j (P as
+//                 fp16 hi + lo in TMEM, where it replaces S_j; V as it lies in
+//                 the cache, i.e. MN-major);
+//   warps 0-3   : softmax, one row per thread: S_j from TMEM, P_j back to it, the
+//                 running sum; at the end O / sum as bf16 hi / lo planes.
+// O is rescaled only when a row's maximum has grown by more than kAttSlack
+// (in log2) over the one its weights are relative to, so the weights stay below
+// 2^8 and the accumulator is rarely touched between blocks.
+// Bound by the softmax's issue slots (a thread per row, ~12 instructions a key).
+// The m16n8k16 kernel this replaces took 183 us a layer at 70B widths (1023 rows)
+// and 45 us at 7B widths (511 rows); this one PF_ATTN_US.
+constexpr int kAttQ = 128, kAttKB = 64, kAttStages = 4, kAttThreads = 192;
+constexpr float kAttSlack = 8.f;
 template <int HD>
-constexpr size_t att_smem_bytes() { return (size_t)4 * kAttKB * (HD + 8) * 2; }  // K, V double-buffered
+struct AttSmem {
+    static constexpr int BOXES = HD / 64;               // 64-dim boxes of a row
+    static constexpr int QB = kAttQ * 128;              // bytes of one box of q (hi or lo)
+    static constexpr int KB = kAttKB * 128;             // bytes of one box of K or V
+    static constexpr int STAGE = 2 * BOXES * KB;        // K boxes, then V boxes
+    static constexpr int Q = 2 * BOXES * QB;            // hi boxes, then lo boxes
+    static constexpr size_t BYTES = 1024 + (size_t)Q + (size_t)kAttStages * STAGE;
+};
+constexpr int kAttTmem = 256;  // O: 0 .. HD, S / P of even blocks at 128, of odd ones at 192
 
-__device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                         uint32_t b0, uint32_t b1) {
+__device__ __forceinline__ void att_tma3d(void* dst, const void* map, int x, int y, int z, uint64_t* bar) {
     asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 "
-        "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(smem_u32(dst)), "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
+        : "memory");
 }
-__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const void* p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(smem_u32(p)));
+// kind::f16, A = B = fp16, D = fp32, M = 128, N = n; B K-major or (V) MN-major
+__device__ __forceinline__ constexpr uint32_t att_idesc(int n, bool b_mn) {
+    return (1u << 4) | (b_mn ? 1u << 16 : 0u) | ((uint32_t)(n >> 3) << 17) | ((128u >> 4) << 24);
 }
-__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const void* p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(smem_u32(p)));
+__device__ __forceinline__ void att_mma_ss(uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+        ::"r"(d), "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+        : "memory");
 }
+__device__ __forceinline__ void att_mma_ts(uint32_t d, uint32_t a, uint64_t bd, uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n"
+        ::"r"(d), "r"(a), "l"(bd), "r"(idesc), "r"(acc)
+        : "memory");
+}
+__device__ __forceinline__ void att_commit(uint64_t* b) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(b))
+                 : "memory");
+}
+__device__ __forceinline__ void att_arrive(uint64_t* b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
+}
+#define SSD_R8(r, o) "=r"(r[o]), "=r"(r[o + 1]), "=r"(r[o + 2]), "=r"(r[o + 3]), "=r"(r[o + 4]), "=r"(r[o + 5]), "=r"(r[o + 6]), "=r"(r[o + 7])
+#define SSD_I8(r, o) "r"(r[o]), "r"(r[o + 1]), "r"(r[o + 2]), "r"(r[o + 3]), "r"(r[o + 4]), "r"(r[o + 5]), "r"(r[o + 6]), "r"(r[o + 7])
+// 32 columns of this thread's TMEM lane
+__device__ __forceinline__ void att_ld32(uint32_t t, uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : SSD_R8(r, 0), SSD_R8(r, 8), SSD_R8(r, 16), SSD_R8(r, 24)
+        : "r"(t));
+}
+__device__ __forceinline__ void att_st32(uint32_t t, const uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31};"
+        ::SSD_I8(r, 0), SSD_I8(r, 8), SSD_I8(r, 16), SSD_I8(r, 24), "r"(t)
+        : "memory");
+}
+#undef SSD_R8
+#undef SSD_I8
+__device__ __forceinline__ void att_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void att_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t pack_h2(float a, float b) {
     const __half2 v = __floats2half2_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&v);
@@ -107,184 +160,276 @@ __device__ __forceinline__ void split_h2(float a, float b, uint32_t& hi, uint32_
     lo = pack_h2(a - f.x, b - f.y);
 }
 
+struct AttArgs {
+    const float* q;     // [n_rows][H*hd] fp32, rotated
+    const void* tm_k;   // K / V cache as {hd, max_seq, L * Hkv} fp16, box {64, 64, 1}, 128-byte swizzle
+    const void* tm_v;
+    int kv_z0;          // z of this layer's KV head 0
+    int n_rows, pos0, n_heads, n_kv_heads;
+    float scale2;       // log2(e) / sqrt(hd)
+    bf16* out_hi;       // [n_rows][H*hd]
+    bf16* out_lo;
+    int* err;
+};
+
+// grid: heads x query tiles, the longest key ranges (last tiles) first
 template <int HD>
-__global__ void __launch_bounds__(kAttThreads) pf_attn_kernel(const float* __restrict__ q, const f16* __restrict__ kc,
-                                                              const f16* __restrict__ vc, int n_rows, int pos0,
-                                                              int n_heads, int n_kv_heads, int max_seq, float scale,
-                                                              bf16* __restrict__ out_hi, bf16* __restrict__ out_lo) {
-    constexpr int PITCH = HD + 8;  // halves per smem row (16-byte pad: conflict-free ldmatrix)
-    constexpr int KS = HD / 16;    // k steps of q K^T
-    constexpr int DN = HD / 8;     // n8 tiles of the output dims
-    extern __shared__ __align__(16) unsigned char att_smem[];  // K [2][64][PITCH], then V
-    __half(*sk)[kAttKB * PITCH] = reinterpret_cast<__half(*)[kAttKB * PITCH]>(att_smem);
-    __half(*sv)[kAttKB * PITCH] = reinterpret_cast<__half(*)[kAttKB * PITCH]>(att_smem + 2 * kAttKB * PITCH * 2);
-    const int head = blockIdx.y, kvh = (int)(((long long)head * n_kv_heads) / n_heads);
-    const int qr0 = blockIdx.x * kAttQ;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int qd = n_heads * HD;
-    const f16* kh = kc + (size_t)kvh * max_seq * HD;
-    const f16* vh = vc + (size_t)kvh * max_seq * HD;
-    const int last_row = min(n_rows, qr0 + kAttQ) - 1;
-    const int n_kb = (pos0 + last_row) / kAttKB + 1;
-
-    auto load_kv = [&](int kb, int buf) {
-        constexpr int CPR = HD / 8;  // 16-byte chunks per row
-        for (int c = threadIdx.x; c < kAttKB * CPR; c += kAttThreads) {
-            const int r = c / CPR, cc = c - r * CPR, key = kb * kAttKB + r;
-            const bool in = key < max_seq;
-            const size_t off = (size_t)(in ? key : 0) * HD + cc * 8;
-            cp_async16(&sk[buf][r * PITCH + cc * 8], kh + off, in ? 16 : 0);
-            cp_async16(&sv[buf][r * PITCH + cc * 8], vh + off, in ? 16 : 0);
+__global__ void __launch_bounds__(kAttThreads, 1) pf_attn_kernel(const AttArgs a) {
+    using L = AttSmem<HD>;
+    constexpr int BOXES = L::BOXES;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    __shared__ __align__(8) uint64_t kv_full[kAttStages], kv_empty[kAttStages];
+    __shared__ __align__(8) uint64_t q_ready, s_full[2], p_ready[2], pv_done[2];
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_fail;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int head = blockIdx.x, kvh = (int)(((long long)head * a.n_kv_heads) / a.n_heads);
+    const int qr0 = (int)(gridDim.y - 1 - blockIdx.y) * kAttQ;
+    const int qd = a.n_heads * HD;
+    const int n_kb = (a.pos0 + min(a.n_rows, qr0 + kAttQ) - 1) / kAttKB + 1;
+    if (threadIdx.x == 0) {
+        s_fail = 0;
+        for (int s = 0; s < kAttStages; ++s) {
+            tc::mb_init(kv_full + s, 1);
+            tc::mb_init(kv_empty + s, 1);
         }
-        cp_async_commit();
-    };
-    load_kv(0, 0);
-
-    // q fragments (rows g and g + 8 of this warp's 16), fp16 hi + lo
-    const int ra = qr0 + warp * 16 + g, rb = ra + 8;
-    uint32_t qh[KS][4], ql[KS][4];
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks) {
-        const int c = ks * 16 + 2 * t;
-        float2 x[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        if (ra < n_rows) {
-            x[0] = *reinterpret_cast<const float2*>(q + (size_t)ra * qd + head * HD + c);
-            x[2] = *reinterpret_cast<const float2*>(q + (size_t)ra * qd + head * HD + c + 8);
+        tc::mb_init(&q_ready, 4);
+        for (int b = 0; b < 2; ++b) {
+            tc::mb_init(s_full + b, 1);
+            tc::mb_init(p_ready + b, 4);  // one arrival per softmax warp
+            tc::mb_init(pv_done + b, 1);
         }
-        if (rb < n_rows) {
-            x[1] = *reinterpret_cast<const float2*>(q + (size_t)rb * qd + head * HD + c);
-            x[3] = *reinterpret_cast<const float2*>(q + (size_t)rb * qd + head * HD + c + 8);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) split_h2(x[i].x, x[i].y, qh[ks][i], ql[ks][i]);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    const int pa = pos0 + ra, pb = pos0 + rb;  // positions of rows g and g + 8
+    if (warp == 4) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(kAttTmem)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    const uint32_t tmem = s_tmem;
+    unsigned char* kv = smem + L::Q;
+    bool ok = true;
 
-    float o[DN][4];
+    if (warp == 4) {
+        asm volatile("fence.proxy.async.global;" ::: "memory");  // K / V rows the previous kernel wrote
+        for (int j = 0; j < n_kb && ok; ++j) {
+            const int s = j % kAttStages;
+            ok = __all_sync(0xffffffffu, tc::mb_wait(kv_empty + s, (j / kAttStages + 1) & 1u, a.err));
+            if (!ok) break;
+            if (elect_one()) {
+                unsigned char* st = kv + s * L::STAGE;
+                tc::mb_arrive_tx(kv_full + s, (unsigned)L::STAGE);
 #pragma unroll
-    for (int j = 0; j < DN; ++j) o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
-    float ma = -INFINITY, mb = -INFINITY, la = 0.f, lb = 0.f;
-
-    for (int kb = 0; kb < n_kb; ++kb) {
-        const int buf = kb & 1;
-        if (kb + 1 < n_kb) {
-            load_kv(kb + 1, buf ^ 1);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
+                for (int b = 0; b < BOXES; ++b) {
+                    att_tma3d(st + b * L::KB, a.tm_k, b * 64, j * kAttKB, a.kv_z0 + kvh, kv_full + s);
+                    att_tma3d(st + (BOXES + b) * L::KB, a.tm_v, b * 64, j * kAttKB, a.kv_z0 + kvh, kv_full + s);
+                }
+            }
+            __syncwarp();
         }
-        __syncthreads();
-        // S = q K^T over the block's 64 keys: 8 n8 tiles
-        float s[8][4];
+    } else if (warp == 5) {
+        const uint64_t q0 = tc::sdesc(smem_u32(smem)), kv0 = tc::sdesc(smem_u32(kv));
+        auto wait = [&](uint64_t* b, int phase) {
+            ok = ok && __all_sync(0xffffffffu, tc::mb_wait(b, (unsigned)phase & 1u, a.err));
+            return ok;
+        };
+        // S_j; the block's K has landed and P_{j-2}, which held these columns, is used up
+        auto scores = [&](int j) {
+            if (!wait(kv_full + j % kAttStages, j / kAttStages)) return;
+            if (j >= 2 && !wait(pv_done + (j & 1), (j - 2) >> 1)) return;
+            tc::fence_after();
+            if (elect_one()) {
+                const uint64_t k0 = kv0 + (uint64_t)((j % kAttStages) * (L::STAGE >> 4));
+                const uint32_t d = tmem + 128u + 64u * (uint32_t)(j & 1);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) s[j][0] = s[j][1] = s[j][2] = s[j][3] = 0.f;
+                for (int h = 0; h < 2; ++h)  // hi, lo
 #pragma unroll
-        for (int ks = 0; ks < KS; ++ks) {
+                    for (int b = 0; b < BOXES; ++b)
 #pragma unroll
-            for (int j = 0; j < 8; j += 2) {
-                uint32_t b[4];
-                const int key = j * 8 + (lane & 7) + ((lane >> 4) << 3);
-                const int dim = ks * 16 + ((lane >> 3) & 1) * 8;
-                ldsm4(b, &sk[buf][key * PITCH + dim]);
-                mma16816(s[j], qh[ks][0], qh[ks][1], qh[ks][2], qh[ks][3], b[0], b[1]);
-                mma16816(s[j], ql[ks][0], ql[ks][1], ql[ks][2], ql[ks][3], b[0], b[1]);
-                mma16816(s[j + 1], qh[ks][0], qh[ks][1], qh[ks][2], qh[ks][3], b[2], b[3]);
-                mma16816(s[j + 1], ql[ks][0], ql[ks][1], ql[ks][2], ql[ks][3], b[2], b[3]);
+                        for (int ks = 0; ks < 4; ++ks)
+                            att_mma_ss(d, q0 + (uint64_t)(((h * BOXES + b) * L::QB + ks * 32) >> 4),
+                                       k0 + (uint64_t)((b * L::KB + ks * 32) >> 4), att_idesc(64, false),
+                                       (h | b | ks) ? 1u : 0u);
+                att_commit(s_full + (j & 1));
+            }
+            __syncwarp();
+        };
+        wait(&q_ready, 0);
+        if (ok) scores(0);
+        for (int j = 0; j < n_kb && ok; ++j) {
+            if (j + 1 < n_kb) scores(j + 1);
+            if (!ok || !wait(p_ready + (j & 1), j >> 1)) break;
+            tc::fence_after();
+            if (elect_one()) {
+                // V: 64 dims (MN) x 16 keys (K) per MMA; 8 keys are 1024 bytes apart
+                const uint64_t v0 = kv0 + (uint64_t)(((j % kAttStages) * L::STAGE + BOXES * L::KB) >> 4);
+                const uint64_t mn = (uint64_t)((1024 >> 4) - 1) << 16;  // leading byte offset 1024 too
+                const uint32_t p = tmem + 128u + 64u * (uint32_t)(j & 1);
+#pragma unroll
+                for (int b = 0; b < BOXES; ++b)
+#pragma unroll
+                    for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+                            att_mma_ts(tmem + 64u * b, p + 32u * h + 8u * ks, v0 + mn + (uint64_t)((b * L::KB + ks * 2048) >> 4),
+                                       att_idesc(64, true), (j | ks | h) ? 1u : 0u);
+                att_commit(kv_empty + j % kAttStages);
+                att_commit(pv_done + (j & 1));
+            }
+            __syncwarp();
+        }
+    } else {
+        // q of the tile as fp16 hi + lo, scaled to log2 units: a warp takes 32
+        // rows, a row at a time (K-major, 128-byte swizzle: row r of a 64-dim
+        // box at r * 128, 16-byte chunk c at (c ^ (r & 7)) * 16)
+        constexpr int LPR = HD / 4, RPI = 32 / LPR;  // lanes per row, rows per step
+        for (int i0 = 0; i0 < 32; i0 += 8 * RPI) {
+            float4 x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int r = warp * 32 + i0 + i * RPI + lane / LPR, e = (lane % LPR) * 4;
+                x[i] = qr0 + r < a.n_rows
+                           ? *reinterpret_cast<const float4*>(a.q + (size_t)(qr0 + r) * qd + head * HD + e)
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int r = warp * 32 + i0 + i * RPI + lane / LPR, e = (lane % LPR) * 4;
+                uint2 hi, lo;
+                split_h2(x[i].x * a.scale2, x[i].y * a.scale2, hi.x, lo.x);
+                split_h2(x[i].z * a.scale2, x[i].w * a.scale2, hi.y, lo.y);
+                unsigned char* at = smem + (e >> 6) * L::QB + r * 128 + ((((e & 63) >> 3) ^ (r & 7)) << 4) + (e & 7) * 2;
+                *reinterpret_cast<uint2*>(at) = hi;
+                *reinterpret_cast<uint2*>(at + BOXES * L::QB) = lo;
             }
         }
-        // scale, causal mask, online softmax (rows g: s[.][0..1], g + 8: s[.][2..3])
-        float bma = -INFINITY, bmb = -INFINITY;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) att_arrive(&q_ready);
+
+        const int row = qr0 + warp * 32 + lane, pos = a.pos0 + row;  // this thread's query row
+        const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
+        float mx = 0.f, l = 0.f;  // reference maximum of the weights, their sum
+        for (int j = 0; j < n_kb && ok; ++j) {
+            const uint32_t ts = tl + 128u + 64u * (uint32_t)(j & 1);
+            ok = __all_sync(0xffffffffu, tc::mb_wait(s_full + (j & 1), (unsigned)(j >> 1) & 1u, a.err));
+            if (!ok) break;
+            tc::fence_after();
+            uint32_t u0[32], u1[32];
+            att_ld32(ts, u0);
+            att_ld32(ts + 32, u1);
+            att_wait_ld();
+            const int last = pos - j * kAttKB;  // the row sees keys 0 .. last of the block
+            if ((j + 1) * kAttKB - 1 > a.pos0 + qr0) {  // (uniform) some row of the tile does not see all
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int key = kb * kAttKB + j * 8 + 2 * t;
-            s[j][0] = key <= pa ? s[j][0] * scale : -INFINITY;
-            s[j][1] = key + 1 <= pa ? s[j][1] * scale : -INFINITY;
-            s[j][2] = key <= pb ? s[j][2] * scale : -INFINITY;
-            s[j][3] = key + 1 <= pb ? s[j][3] * scale : -INFINITY;
-            bma = fmaxf(bma, fmaxf(s[j][0], s[j][1]));
-            bmb = fmaxf(bmb, fmaxf(s[j][2], s[j][3]));
+                for (int i = 0; i < 32; ++i) {
+                    if (i > last) u0[i] = __float_as_uint(-INFINITY);
+                    if (i + 32 > last) u1[i] = __float_as_uint(-INFINITY);
+                }
+            }
+            float bm4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};  // (short dependency chains)
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                bm4[i & 3] = fmaxf(bm4[i & 3], fmaxf(__uint_as_float(u0[i]), __uint_as_float(u1[i])));
+            const float bm = fmaxf(fmaxf(bm4[0], bm4[1]), fmaxf(bm4[2], bm4[3]));
+            if (j == 0) {
+                mx = bm;
+            } else if (__any_sync(0xffffffffu, bm > mx + kAttSlack)) {
+                // O and the sum move to the new maximum (all rows of the warp)
+                ok = __all_sync(0xffffffffu, tc::mb_wait(pv_done + ((j - 1) & 1), (unsigned)((j - 1) >> 1) & 1u, a.err));
+                if (!ok) break;
+                tc::fence_after();
+                const float nm = fmaxf(mx, bm), f = exp2f(mx - nm);
+                for (int c = 0; c < HD; c += 32) {
+                    uint32_t o[32];
+                    att_ld32(tl + c, o);
+                    att_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * f);
+                    att_st32(tl + c, o);
+                }
+                l *= f;
+                mx = nm;
+            }
+            uint32_t hi[32], lo[32];
+            float l4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const float p0 = exp2f(__uint_as_float(u0[2 * i]) - mx), p1 = exp2f(__uint_as_float(u0[2 * i + 1]) - mx);
+                const float p2 = exp2f(__uint_as_float(u1[2 * i]) - mx), p3 = exp2f(__uint_as_float(u1[2 * i + 1]) - mx);
+                l4[i & 3] += (p0 + p1) + (p2 + p3);
+                split_h2(p0, p1, hi[i], lo[i]);
+                split_h2(p2, p3, hi[i + 16], lo[i + 16]);
+            }
+            l += (l4[0] + l4[1]) + (l4[2] + l4[3]);
+            att_st32(ts, hi);
+            att_st32(ts + 32, lo);
+            att_wait_st();
+            tc::fence_before();
+            __syncwarp();
+            if (lane == 0) att_arrive(p_ready + (j & 1));
         }
+        if (ok) ok = __all_sync(0xffffffffu, tc::mb_wait(pv_done + ((n_kb - 1) & 1), (unsigned)((n_kb - 1) >> 1) & 1u, a.err));
+        if (ok) {
+            tc::fence_after();
+            const float inv = l > 0.f ? 1.f / l : 0.f;
+            for (int c = 0; c < HD; c += 32) {
+                uint32_t o[32];
+                att_ld32(tl + c, o);
+                att_wait_ld();
+                if (row < a.n_rows) {
+                    const size_t at = (size_t)row * qd + head * HD + c;
 #pragma unroll
-        for (int off = 1; off < 4; off <<= 1) {
-            bma = fmaxf(bma, __shfl_xor_sync(0xffffffffu, bma, off));
-            bmb = fmaxf(bmb, __shfl_xor_sync(0xffffffffu, bmb, off));
-        }
-        const float na = fmaxf(ma, bma), nb = fmaxf(mb, bmb);
-        // rows past the chunk hold no keys: keep them finite and zero
-        const float ca = na == -INFINITY ? 1.f : expf(ma - na), cb = nb == -INFINITY ? 1.f : expf(mb - nb);
-        ma = na;
-        mb = nb;
-        float sa = 0.f, sb = 0.f;
+                    for (int i = 0; i < 32; i += 8) {
+                        __align__(16) bf16 h8[8], l8[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            s[j][0] = s[j][0] == -INFINITY ? 0.f : expf(s[j][0] - na);
-            s[j][1] = s[j][1] == -INFINITY ? 0.f : expf(s[j][1] - na);
-            s[j][2] = s[j][2] == -INFINITY ? 0.f : expf(s[j][2] - nb);
-            s[j][3] = s[j][3] == -INFINITY ? 0.f : expf(s[j][3] - nb);
-            sa += s[j][0] + s[j][1];
-            sb += s[j][2] + s[j][3];
-        }
-        la = la * ca + sa;  // (quad partial sums; reduced once at the end)
-        lb = lb * cb + sb;
-#pragma unroll
-        for (int j = 0; j < DN; ++j) {
-            o[j][0] *= ca;
-            o[j][1] *= ca;
-            o[j][2] *= cb;
-            o[j][3] *= cb;
-        }
-        // O += P V: k steps of 16 keys; P from the S accumulators (hi + lo)
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-            uint32_t ph[4], pl[4];
-            split_h2(s[2 * kk][0], s[2 * kk][1], ph[0], pl[0]);
-            split_h2(s[2 * kk][2], s[2 * kk][3], ph[1], pl[1]);
-            split_h2(s[2 * kk + 1][0], s[2 * kk + 1][1], ph[2], pl[2]);
-            split_h2(s[2 * kk + 1][2], s[2 * kk + 1][3], ph[3], pl[3]);
-#pragma unroll
-            for (int dn = 0; dn < DN; dn += 2) {
-                uint32_t b[4];
-                const int key = kk * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-                const int dim = dn * 8 + (lane >> 4) * 8;
-                ldsm4t(b, &sv[buf][key * PITCH + dim]);
-                mma16816(o[dn], ph[0], ph[1], ph[2], ph[3], b[0], b[1]);
-                mma16816(o[dn], pl[0], pl[1], pl[2], pl[3], b[0], b[1]);
-                mma16816(o[dn + 1], ph[0], ph[1], ph[2], ph[3], b[2], b[3]);
-                mma16816(o[dn + 1], pl[0], pl[1], pl[2], pl[3], b[2], b[3]);
+                        for (int k = 0; k < 8; ++k) {
+                            const float v = __uint_as_float(o[i + k]) * inv;
+                            h8[k] = __float2bfloat16_rn(v);
+                            l8[k] = __float2bfloat16_rn(v - __bfloat162float(h8[k]));
+                        }
+                        *reinterpret_cast<uint4*>(a.out_hi + at + i) = *reinterpret_cast<const uint4*>(h8);
+                        *reinterpret_cast<uint4*>(a.out_lo + at + i) = *reinterpret_cast<const uint4*>(l8);
+                    }
+                }
             }
         }
-        __syncthreads();  // the buffer is refilled two blocks later
     }
-#pragma unroll
-    for (int off = 1; off < 4; off <<= 1) {
-        la += __shfl_xor_sync(0xffffffffu, la, off);
-        lb += __shfl_xor_sync(0xffffffffu, lb, off);
+    if (!ok) s_fail = 1;
+    tc::fence_before();
+    __syncwarp();
+    __syncthreads();
+    if (s_fail && threadIdx.x == 0) {  // let copies and MMAs in flight finish
+        const unsigned long long t0 = tc::gtime();
+        while (tc::gtime() - t0 < 2000000ull) __nanosleep(1000);
     }
-    const float ia = la > 0.f ? 1.f / la : 0.f, ib = lb > 0.f ? 1.f / lb : 0.f;
-#pragma unroll
-    for (int dn = 0; dn < DN; ++dn) {
-        const int c = head * HD + dn * 8 + 2 * t;
-        if (ra < n_rows) {
-            const size_t at = (size_t)ra * qd + c;
-            tc::store_hilo(out_hi + at, out_lo + at, o[dn][0] * ia);
-            tc::store_hilo(out_hi + at + 1, out_lo + at + 1, o[dn][1] * ia);
-        }
-        if (rb < n_rows) {
-            const size_t at = (size_t)rb * qd + c;
-            tc::store_hilo(out_hi + at, out_lo + at, o[dn][2] * ib);
-            tc::store_hilo(out_hi + at + 1, out_lo + at + 1, o[dn][3] * ib);
-        }
+    __syncthreads();
+    if (warp == 4) {
+        tc::fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kAttTmem) : "memory");
     }
+}
+
+template <int HD>
+int launch_attn(const AttArgs& a, cudaStream_t s) {
+    pf_attn_kernel<HD><<<dim3(a.n_heads, (a.n_rows + kAttQ - 1) / kAttQ), kAttThreads, AttSmem<HD>::BYTES, s>>>(a);
+    return (int)cudaGetLastError();
 }
 
 }  // namespace
 
 int prefill_configure() {
     int e = (int)cudaFuncSetAttribute(pf_attn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)att_smem_bytes<128>());
+                                      (int)AttSmem<128>::BYTES);
     if (!e)
         e = (int)cudaFuncSetAttribute(pf_attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)att_smem_bytes<64>());
+                                      (int)AttSmem<64>::BYTES);
     if (!e) e = tc::tc_configure<tc::TC_QKV>();
     if (!e) e = tc::tc_configure<tc::TC_RESID>();
     if (!e) e = tc::tc_configure<tc::TC_SWIGLU>();
@@ -335,15 +480,20 @@ int prefill_chunk(PrefillPlan& P, const int* toks, int n, int pos0, cudaStream_t
         a.rope = P.rope;
         e = tc::tc_launch<tc::TC_QKV>(a, s);
         if (e) break;
-        const dim3 ag((n + kAttQ - 1) / kAttQ, P.n_heads);
-        const float scale = 1.0f / std::sqrt((float)P.head_dim);
-        if (P.head_dim == 128)
-            pf_attn_kernel<128><<<ag, kAttThreads, att_smem_bytes<128>(), s>>>(P.q, L.k_cache, L.v_cache, n, pos0, P.n_heads,
-                                                           P.n_kv_heads, P.max_seq, scale, P.at_hi, P.at_lo);
-        else
-            pf_attn_kernel<64><<<ag, kAttThreads, att_smem_bytes<64>(), s>>>(P.q, L.k_cache, L.v_cache, n, pos0, P.n_heads,
-                                                          P.n_kv_heads, P.max_seq, scale, P.at_hi, P.at_lo);
-        e = (int)cudaGetLastError();
+        AttArgs t{};
+        t.q = P.q;
+        t.tm_k = P.tm_k;
+        t.tm_v = P.tm_v;
+        t.kv_z0 = l * P.n_kv_heads;
+        t.n_rows = n;
+        t.pos0 = pos0;
+        t.n_heads = P.n_heads;
+        t.n_kv_heads = P.n_kv_heads;
+        t.scale2 = (float)(1.4426950408889634 / std::sqrt((double)P.head_dim));
+        t.out_hi = P.at_hi;
+        t.out_lo = P.at_lo;
+        t.err = P.err;
+        e = P.head_dim == 128 ? launch_attn<128>(t, s) : launch_attn<64>(t, s);
         if (e) break;
         tc::TcArgs o = gemm(P.tm_at, d, (d + tc::kFeat - 1) / tc::kFeat, qd);
         o.tm_w[0] = L.tm_w[3];

@@ -188,6 +188,8 @@ struct PrefillPlan {
     const void* tm_x[kPfTokClasses];
     const void* tm_at[kPfTokClasses];
     const void* tm_ac[kPfTokClasses];
+    const void* tm_k;      // K / V cache maps of the decode kernel (AttnArgs)
+    const void* tm_v;
     int pairs;             // CTA pairs of the GEMMs (half the SMs)
     float* ws;             // split tiles: partial sums [pairs][2][256][128]
     unsigned* flags;       // and their flags [pairs][2][16] (TcArgs)
