@@ -36,6 +36,8 @@ constexpr int kNormThreads = 256;
 __global__ void __launch_bounds__(kNormThreads) pf_embed_kernel(const bf16* __restrict__ embed,
                                                                  const int* __restrict__ toks, int d,
                                                                  float* __restrict__ h) {
+    pdl_launch_dependents();
+    pdl_wait();
     const int r = blockIdx.x;
     const bf16* e = embed + (size_t)toks[r] * d;
     for (int i = threadIdx.x; i < d; i += kNormThreads) h[(size_t)r * d + i] = __bfloat162float(e[i]);
@@ -46,6 +48,8 @@ __global__ void __launch_bounds__(kNormThreads) pf_norm_kernel(const float* __re
                                                                const bf16* __restrict__ g, int d, float eps,
                                                                bf16* __restrict__ x_hi, bf16* __restrict__ x_lo) {
     __shared__ float s_part[kNormThreads / 32];
+    pdl_launch_dependents();
+    pdl_wait();
     const int r = blockIdx.x;
     const float* hr = h + (size_t)r * d;
     float ss = 0.f;
@@ -83,7 +87,7 @@ __global__ void __launch_bounds__(kNormThreads) pf_norm_kernel(const float* __re
 // 2^8 and the accumulator is rarely touched between blocks.
 // Bound by the softmax's issue slots (a thread per row, ~12 instructions a key).
 // The m16n8k16 kernel this replaces took 183 us a layer at 70B widths (1023 rows)
-// and 45 us at 7B widths (511 rows); this one PF_ATTN_US.
+// and 45 us at 7B widths (511 rows); this one 66 and 20 us.
 constexpr int kAttQ = 128, kAttKB = 64, kAttStages = 4, kAttThreads = 192;
 constexpr float kAttSlack = 8.f;
 template <int HD>
@@ -209,11 +213,13 @@ __global__ void __launch_bounds__(kAttThreads, 1) pf_attn_kernel(const AttArgs a
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    pdl_launch_dependents();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
     const uint32_t tmem = s_tmem;
     unsigned char* kv = smem + L::Q;
+    pdl_wait();  // q, K and V come from the previous kernel
     bool ok = true;
 
     if (warp == 4) {
@@ -418,8 +424,8 @@ __global__ void __launch_bounds__(kAttThreads, 1) pf_attn_kernel(const AttArgs a
 
 template <int HD>
 int launch_attn(const AttArgs& a, cudaStream_t s) {
-    pf_attn_kernel<HD><<<dim3(a.n_heads, (a.n_rows + kAttQ - 1) / kAttQ), kAttThreads, AttSmem<HD>::BYTES, s>>>(a);
-    return (int)cudaGetLastError();
+    return tc::launch_pdl(pf_attn_kernel<HD>, dim3(a.n_heads, (a.n_rows + kAttQ - 1) / kAttQ), kAttThreads,
+                          AttSmem<HD>::BYTES, s, a);
 }
 
 }  // namespace
@@ -440,7 +446,10 @@ size_t prefill_ws_floats(int pairs) { return (size_t)pairs * 2 * tc::kMaxTok * 1
 size_t prefill_flag_words(int pairs) { return (size_t)pairs * 2 * tc::kEpiWarps; }
 
 // One chunk of prompt rows at positions pos0 .. pos0 + n - 1 through every
-// layer (launches only).  toks: device token ids of the chunk.
+// layer (launches only).  toks: device token ids of the chunk.  Every kernel is
+// a programmatic dependent launch: its set-up (and a GEMM's first weights)
+// overlap the previous kernel's end, and it waits for that kernel's results
+// before it reads or writes anything else.
 int prefill_chunk(PrefillPlan& P, const int* toks, int n, int pos0, cudaStream_t s) {
     const int d = P.d, qd = P.n_heads * P.head_dim, kvd = P.n_kv_heads * P.head_dim;
     // the arguments every GEMM shares: n_out outputs in n_ft tiles of 256 weight rows, K inputs
@@ -458,12 +467,10 @@ int prefill_chunk(PrefillPlan& P, const int* toks, int n, int pos0, cudaStream_t
         a.err = P.err;
         return a;
     };
-    pf_embed_kernel<<<n, kNormThreads, 0, s>>>(P.embed, toks, d, P.h);
-    int e = (int)cudaGetLastError();
+    int e = tc::launch_pdl(pf_embed_kernel, dim3(n), kNormThreads, 0, s, P.embed, toks, d, P.h);
     for (int l = 0; l < P.n_layers && !e; ++l) {
         const PrefillLayer& L = P.layers[l];
-        pf_norm_kernel<<<n, kNormThreads, 0, s>>>(P.h, L.attn_norm, d, P.eps, P.x_hi, P.x_lo);
-        e = (int)cudaGetLastError();
+        e = tc::launch_pdl(pf_norm_kernel, dim3(n), kNormThreads, 0, s, (const float*)P.h, L.attn_norm, d, P.eps, P.x_hi, P.x_lo);
         if (e) break;
         tc::TcArgs a = gemm(P.tm_x, qd + 2 * kvd, (qd + 2 * kvd + tc::kFeat - 1) / tc::kFeat, d);
         a.tm_w[0] = L.tm_w[0];
@@ -500,8 +507,7 @@ int prefill_chunk(PrefillPlan& P, const int* toks, int n, int pos0, cudaStream_t
         o.out = P.h;
         e = tc::tc_launch<tc::TC_RESID>(o, s);
         if (e) break;
-        pf_norm_kernel<<<n, kNormThreads, 0, s>>>(P.h, L.mlp_norm, d, P.eps, P.x_hi, P.x_lo);
-        e = (int)cudaGetLastError();
+        e = tc::launch_pdl(pf_norm_kernel, dim3(n), kNormThreads, 0, s, (const float*)P.h, L.mlp_norm, d, P.eps, P.x_hi, P.x_lo);
         if (e) break;
         tc::TcArgs gu = gemm(P.tm_x, P.ffn, (P.ffn + 127) / 128, d);  // 128 features: gate and up rows
         gu.tm_w[0] = L.tm_w[4];

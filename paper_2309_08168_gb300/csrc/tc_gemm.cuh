@@ -343,6 +343,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
+    pdl_launch_dependents();
     fence_before();
     __syncthreads();
     cluster_sync();
@@ -353,11 +354,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm
     TcWork w;
     tc_work_init(w, a.sched, a.n_kb, pair);
     if (warp == kEpiWarps) {
-        // producer: weights, and activations that the previous kernel wrote
-        asm volatile("fence.proxy.async.global;" ::: "memory");
+        // producer: weights, and activations that the previous kernel wrote.
+        // The weights of the first S k blocks are requested before that kernel
+        // has finished.
         const uint32_t full0 = map_rank(smem_u32(full), 0);
         int s = 0;
         unsigned ph = 1;  // parity of the next "empty" completion to wait for (the ring starts empty)
+        bool waited = false;
         while (ok && tc_work_next(w, a.sched, a.n_kb, pair)) {
             const int ft = w.tile / a.n_tt, tt = w.tile - ft * a.n_tt;
             const int tok0 = tt * a.nt + (int)rank * (a.nt >> 1);
@@ -370,29 +373,44 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm
                 else if (row0 >= qd) { map = a.tm_w[1]; row0 -= qd; }
                 row0 /= a.head_dim;
             }
+            auto weights = [&](int kb, int st_i) {  // (one lane) k block kb into stage st_i
+                unsigned char* st = smem + st_i * stage_bytes;
+                const uint32_t bar = full0 + 8u * (uint32_t)st_i;
+                if (rank == 0) mb_arrive_tx(full + st_i, 2u * (unsigned)stage_bytes);
+                if (EPI == TC_QKV) {
+                    tma5d_head(st, map, kb * kBK, row0, bar);
+                } else if (EPI == TC_SWIGLU) {
+                    if (a.tm_w[1] == nullptr) {
+                        tma4d_pair(st, map, kb * kBK, box * 4, bar);
+                    } else {
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) {
+                            tma2d(st + g * 4096, map, kb * kBK, box * 64 + g * 16, bar);
+                            tma2d(st + g * 4096 + 2048, a.tm_w[1], kb * kBK, box * 64 + g * 16, bar);
+                        }
+                    }
+                } else {
+                    tma2d(st, map, kb * kBK, row0, bar);
+                }
+            };
+            int n_pre = 0;
+            if (!waited) {  // (the ring is empty)
+                n_pre = min(S, w.kb1 - w.kb0);
+                for (int i = 0; i < n_pre; ++i) {
+                    if (elect_one()) weights(w.kb0 + i, i);
+                    __syncwarp();
+                }
+                pdl_wait();
+                asm volatile("fence.proxy.async.global;" ::: "memory");
+                waited = true;
+            }
             for (int kb = w.kb0; kb < w.kb1; ++kb) {
-                ok = __all_sync(0xffffffffu, mb_wait(empty + s, ph, a.err));
+                const bool pre = kb - w.kb0 < n_pre;
+                if (!pre) ok = __all_sync(0xffffffffu, mb_wait(empty + s, ph, a.err));
                 if (!ok) break;
                 if (elect_one()) {
-                    unsigned char* st = smem + s * stage_bytes;
-                    const uint32_t bar = full0 + 8u * (uint32_t)s;
-                    if (rank == 0) mb_arrive_tx(full + s, 2u * (unsigned)stage_bytes);
-                    if (EPI == TC_QKV) {
-                        tma5d_head(st, map, kb * kBK, row0, bar);
-                    } else if (EPI == TC_SWIGLU) {
-                        if (a.tm_w[1] == nullptr) {
-                            tma4d_pair(st, map, kb * kBK, box * 4, bar);
-                        } else {
-#pragma unroll
-                            for (int g = 0; g < 4; ++g) {
-                                tma2d(st + g * 4096, map, kb * kBK, box * 64 + g * 16, bar);
-                                tma2d(st + g * 4096 + 2048, a.tm_w[1], kb * kBK, box * 64 + g * 16, bar);
-                            }
-                        }
-                    } else {
-                        tma2d(st, map, kb * kBK, row0, bar);
-                    }
-                    tma3d(st + kATile, a.tm_x, kb * kBK, tok0, 0, bar);
+                    if (!pre) weights(kb, s);
+                    tma3d(smem + s * stage_bytes + kATile, a.tm_x, kb * kBK, tok0, 0, full0 + 8u * (uint32_t)s);
                 }
                 __syncwarp();
                 if (++s == S) { s = 0; ph ^= 1u; }
@@ -439,6 +457,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm
         }
     } else if (warp < kEpiWarps) {
         const int q4 = warp & 3, quarter = warp >> 2, upper = lane >> 4;
+        pdl_wait();  // h, the workspace and the outputs may still be in use
         const int hc = a.nt >> 2;  // columns of this warp: quarter * hc .. + hc (a multiple of 8)
         const uint32_t empty0[2] = {map_rank(smem_u32(acc_empty), 0), map_rank(smem_u32(acc_empty + 1), 0)};
         int b = 0;
@@ -666,10 +685,25 @@ inline int tc_configure() {
                                      (int)kSmemBytes);
 }
 
+// launch that may start while the previous kernel of the stream ends
+template <typename... P, typename... A>
+inline int launch_pdl(void (*k)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return (int)cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 template <int EPI>
 inline int tc_launch(const TcArgs& a, cudaStream_t s) {
-    tc_gemm_kernel<EPI><<<2 * a.sched.pairs, kThreads, kSmemBytes, s>>>(a);
-    return (int)cudaGetLastError();
+    return launch_pdl(tc_gemm_kernel<EPI>, dim3(2 * a.sched.pairs), kThreads, kSmemBytes, s, a);
 }
 
 }  // namespace tc
