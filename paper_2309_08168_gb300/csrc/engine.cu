@@ -15,6 +15,7 @@
 // Everything between two rounds stays on the device; the host reads one int
 // (tokens emitted so far) per round to size the next round.
 #include <cmath>
+#include <cstddef>
 #include <cstdlib>
 #include <cstring>
 #include <map>
@@ -103,7 +104,7 @@ struct ssd_handle {
     bf16* ac_hi = nullptr;  // SwiGLU output planes [16][ffn]
     bf16* ac_lo = nullptr;
     int n_sms = 0;
-    unsigned* bar = nullptr;            // grid-barrier counter of the forward kernel, then its sequence number
+    unsigned* bar = nullptr;            // [2] grid-barrier counters of the forward kernel, then its sequence number
     unsigned long long* trace = nullptr;  // per-op timestamps (profiling hook, FwdParams::trace)
     int trace_op = -1;                    // op traced per unit and per CTA
     CUtensorMap* tmaps = nullptr;       // TMA descriptors (weights, input planes) in device memory
@@ -119,7 +120,7 @@ struct ssd_handle {
     float* attn_part = nullptr;
     int n_chunks = 0;
     float2* rope = nullptr;
-    int* tok = nullptr;  // [max_seq] prompt | [16] debug rows
+    int* tok = nullptr;  // [max_seq] prompt
     int* out = nullptr;  // [max_seq]
     int* argbuf = nullptr;
     DecodeState* st = nullptr;
@@ -130,6 +131,7 @@ struct ssd_handle {
     std::map<int, int> graph_launches;  // kernels per replay
     std::vector<cudaEvent_t> events;
 
+    bool clean = false;  // error flag and counters are at zero (begin_launches)
     bool prefilled = false;
     int n_prompt = 0;
     int last_prompt_token = 0;
@@ -480,7 +482,8 @@ int upload_ops(ssd_handle* h, bool draft) {
 
 // One decoder forward over M rows: a single cooperative launch of the forward
 // kernel over the op list (lm_head dropped when no logits are needed).
-// Launches only; no host synchronisation (graph-capturable).
+// Launches only; no host synchronisation (graph-capturable).  toks: M token ids
+// in host memory (SRC_TOKENS), passed as kernel arguments.
 int forward(ssd_handle* h, int M, int src, const int* toks, int pos0, bool draft, bool logits,
             int* n_launch = nullptr, unsigned long long* trace = nullptr, int stall_barrier = 0) {
     const ssd_config& c = h->cfg;
@@ -489,7 +492,7 @@ int forward(ssd_handle* h, int M, int src, const int* toks, int pos0, bool draft
     p.n_ops = (draft ? h->n_ops_draft : h->n_ops_full) - (logits ? 0 : 1);
     p.M = M;
     p.src = src;
-    p.toks = toks;
+    if (toks) std::memcpy(p.toks, toks, sizeof(int) * M);
     p.pos0_arg = pos0;
     p.st = h->st;
     p.embed = h->embed;
@@ -500,15 +503,43 @@ int forward(ssd_handle* h, int M, int src, const int* toks, int pos0, bool draft
     p.xn_lo = h->xn_lo;
     p.ss = h->ss;
     p.bar = h->bar;
-    p.seq = h->bar + 1;
+    p.seq = h->bar + 2;
     p.err = &h->st->err;
     p.trace = trace;
     p.trace_op = h->trace_op;
     p.wait_ns = h->wait_ns;
     p.stall_barrier = stall_barrier;
-    CUDA_TRY(cudaMemsetAsync(h->bar, 0, sizeof(unsigned), h->stream), "barrier reset");
     LAUNCH(h, launch_forward(p, c.head_dim, h->n_sms, h->stream), "forward kernel", -1);
     if (n_launch) *n_launch = 1;
+    return SSD_OK;
+}
+
+// Before launches whose outcome the call checks.  A completed forward leaves the
+// device error flag, the acceptance kernels' arrival counter and the next
+// forward's barrier counter at zero; after a failed one, or one that nothing
+// checked, they are cleared here.
+int begin_launches(ssd_handle* h) {
+    if (!h->clean) {
+        CUDA_TRY(cudaMemsetAsync(&h->st->err, 0, sizeof(int), h->stream), "error flag reset");
+        CUDA_TRY(cudaMemsetAsync(h->counters, 0, 4 * sizeof(unsigned), h->stream), "counter reset");
+        CUDA_TRY(cudaMemsetAsync(h->bar, 0, 2 * sizeof(unsigned), h->stream), "barrier reset");
+    }
+    h->clean = false;  // until end_launches has seen the flag
+    return SSD_OK;
+}
+
+// Enqueues the read of the error flag; the caller synchronises and then calls
+// end_launches.
+int read_error(ssd_handle* h) {
+    CUDA_TRY(cudaMemcpyAsync(h->emitted_host + 1, &h->st->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream),
+             "error flag");
+    return SSD_OK;
+}
+int end_launches(ssd_handle* h) {
+    const int e = h->emitted_host[1];
+    if (e == kDevErrTimeout) return fail(SSD_ERR_TIMEOUT, "a wait of the forward kernel timed out");
+    if (e) return fail(SSD_ERR_CUDA, "device check failed with code " + std::to_string(e));
+    h->clean = true;
     return SSD_OK;
 }
 
@@ -743,7 +774,7 @@ int ssd_create(const ssd_config* cfg, const ssd_weights* w, void* cuda_stream, s
         (rc = dalloc(h, &h->counters, (size_t)4, &B)) ||
         (rc = dalloc(h, &h->attn_part, (size_t)c.n_kv_heads * h->n_chunks * G * kMaxRows * attn_part_floats((int)HD), &B)) ||
         (rc = dalloc(h, &h->rope, (size_t)c.max_seq * (HD / 2), &B)) ||
-        (rc = dalloc(h, &h->tok, (size_t)c.max_seq + kMaxRows, &B)) ||
+        (rc = dalloc(h, &h->tok, (size_t)c.max_seq, &B)) ||
         (rc = dalloc(h, &h->out, (size_t)c.max_seq, &B)) || (rc = dalloc(h, &h->argbuf, 32, &B)) ||
         (rc = dalloc(h, &h->st, 1, &B)) || (rc = dalloc(h, &h->bar, 4, &B)))
         return bail(rc);
@@ -873,12 +904,7 @@ int ssd_prefill(ssd_handle* h, const int32_t* prompt, int n_prompt) {
         if (prompt[i] < 0 || prompt[i] >= h->cfg.vocab) return fail(SSD_ERR_INVALID_ARG, "prompt token out of range");
     CUDA_TRY(cudaSetDevice(h->device), "set device");
     h->prefilled = false;
-    CUDA_TRY(cudaMemsetAsync(&h->st->err, 0, sizeof(int), h->stream), "error flag reset");
-    // the acceptance kernels' arrival counter is left at zero by every
-    // completed launch; after a failed one it may not be, so a new prompt
-    // starts from clean counters
-    CUDA_TRY(cudaMemsetAsync(h->counters, 0, 4 * sizeof(unsigned), h->stream),
-             "counter reset");
+    if (int rc = begin_launches(h)) return rc;
     if (n_prompt > 1)
         CUDA_TRY(cudaMemcpyAsync(h->tok, prompt, sizeof(int) * (n_prompt - 1), cudaMemcpyHostToDevice, h->stream),
                  "prompt upload");
@@ -893,23 +919,13 @@ int ssd_prefill(ssd_handle* h, const int32_t* prompt, int n_prompt) {
     } else {
         for (int p0 = 0; p0 < n_prompt - 1; p0 += kMaxRows) {
             int M = std::min(kMaxRows, n_prompt - 1 - p0);
-            int rc = forward(h, M, SRC_TOKENS, h->tok + p0, p0, false, false);
+            int rc = forward(h, M, SRC_TOKENS, prompt + p0, p0, false, false);
             if (rc) return rc;
         }
     }
+    if (int rc = read_error(h)) return rc;
     CUDA_TRY(cudaStreamSynchronize(h->stream), "prefill");
-    {
-        int derr = 0;
-        CUDA_TRY(cudaMemcpy(&derr, &h->st->err, sizeof(int), cudaMemcpyDeviceToHost), "error flag");
-        if (derr == kDevErrTimeout) return fail(SSD_ERR_TIMEOUT, "a wait of the forward kernel timed out");
-    }
-#ifdef SSD_CHECKED
-    {
-        int derr = 0;
-        CUDA_TRY(cudaMemcpy(&derr, &h->st->err, sizeof(int), cudaMemcpyDeviceToHost), "error flag");
-        if (derr) return fail(SSD_ERR_CUDA, "device check failed with code " + std::to_string(derr));
-    }
-#endif
+    if (int rc = end_launches(h)) return rc;
     h->prefilled = true;
     h->n_prompt = n_prompt;
     h->last_prompt_token = prompt[n_prompt - 1];
@@ -949,6 +965,7 @@ int ssd_generate(ssd_handle* h, const int32_t* prompt, int n_prompt, int n_new, 
     init->beta1 = h->beta1;
     init->beta2 = h->beta2;
     CUDA_TRY(cudaMemcpyAsync(h->st, init, sizeof(DecodeState), cudaMemcpyHostToDevice, h->stream), "state upload");
+    if (int rc = begin_launches(h)) return rc;
 
     // graphs needed by this call (captured once, replayed every round)
     cudaGraphExec_t g_draft = nullptr;
@@ -994,13 +1011,12 @@ int ssd_generate(ssd_handle* h, const int32_t* prompt, int n_prompt, int n_new, 
         launches += (long long)Kd * draft_launches + verify_launches;
         CUDA_TRY(cudaGraphLaunch(g_verify, h->stream), "verification step");
         CUDA_TRY(cudaEventRecord(ev[2], h->stream), "event");
-        CUDA_TRY(cudaMemcpyAsync(h->emitted_host, &h->st->emitted, sizeof(int), cudaMemcpyDeviceToHost, h->stream),
-                 "state read");
-        CUDA_TRY(cudaMemcpyAsync(h->emitted_host + 1, &h->st->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream),
+        static_assert(offsetof(DecodeState, err) == offsetof(DecodeState, emitted) + sizeof(int), "read together");
+        CUDA_TRY(cudaMemcpyAsync(h->emitted_host, &h->st->emitted, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream),
                  "state read");
         CUDA_TRY(cudaStreamSynchronize(h->stream), "round");
-        if (h->emitted_host[1] == kDevErrTimeout)
-            return fail(SSD_ERR_TIMEOUT, "a grid barrier of the forward kernel timed out");
+        if (int rc = end_launches(h)) return rc;
+        h->clean = false;  // (another round, or the end below)
         const int e = *h->emitted_host;
         if (e <= emitted || e > n_new) return fail(SSD_ERR_CUDA, "decode state corrupted");
         emitted = e;
@@ -1010,6 +1026,7 @@ int ssd_generate(ssd_handle* h, const int32_t* prompt, int n_prompt, int n_new, 
     CUDA_TRY(cudaMemcpyAsync(out_tokens, h->out, sizeof(int) * n_new, cudaMemcpyDeviceToHost, h->stream), "tokens");
     CUDA_TRY(cudaMemcpyAsync(h->st_host, h->st, sizeof(DecodeState), cudaMemcpyDeviceToHost, h->stream), "stats");
     CUDA_TRY(cudaStreamSynchronize(h->stream), "generate");
+    h->clean = true;
     if (stats) {
         const DecodeState* s = h->st_host;
         stats->rounds = s->rounds;
@@ -1044,28 +1061,22 @@ int ssd_debug_forward(ssd_handle* h, int draft, const int32_t* tokens, int n_row
     for (int i = 0; i < n_rows; ++i)
         if (tokens[i] < 0 || tokens[i] >= h->cfg.vocab) return fail(SSD_ERR_INVALID_ARG, "token out of range");
     CUDA_TRY(cudaSetDevice(h->device), "set device");
-    int* dt = h->tok + h->cfg.max_seq;
-    CUDA_TRY(cudaMemsetAsync(&h->st->err, 0, sizeof(int), h->stream), "error flag reset");
-    CUDA_TRY(cudaMemcpyAsync(dt, tokens, sizeof(int) * n_rows, cudaMemcpyHostToDevice, h->stream), "upload");
+    if (int rc = begin_launches(h)) return rc;
     const int stall = h->stall_barrier;
     const unsigned long long wait_ns = h->wait_ns;
     if (stall) {  // armed by ssd_debug_stall_barrier for this one forward
         h->wait_ns = h->stall_wait_ns;
         h->stall_barrier = 0;
     }
-    int rc = forward(h, n_rows, SRC_TOKENS, dt, pos0, draft != 0, true, nullptr, nullptr, stall);
+    int rc = forward(h, n_rows, SRC_TOKENS, tokens, pos0, draft != 0, true, nullptr, nullptr, stall);
     h->wait_ns = wait_ns;
     if (rc) return rc;
+    // (the logits last: their copy to the caller's memory may wait for the stream)
+    if ((rc = read_error(h))) return rc;
     CUDA_TRY(cudaMemcpyAsync(logits_out, h->logits, sizeof(float) * n_rows * h->cfg.vocab,
                              cudaMemcpyDeviceToHost, h->stream), "logits");
-    int derr = 0;
-    CUDA_TRY(cudaMemcpyAsync(&h->st_host->err, &h->st->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream),
-             "error flag");
     CUDA_TRY(cudaStreamSynchronize(h->stream), "debug forward");
-    derr = h->st_host->err;
-    if (derr == kDevErrTimeout) return fail(SSD_ERR_TIMEOUT, "a wait of the forward kernel timed out");
-    if (derr) return fail(SSD_ERR_CUDA, "device check failed with code " + std::to_string(derr));
-    return SSD_OK;
+    return end_launches(h);
 }
 
 int ssd_debug_stall_barrier(ssd_handle* h, int barrier, double wait_limit_s) {
@@ -1095,8 +1106,8 @@ int trace_forward(ssd_handle* h, cudaGraphExec_t exec, int n_ops, std::vector<fl
 
 int capture_debug_forward(ssd_handle* h, int draft, int rows, bool traced, cudaGraphExec_t* exec, int* n) {
     const int pos0 = h->cfg.max_seq - rows;
-    int* dt = h->tok + h->cfg.max_seq;
-    CUDA_TRY(cudaMemsetAsync(dt, 0, sizeof(int) * rows, h->stream), "tokens");
+    if (int rc = begin_launches(h)) return rc;
+    const int dt[kMaxRows] = {};
     cudaGraph_t g = nullptr;
     CUDA_TRY(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
     int rc = forward(h, rows, SRC_TOKENS, dt, pos0, draft != 0, true, n, traced ? h->trace : nullptr);

@@ -1466,18 +1466,23 @@ __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams
         // profiling hook p.stall_barrier (0: none) makes barrier number n
         // unreachable, so that its bounded wait runs out and the launch ends with
         // the timeout recorded.
+        unsigned* const bar = p.bar + (s_seq & 1u);
         unsigned target = 0;
         int n_barrier = 0;
         auto barrier_arrive = [&]() {
             target += gridDim.x;
             ++n_barrier;
-            if (threadIdx.x == 0) grid_arrive(p.bar);
+            if (threadIdx.x == 0) grid_arrive(bar);
         };
         auto barrier_wait = [&]() {  // thread 0
             const unsigned extra = n_barrier == p.stall_barrier ? 1u : 0u;
-            const bool passed = grid_wait(p.bar, target + extra, p.err, p.wait_ns);
-            // every CTA has read the sequence number before the first barrier
-            if (passed && n_barrier == 1 && blockIdx.x == 0) *p.seq = s_seq + 1u;
+            const bool passed = grid_wait(bar, target + extra, p.err, p.wait_ns);
+            // every CTA has read the sequence number before the first barrier;
+            // the other counter was the previous launch's
+            if (passed && n_barrier == 1 && blockIdx.x == 0) {
+                *p.seq = s_seq + 1u;
+                p.bar[(s_seq + 1u) & 1u] = 0u;
+            }
             return passed;
         };
         // every row's attention within the first segment: no partials to combine

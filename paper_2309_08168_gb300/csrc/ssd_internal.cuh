@@ -32,6 +32,7 @@ struct DecodeState {
     int x_last;     // last emitted token; sits at position len
     int j;          // drafts produced in the current round
     int emitted;    // tokens written to the output buffer by this generate call
+    int err;        // device-side error code (0 = none); read by the host together with emitted
     int rounds, drafted, accepted;
     int hist[33];
     int drafts[kMaxK + 1];
@@ -40,7 +41,6 @@ struct DecodeState {
     float inv_temperature;
     float top_p;
     unsigned long long seed;
-    int err;        // device-side error code (0 = none)
     // adaptive draft exit (Sec. 3.4, Eqs. 2-4); exit_on = 0: off
     int exit_on;
     int exited;     // the current round's drafting stage has ended
@@ -132,7 +132,7 @@ struct FwdParams {
     int n_ops;
     int M;                // rows of this forward (1..16)
     int src;              // EmbedSrc: where the tokens and the first position come from
-    const int* toks;      // SRC_TOKENS: device token ids
+    int toks[kMaxRows];   // SRC_TOKENS: token ids
     int pos0_arg;         // SRC_TOKENS: first position
     DecodeState* st;
     const bf16* embed;
@@ -142,7 +142,8 @@ struct FwdParams {
     bf16* xn_hi;          // planes of h * g [16][d]
     bf16* xn_lo;
     float* ss;            // per-128-column sums of h^2 [16][d/128]
-    unsigned* bar;        // grid-barrier counter, zero at launch
+    unsigned* bar;        // [2] grid-barrier counters: launch number seq counts on bar[seq & 1], zero at
+                          // launch, and zeroes the other one for the next launch
     unsigned* seq;        // forward sequence number (tags split-K partials; +1 per launch)
     int* err;             // device error code
     // Profiling hook: nullptr, or globaltimer stamps: [0, n_ops] start, end of
