@@ -980,12 +980,31 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
     auto stamp = [&](int it, int k) {
         if (ut && tid == 0 && it - ar.i_begin < 31) ut[(it - ar.i_begin) * 8 + k] = globaltimer();
     };
+    // (KV head, vector group, segment) of the item, stepped along: the divisions
+    // by run-time values are made once per op and vector group, not per item
+    int hv = ar.i_begin / ar.n_seg, sg = ar.i_begin - hv * ar.n_seg - 1;
+    int kvh = hv / ar.n_vg, vg = hv - kvh * ar.n_vg;
+    int vg_rows = -1;  // the vector group whose rows are in mrow
+    int mrow[2][2];    // input row of vector 8 nt + 2 tg + cx
     for (int it = ar.i_begin; it < ar.i_end; ++it) {
         stamp(it, 0);
-        const int hv = it / ar.n_seg, sg = it - hv * ar.n_seg, t0 = sg * SP;
-        const int kvh = hv / ar.n_vg, vg = hv - kvh * ar.n_vg;
+        if (++sg == ar.n_seg) {
+            sg = 0;
+            if (++vg == ar.n_vg) {
+                vg = 0;
+                ++kvh;
+            }
+        }
+        const int t0 = sg * SP;
         const int n_u = min(SC, ar.n_ch - sg * SC);  // chunks of this segment
         const int v0 = vg * VG, nv = min(VG, NV - v0);
+        if (vg != vg_rows) {
+            vg_rows = vg;
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                for (int cx = 0; cx < 2; ++cx) mrow[nt][cx] = (v0 + nt * 8 + 2 * tg + cx) / G;
+        }
         float* part = a.part + ((size_t)kvh * a.n_chunks + sg) * NV * part_v;
         // q of this item's vectors as fp16 hi + lo (other CTAs wrote q: L2);
         // every thread issues all its 16-byte loads before converting, and the
@@ -1079,8 +1098,7 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
                     const int vl = nt * 8 + 2 * tg + (x & 1), pq = p0 + g + 8 * (x >> 1);
-                    const int m = (v0 + vl) / G;
-                    const bool vis = j < n_u && vl < nv && t0 + pq <= pos0 + m;
+                    const bool vis = j < n_u && vl < nv && t0 + pq <= pos0 + mrow[nt][x & 1];
                     c[nt][x] = vis ? c[nt][x] * a.scale : -INFINITY;
                 }
 #pragma unroll
