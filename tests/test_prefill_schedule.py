@@ -38,11 +38,11 @@ int main(int argc, char** argv) {
         a.n_kb = (K + kBK - 1) / kBK;
         tc_plan(a, n_ft, P, K);
         const TcSched& s = a.sched;
-        if (a.nt % 32 || a.nt < 32 || a.nt > kMaxTok || a.n_tt * a.nt < a.rows || (a.n_tt - 1) * a.nt >= a.rows)
+        if (a.nt % 32 || a.nt < 32 || a.nt > kMaxTok || s.n_tt * a.nt < a.rows || (s.n_tt - 1) * a.nt >= a.rows)
             return bad("token tiles", a, n_ft);
         if (a.stages < 4 || a.stages > kMaxStages || a.stages * (kATile + a.nt * 128) > kRingBytes)
             return bad("ring", a, n_ft);
-        if (s.n_tiles != n_ft * a.n_tt || s.pairs < 1 || s.pairs > P || s.split_pairs > P) return bad("grid", a, n_ft);
+        if (s.n_tiles != n_ft * s.n_tt || s.pairs < 1 || s.pairs > P || s.split_pairs > P) return bad("grid", a, n_ft);
         if ((long)s.n_tiles * a.n_kb > 200000) continue;
         std::vector<char> seen((size_t)s.n_tiles * a.n_kb, 0);
         std::vector<int> partial_of(s.pairs, -1), fin(s.n_tiles, -1), contrib(s.n_tiles, 0);
