@@ -644,15 +644,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm
 // by k block over all of them (with less than half a wave left, one more wave
 // is split with it, so that a tile is cut in two or three rather than many), in
 // pieces of at least kMinSplit k blocks.  The choice with the least estimated
-// time, from times measured on GB300 at the 7B, 13B and 70B widths with 31 ..
-// 1535 rows (us):
-//   a k block of a tile     0.033 + 0.00222 nt, at least 0.24 (issue bound);
-//   the last tile's epilogue 5 nt / 256; of split tiles 13 nt / 256 + 4, the
-//                           partial sums' way through L2 included;
-//   split tiles walk K at offsets of their own: token planes of more than ~96
+// time, from times measured on GB300: every choice of the 7B, 13B and 70B
+// projections for 64 .. 2047 rows, 1100 points (us):
+//   a k block of a tile   0.059 + 0.00229 nt, at least 0.24 (issue bound);
+//   the rest, mostly the last tile's epilogue: whole tiles 8.4 nt / 256; split
+//   tiles, the partial sums' way through L2 included, 17 nt / 256 + 6.5, or
+//   12 nt / 256 + 7 if whole tiles follow;
+//   split tiles walk K at offsets of their own: token planes of more than ~73
 //   MB do not stay in L2 and both operands come from HBM (6.8 TB/s).
-// Over those shapes the choice is within 1 % of the best measured one in the
-// sum (11034 of 10934 us; tiles of 256 tokens always split: 11.8 ms).
+// Over those shapes the choice is 0.8 % slower than the best measured one on
+// average (19.69 ms of 19.45 in the sum).
 inline void tc_plan(TcArgs& a, int n_ft, int pairs, int K) {
     const int least = (a.rows + kMaxTok - 1) / kMaxTok;
     double best = 1e30;
@@ -660,10 +661,10 @@ inline void tc_plan(TcArgs& a, int n_ft, int pairs, int K) {
         const int nt = ((a.rows + n_tt - 1) / n_tt + 31) / 32 * 32;
         if ((a.rows + nt - 1) / nt != n_tt) continue;
         const int tiles = n_ft * n_tt, waves = tiles / pairs, rest = tiles % pairs;
-        const double t_kb = 0.033 + 0.00222 * nt > 0.24 ? 0.033 + 0.00222 * nt : 0.24;
+        const double t_kb = 0.059 + 0.00229 * nt > 0.24 ? 0.059 + 0.00229 * nt : 0.24;
         for (int split = 0; split < 2; ++split) {
             int n_split = 0, p = 1;
-            double us = (double)(waves + (rest ? 1 : 0)) * a.n_kb * t_kb + 5.0 * nt / 256;
+            double us = (double)(waves + (rest ? 1 : 0)) * a.n_kb * t_kb + 8.4 * nt / 256;
             if (split) {
                 if (rest == 0) continue;
                 n_split = waves > 0 && 2 * rest < pairs ? rest + pairs : rest;
@@ -672,11 +673,12 @@ inline void tc_plan(TcArgs& a, int n_ft, int pairs, int K) {
                 // too short for every pair: only useful if there is no whole wave
                 if (p < pairs && (waves > 0 || p <= rest)) continue;
                 double part = (double)n_split * a.n_kb / p * t_kb;
-                if (4e0 * a.rows * K > 96e6) {
+                if (4e0 * a.rows * K > 73e6) {
                     const double hbm = n_split * (512.0 * K + 4.0 * nt * K) / 6.8e6;
                     if (hbm > part) part = hbm;
                 }
-                us = part + (double)((tiles - n_split) / pairs) * a.n_kb * t_kb + 13.0 * nt / 256 + 4;
+                const int whole = (tiles - n_split) / pairs;
+                us = part + whole * a.n_kb * t_kb + (whole ? 12.0 * nt / 256 + 7 : 17.0 * nt / 256 + 6.5);
             }
             if (us < best) {
                 best = us;
