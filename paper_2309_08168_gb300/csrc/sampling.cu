@@ -129,12 +129,18 @@ __device__ int block_argmax(const float* x, int V, float* redf, int* redi) {
 // >= top_p of the mass, renormalised.  s: shared row; thread t owns the
 // contiguous segment [t*seg, t*seg + seg) and keeps it in registers.  tau* is
 // found exactly by bisection over the fp32 bit patterns of pi (non-negative
-// floats order like their bits), at most 30 passes of one threshold: the row is
-// a CTA's, so a pass costs its instructions (two per element), and 15 thresholds
-// in each of 8 passes cost four times as many.  (Vocabulary 32000, top-p 0.95,
-// the whole sampling draft kernel: 302 us with both, the row in
-// shared memory without padding, 49 us now.)
+// floats order like their bits).  The row is a CTA's, so a pass over it costs its
+// instructions (two per element): one threshold at a time (15 in each of 8 passes
+// cost four times as many), until the bracket is 2^20 patterns wide (1/8 octave,
+// 10 passes).  The values inside it, 2-3 % of a flat row, are then listed in
+// the row's shared memory, and the other 20 bits take 10 passes of three
+// thresholds over the list.
+// (Vocabulary 32000, top-p 0.95, the whole sampling draft kernel: 302 us with 15
+// thresholds a pass and the row in shared memory without padding, 48.7 with 30
+// one-threshold passes over registers, 44.9 now.)
 // ---------------------------------------------------------------------------
+constexpr uint32_t kBracket = 1u << 20;
+
 __device__ void nucleus_row(const float* logits, int V, float inv_t, float top_p, float* s,
                             float* red) {
     const int seg = (V + kRowThreads - 1) / kRowThreads;
@@ -163,11 +169,14 @@ __device__ void nucleus_row(const float* logits, int V, float inv_t, float top_p
         pmax = fmaxf(pmax, r[k]);
     }
     if (top_p < 1.f) {
-        __shared__ float wsum[2][kRowThreads / 32];
+        __shared__ float wsum[2][3][32];
+        __shared__ int first[33];
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        // invariant: f(lo) >= top_p > f(hi), f(t) = mass of the values >= t
+        // invariant: f(lo) >= top_p > f(hi), f(t) = mass of the values >= t; f(hi) = above
         uint32_t lo = 0u, hi = __float_as_uint(block_max(pmax, red)) + 1u;
-        for (int it = 0; hi - lo > 1u; ++it) {
+        float above = 0.f;
+        int it = 0;  // (two buffers: a warp is at most one pass ahead of another's reads)
+        for (; hi - lo > kBracket; ++it) {
             const uint32_t mid = lo + ((hi - lo) >> 1);
             const float t = __uint_as_float(mid);
             float part = 0.f;
@@ -175,14 +184,69 @@ __device__ void nucleus_row(const float* logits, int V, float inv_t, float top_p
             for (int k = 0; k < kSegMax; ++k)
                 if (r[k] >= t) part += r[k];
             part = warp_sum(part);
-            if (lane == 0) wsum[it & 1][warp] = part;
+            if (lane == 0) wsum[it & 1][0][warp] = part;
             __syncthreads();
-            // (two buffers: a warp is at most one pass ahead of another's reads)
-            float tot = 0.f;
-#pragma unroll
-            for (int w = 0; w < kRowThreads / 32; ++w) tot += wsum[it & 1][w];
+            const float tot = warp_sum(wsum[it & 1][0][lane]);
             if (tot >= top_p) lo = mid;
-            else hi = mid;
+            else { hi = mid; above = tot; }
+        }
+        if (hi - lo > 1u) {  // (uniform)
+            const float from = __uint_as_float(lo), to = __uint_as_float(hi);
+            int mine = 0;
+#pragma unroll
+            for (int k = 0; k < kSegMax; ++k) mine += r[k] >= from && r[k] < to;
+            int incl = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            if (lane == 31) first[warp] = incl;
+            __syncthreads();
+            if (warp == 0) {
+                const int c = first[lane];
+                int in2 = c;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, in2, o);
+                    if (lane >= o) in2 += y;
+                }
+                first[lane] = in2 - c;
+                if (lane == 31) first[32] = in2;
+            }
+            __syncthreads();
+            int at = first[warp] + incl - mine;
+#pragma unroll
+            for (int k = 0; k < kSegMax; ++k)
+                if (r[k] >= from && r[k] < to) s[at++] = r[k];
+            __syncthreads();
+            const int n_list = first[32];
+            for (; hi - lo > 1u; ++it) {
+                uint32_t m[3];
+                float part[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+                for (int j = 0; j < 3; ++j) m[j] = lo + max(1u, (uint32_t)(j + 1) * (hi - lo) >> 2);
+                for (int i = threadIdx.x; i < n_list; i += kRowThreads) {
+                    const float v = s[i];
+#pragma unroll
+                    for (int j = 0; j < 3; ++j)
+                        if (v >= __uint_as_float(m[j])) part[j] += v;
+                }
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    part[j] = warp_sum(part[j]);
+                    if (lane == 0) wsum[it & 1][j][warp] = part[j];
+                }
+                __syncthreads();
+                bool in[3];
+#pragma unroll
+                for (int j = 0; j < 3; ++j) in[j] = above + warp_sum(wsum[it & 1][j][lane]) >= top_p;
+                if (in[2]) lo = m[2];
+                else if (in[1]) { lo = m[1]; hi = m[2]; }
+                else if (in[0]) { lo = m[0]; hi = m[1]; }
+                else hi = m[0];
+            }
+            __syncthreads();  // the list has been read
         }
         // kept mass (deterministic recount) and renormalisation
         const float tau = __uint_as_float(lo);
