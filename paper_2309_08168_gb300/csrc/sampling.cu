@@ -127,19 +127,24 @@ __device__ int block_argmax(const float* x, int V, float* redf, int* redi) {
 // sampling distribution of one row: softmax(logits / T) restricted to the
 // nucleus {x : pi(x) >= tau*}, tau* = the largest value whose upper set holds
 // >= top_p of the mass, renormalised.  s: shared row; thread t owns the
-// contiguous segment [t*seg, t*seg + seg) and keeps it in registers.  tau* is
-// found exactly by bisection over the fp32 bit patterns of pi (non-negative
-// floats order like their bits).  The row is a CTA's, so a pass over it costs its
-// instructions (two per element): one threshold at a time (15 in each of 8 passes
-// cost four times as many), until the bracket is 2^20 patterns wide (1/8 octave,
-// 10 passes).  The values inside it, 2-3 % of a flat row, are then listed in
-// the row's shared memory, and the other 20 bits take 10 passes of three
-// thresholds over the list.
+// contiguous segment [t*seg, t*seg + seg) and keeps exp(x - max) in registers;
+// the search runs on these values (tau* and the mass scaled by their sum z), so
+// that a kept value is divided once.  tau* is found exactly by bisection over the
+// fp32 bit patterns (non-negative floats order like their bits), from below
+// (1 - top_p) z / 2V, where at most half of 1 - top_p is cut off.  The row is a
+// CTA's, so a pass over it costs its instructions (two per element): one
+// threshold at a time, until the bracket is 2^20 patterns wide (1/8 octave, 7
+// passes at top_p 0.95).  The values inside it, 2-3 % of a flat row, are then
+// listed in the row's shared memory, and the other 20 bits take 10 passes of
+// three thresholds over the list, by one warp if it is short (with 32 warps
+// such a pass is 960 shuffles, 0.8 us; with one 0.2 us).
 // (Vocabulary 32000, top-p 0.95, the whole sampling draft kernel: 302 us with 15
 // thresholds a pass and the row in shared memory without padding, 48.7 with 30
-// one-threshold passes over registers, 44.9 now.)
+// one-threshold passes over registers, 44.9 with the list, all warps and two
+// divisions, 33.1 now; a row of the acceptance kernel 58.8, 53.7, 41.1.)
 // ---------------------------------------------------------------------------
 constexpr uint32_t kBracket = 1u << 20;
+constexpr int kShortList = 1024;
 
 __device__ void nucleus_row(const float* logits, int V, float inv_t, float top_p, float* s,
                             float* red) {
@@ -162,18 +167,16 @@ __device__ void nucleus_row(const float* logits, int V, float inv_t, float top_p
         z += r[k];
     }
     z = block_sum(z, red);
-    float pmax = 0.f;
-#pragma unroll
-    for (int k = 0; k < kSegMax; ++k) {
-        r[k] = r[k] / z;
-        pmax = fmaxf(pmax, r[k]);
-    }
     if (top_p < 1.f) {
         __shared__ float wsum[2][3][32];
         __shared__ int first[33];
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        // invariant: f(lo) >= top_p > f(hi), f(t) = mass of the values >= t; f(hi) = above
-        uint32_t lo = 0u, hi = __float_as_uint(block_max(pmax, red)) + 1u;
+        // invariant: f(lo) >= top_p z > f(hi), f(t) = sum of the values >= t; f(hi) = above
+        // (the largest value is exp(0) = 1; the first lo only where rounding is far below 1 - top_p)
+        const float target = top_p * z;
+        uint32_t lo = top_p < 0.999f ? __float_as_uint((1.f - top_p) * z / (2.f * V)) : 0u;
+        uint32_t hi = __float_as_uint(1.f) + 1u;
+        if (!(z >= 1.f)) lo = 0u;  // NaN
         float above = 0.f;
         int it = 0;  // (two buffers: a warp is at most one pass ahead of another's reads)
         for (; hi - lo > kBracket; ++it) {
@@ -187,11 +190,12 @@ __device__ void nucleus_row(const float* logits, int V, float inv_t, float top_p
             if (lane == 0) wsum[it & 1][0][warp] = part;
             __syncthreads();
             const float tot = warp_sum(wsum[it & 1][0][lane]);
-            if (tot >= top_p) lo = mid;
+            if (tot >= target) lo = mid;
             else { hi = mid; above = tot; }
         }
         if (hi - lo > 1u) {  // (uniform)
-            const float from = __uint_as_float(lo), to = __uint_as_float(hi);
+            // (zeros, the padding of the last segments among them, are never listed: at most V values)
+            const float from = __uint_as_float(max(lo, 1u)), to = __uint_as_float(hi);
             int mine = 0;
 #pragma unroll
             for (int k = 0; k < kSegMax; ++k) mine += r[k] >= from && r[k] < to;
@@ -221,35 +225,41 @@ __device__ void nucleus_row(const float* logits, int V, float inv_t, float top_p
                 if (r[k] >= from && r[k] < to) s[at++] = r[k];
             __syncthreads();
             const int n_list = first[32];
-            for (; hi - lo > 1u; ++it) {
+            const bool one = n_list <= kShortList;
+            const int i0 = one ? lane : threadIdx.x, step = one ? 32 : kRowThreads;
+            for (; hi - lo > 1u && !(one && warp); ++it) {
                 uint32_t m[3];
                 float part[3] = {0.f, 0.f, 0.f};
 #pragma unroll
                 for (int j = 0; j < 3; ++j) m[j] = lo + max(1u, (uint32_t)(j + 1) * (hi - lo) >> 2);
-                for (int i = threadIdx.x; i < n_list; i += kRowThreads) {
+#pragma unroll 4
+                for (int i = i0; i < n_list; i += step) {
                     const float v = s[i];
 #pragma unroll
                     for (int j = 0; j < 3; ++j)
                         if (v >= __uint_as_float(m[j])) part[j] += v;
                 }
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    part[j] = warp_sum(part[j]);
-                    if (lane == 0) wsum[it & 1][j][warp] = part[j];
-                }
-                __syncthreads();
-                bool in[3];
+                for (int j = 0; j < 3; ++j) part[j] = warp_sum(part[j]);
+                if (!one) {
 #pragma unroll
-                for (int j = 0; j < 3; ++j) in[j] = above + warp_sum(wsum[it & 1][j][lane]) >= top_p;
-                if (in[2]) lo = m[2];
-                else if (in[1]) { lo = m[1]; hi = m[2]; }
-                else if (in[0]) { lo = m[0]; hi = m[1]; }
+                    for (int j = 0; j < 3; ++j)
+                        if (lane == 0) wsum[it & 1][j][warp] = part[j];
+                    __syncthreads();
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) part[j] = warp_sum(wsum[it & 1][j][lane]);
+                }
+                if (above + part[2] >= target) lo = m[2];
+                else if (above + part[1] >= target) { lo = m[1]; hi = m[2]; }
+                else if (above + part[0] >= target) { lo = m[0]; hi = m[1]; }
                 else hi = m[0];
             }
-            __syncthreads();  // the list has been read
+            if (threadIdx.x == 0) first[0] = (int)lo;
+            __syncthreads();  // (also: the list has been read)
+            lo = (uint32_t)first[0];
         }
-        // kept mass (deterministic recount) and renormalisation
-        const float tau = __uint_as_float(lo);
+        // kept mass (deterministic recount) and renormalisation (a NaN row keeps nothing)
+        const float tau = z >= 1.f ? __uint_as_float(lo) : z;
         float kept = 0.f;
 #pragma unroll
         for (int k = 0; k < kSegMax; ++k)
@@ -257,6 +267,9 @@ __device__ void nucleus_row(const float* logits, int V, float inv_t, float top_p
         kept = block_sum(kept, red);
 #pragma unroll
         for (int k = 0; k < kSegMax; ++k) r[k] = r[k] >= tau ? r[k] / kept : 0.f;
+    } else {
+#pragma unroll
+        for (int k = 0; k < kSegMax; ++k) r[k] = r[k] / z;
     }
 #pragma unroll
     for (int k = 0; k < kSegMax; ++k)

@@ -12,7 +12,15 @@ Stand-alone projection: activations as bf16 pairs (2^-17 per element, in the
 same bits whatever rows come with it.
 
 Sampling: with a nucleus of one token the draw is the argmax, for any
-vocabulary, so sampled and greedy sequences are equal.
+vocabulary, so sampled and greedy sequences are equal.  With any other
+nucleus a drawn token has less than top_p of the mass above it (1e-5 for the
+32-bit sums: a sum of at most 32768 values in trees of 32 + 10 additions is
+within 42 * 2^-24 = 2.5e-6, on both sides), counting as above it only tokens
+whose probability is larger by more than 32 bits can confuse (the exponent
+x / T - max has an error of 2^-23 of its size, exp and the rounding to 1 a few
+2^-24: at T = 1e4 many of 32000 probabilities are the same 32-bit number).  The
+last tenth of the nucleus is drawn from.  High temperatures put most of the row into the list that the
+threshold is searched in, top_p next to 1 takes the search down to zero.
 
 Decode: forwards around the first segment's end (position 128), where
 attention without partials takes over, and with K of one to four chunks,
@@ -136,6 +144,36 @@ def test_one_token_nucleus_is_greedy(vocab):
     sampled, st = dec.generate(None, 24, 4, mode=ssd.SSD_SAMPLE, seed=3)
     assert np.array_equal(greedy, sampled) and st["drafted"] > 0
     dec.close()
+
+
+@pytest.mark.parametrize("vocab", [3, 300, 2049, 32000])
+@pytest.mark.parametrize("temperature,top_p", [(1.0, 0.5), (1.0, 0.95), (40.0, 0.95), (1e4, 0.3), (1.0, 0.9995),
+                                               (1.0, 0.99999994), (0.02, 0.99999994)])
+def test_nucleus_cut(vocab, temperature, top_p):
+    import paper_2309_08168_gb300 as ssd
+    w = model(vocab=vocab)
+    hw = synth.host_weights(w, seed=26)
+    dw = synth.host_to_device_weights(hw)
+    torch.cuda.synchronize()
+    dec = decoder(w, dw, 64, mask=[0, 1, 0, 0])
+    prompt = synth.prompt(20, seed=8, vocab=vocab)
+    dec.set_sampling(temperature, top_p)
+    dec.prefill(prompt)
+    x = dec.debug_forward(False, prompt[-1:], len(prompt) - 1)[0].astype(np.float64) / temperature
+    dec.prefill(prompt)
+    n = 200
+    drawn = np.array([dec.generate(None, 2, 1, mode=ssd.SSD_SAMPLE, seed=100 + i)[0][0] for i in range(n)])
+    dec.close()
+    pi = np.exp(x - x.max())
+    pi /= pi.sum()
+    order = np.argsort(-pi, kind="stable")
+    above = np.empty(vocab)
+    above[order] = np.concatenate([[0.0], np.cumsum(pi[order])[:-1]])
+    p_min = pi[drawn].min() * (1 + (4 + np.abs(x).max()) * 2.0 ** -22)
+    assert pi[pi > p_min].sum() < top_p + 1e-5
+    last = (above >= 0.9 * top_p) & (above < top_p)
+    if pi[last].sum() >= 0.05 * top_p:  # missed by 200 draws: 0.95 ** 200 = 4e-5
+        assert (above[drawn] >= 0.9 * top_p).any()
 
 
 @pytest.mark.parametrize("d,heads,hd,ffn", [(128, 2, 64, 64), (256, 2, 128, 384), (384, 6, 64, 400), (512, 4, 128, 528)])
