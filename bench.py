@@ -267,7 +267,7 @@ def draft_launches(w, mask):
 # bytes streamed, so a full launch is scaled by this ratio).  It belongs to
 # the kernel version it was captured on: None after a kernel change until
 # re-captured.
-DRAFT_TRAFFIC_RATIO = 1.0013  # 1-layer model at LLaMA-2-70B widths, current kernel
+DRAFT_TRAFFIC_RATIO = 1.0017  # 1-layer model at LLaMA-2-70B widths, current kernel
 
 
 # the paper's draft-exit hyperparameters (App. B, tab. Hyper): gamma0, alpha,
