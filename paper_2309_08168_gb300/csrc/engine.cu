@@ -424,6 +424,7 @@ std::vector<FwdOp> build_ops(ssd_handle* h, bool draft) {
             t.out_hi = h->at_hi; t.out_lo = h->at_lo;
             t.part = h->attn_part;
             t.n_heads = c.n_heads; t.n_kv_heads = c.n_kv_heads; t.head_dim = c.head_dim;
+            t.group = c.n_heads / c.n_kv_heads; t.group_inv = attn_group_inv(t.group);
             t.max_seq = c.max_seq; t.n_chunks = h->n_chunks;
             t.scale = 1.0f / std::sqrt((float)c.head_dim); t.st = h->st; t.err = &h->st->err;
             ops.push_back(at);

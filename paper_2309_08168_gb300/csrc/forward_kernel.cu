@@ -851,6 +851,11 @@ __device__ __forceinline__ void store_pair(bf16* hi_at, bf16* lo_at, float v0, f
     *reinterpret_cast<__nv_bfloat162*>(lo_at) = lo;
 }
 
+template <int N>
+struct Int {
+    static constexpr int value = N;
+};
+
 // ---------------------------------------------------------------------------
 // attention op: items (KV head, vector group, 128-position segment), through
 // the TMA ring
@@ -875,10 +880,14 @@ __device__ __forceinline__ AttnRange attn_range(const AttnArgs& a, int M, int po
     AttnRange r;
     r.n_ch = (pos0 + M + kAttnChunk - 1) / kAttnChunk;  // chunks holding any visible position
     r.n_seg = (r.n_ch + S - 1) / S;
-    r.n_vg = (a.n_heads / a.n_kv_heads * M + 15) / 16;
-    const long long I = (long long)a.n_kv_heads * r.n_seg * r.n_vg, GR = gridDim.x;
-    r.i_begin = (int)((long long)blockIdx.x * I / GR);
-    r.i_end = (int)((long long)(blockIdx.x + 1) * I / GR);
+    r.n_vg = (a.group * M + 15) / 16;
+    // One 32-bit division: this is on the way to the first item, which began 0.9 us
+    // after the op with two 64-bit ones and a division per vector, 0.5 us now (with
+    // the combine's share worked out before its barrier and the empty half of the
+    // vectors left out, 7B widths, one row: 10.82 -> 10.18 us per layer).
+    const int I = a.n_kv_heads * r.n_seg * r.n_vg, GR = gridDim.x, b = blockIdx.x, n = I / GR, more = I - n * GR;
+    r.i_begin = b * n + min(b, more);
+    r.i_end = r.i_begin + n + (b < more);
     return r;
 }
 
@@ -954,7 +963,7 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
     using L = GemmSmem<R>;
     constexpr int S = L::S, VG = L::VG, SC = kAttnSegChunks, SP = SC * kAttnChunk;  // positions per segment
     static_assert(SC <= S, "a segment's chunks are held in the ring at once");
-    const int G = a.n_heads / a.n_kv_heads, NV = G * M;
+    const int G = a.group, NV = G * M;
     const AttnRange ar = attn_range(a, M, pos0);
 
     constexpr int QST = L::QST, PST = L::PST;
@@ -1003,7 +1012,7 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
 #pragma unroll
             for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-                for (int cx = 0; cx < 2; ++cx) mrow[nt][cx] = (v0 + nt * 8 + 2 * tg + cx) / G;
+                for (int cx = 0; cx < 2; ++cx) mrow[nt][cx] = a.row_of(v0 + nt * 8 + 2 * tg + cx);
         }
         float* part = a.part + ((size_t)kvh * a.n_chunks + sg) * NV * part_v;
         // q of this item's vectors as fp16 hi + lo (other CTAs wrote q: L2);
@@ -1020,7 +1029,7 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
                 const int k4 = tid + j * kConsumers, vl = k4 / HD4, e = (k4 - vl * HD4) * 4;
                 qv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (vl < nv) {
-                    const int v = v0 + vl, m = v / G, gi = v - m * G;
+                    const int v = v0 + vl, m = a.row_of(v), gi = v - m * G;
                     qv[j] = __ldcg(reinterpret_cast<const float4*>(a.q + (size_t)m * a.n_heads * HD +
                                                                    (size_t)(kvh * G + gi) * HD + e));
                 }
@@ -1063,13 +1072,16 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
         // sums (the partial's sum adds the 8 warps' sums in order)
         float* wmax = sc;           // [8 warps][VG vectors]
         float* wsum = sc + 8 * VG;  // [8 warps][VG vectors]
-        {
+        // nt_c: 8-vector halves of the tile in use (compiled for each: with the second
+        // half skipped by branches, 13 rows took 20.7 us per layer instead of 20.0)
+        auto weights = [&](auto nt_c) {
+            constexpr int NT = decltype(nt_c)::value;
             const int p0 = warp * 16, j = p0 / kAttnChunk;
-            float c[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+            float c[NT][4] = {};
             if (j < n_u) {
                 // K q_hi and K q_lo in separate accumulators (two short
                 // dependency chains instead of one long one), added at the end
-                float cl[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+                float cl[NT][4] = {};
                 const unsigned char* kst = j ? stage[1] : stage[0];
                 const int t = (p0 % kAttnChunk) + (lane & 7) + 8 * ((lane >> 3) & 1);
                 const int qv = (lane & 7) + 8 * (lane >> 4), qk = ((lane >> 3) & 1) * 8;
@@ -1082,19 +1094,19 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
                     ldsm_x4(bl, ql + qv * QST + ks * 16 + qk);
                     mma_f16_16816(c[0], af[0], af[1], af[2], af[3], bh[0], bh[1]);
                     mma_f16_16816(cl[0], af[0], af[1], af[2], af[3], bl[0], bl[1]);
-                    if (nv > 8) {  // vectors 8..15
+                    if constexpr (NT == 2) {  // vectors 8..15
                         mma_f16_16816(c[1], af[0], af[1], af[2], af[3], bh[2], bh[3]);
                         mma_f16_16816(cl[1], af[0], af[1], af[2], af[3], bl[2], bl[3]);
                     }
                 }
 #pragma unroll
-                for (int nt = 0; nt < 2; ++nt)
+                for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
                     for (int x = 0; x < 4; ++x) c[nt][x] += cl[nt][x];
             }
             // C: rows = positions p0 + g (+8), columns = vectors 8 nt + 2 tg (+1)
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
+            for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
                     const int vl = nt * 8 + 2 * tg + (x & 1), pq = p0 + g + 8 * (x >> 1);
@@ -1102,7 +1114,7 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
                     c[nt][x] = vis ? c[nt][x] * a.scale : -INFINITY;
                 }
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
+            for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
                 for (int cx = 0; cx < 2; ++cx) {
                     float v = fmaxf(c[nt][cx], c[nt][cx + 2]);
@@ -1114,7 +1126,7 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
             consumer_sync();
             stamp(it, 4);
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt)
+            for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
                 for (int cx = 0; cx < 2; ++cx) {
                     const int vl = nt * 8 + 2 * tg + cx;
@@ -1137,12 +1149,14 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
                     l += __shfl_xor_sync(0xffffffffu, l, 16);
                     if (g == 0) wsum[warp * VG + vl] = l;
                 }
-        }
+        };
+        if (nv > 8) weights(Int<2>{});
+        else weights(Int<1>{});
         consumer_sync();
         stamp(it, 5);
         // the segment's (max, sum) of each vector; -inf: nothing visible
         if (tid < nv && ar.n_seg > 1) {
-            const int v = v0 + tid, m = v / G;
+            const int v = v0 + tid, m = a.row_of(v);
             float mx = -INFINITY, l = 0.f;
 #pragma unroll
             for (int w2 = 0; w2 < kConsumers / 32; ++w2) {
@@ -1196,7 +1210,7 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
 #pragma unroll
                     for (int w2 = 0; w2 < kConsumers / 32; ++w2) l += wsum[w2 * VG + vl];
                     const float inv = 1.f / l;
-                    const int v = v0 + vl, m = v / G, gi = v - m * G;
+                    const int v = v0 + vl, m = a.row_of(v), gi = v - m * G;
                     const size_t at = (size_t)m * a.n_heads * HD + (size_t)(kvh * G + gi) * HD + warp * 16 + 2 * tg;
 #pragma unroll
                     for (int nt = 0; nt < 2; ++nt)
@@ -1238,25 +1252,41 @@ __device__ bool attn_consume(const AttnArgs& a, int M, int pos0, unsigned char* 
 // maximum and the sum of the weighted sums are shuffle trees, the weighted
 // dims are added in segment order, and batches fold into running sums scaled
 // to the running maximum.  The order depends only on the row's position.
+// A warp's first share is worked out before the barrier (combine_item).
 constexpr int kCombineBatch = 16;
+struct CombineItem {
+    const float* pv;  // the vector's partial of segment 0
+    size_t at;        // output element
+    int nsg;          // segments of its row
+};
 template <int HD>
-__device__ void attn_combine(const AttnArgs& a, int M, int pos0) {
-    constexpr int SP = kAttnSegChunks * kAttnChunk, HALVES = HD / 64, B = kCombineBatch;
-    static_assert(B <= 32, "one lane per segment of a batch");
-    const int G = a.n_heads / a.n_kv_heads, NV = G * M;
+__device__ __forceinline__ CombineItem combine_item(const AttnArgs& a, int M, int pos0, int wk) {
+    constexpr int SP = kAttnSegChunks * kAttnChunk, HALVES = HD / 64;
     constexpr size_t part_v = attn_part_floats(HD);  // floats per partial: o[HD], max, sum, pad
-    const size_t qs_stride = (size_t)NV * part_v;    // next segment of the same vector
-    const int n_work = a.n_kv_heads * NV * HALVES;   // (vector, 64 dims) per warp
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int G = a.group, NV = G * M;
+    const int gv = wk / HALVES, kvh = gv / NV, v = gv - kvh * NV;
+    const int m = a.row_of(v), gi = v - m * G;
+    CombineItem c;
+    c.pv = a.part + ((size_t)kvh * a.n_chunks * NV + v) * part_v;
+    c.at = (size_t)m * a.n_heads * HD + (size_t)(kvh * G + gi) * HD + (wk & (HALVES - 1)) * 64 + 2 * (threadIdx.x & 31);
+    c.nsg = (pos0 + m) / SP + 1;
+    return c;
+}
+// warp-major over the CTAs: the first work items go to warp 0 of every CTA
+__device__ __forceinline__ int combine_first() { return (threadIdx.x >> 5) * gridDim.x + blockIdx.x; }
+
+template <int HD>
+__device__ void attn_combine(const AttnArgs& a, int M, int pos0, CombineItem c) {
+    constexpr int HALVES = HD / 64, B = kCombineBatch;
+    static_assert(B <= 32, "one lane per segment of a batch");
+    static_assert(HALVES == 1 || HALVES == 2, "the half is the work item's lowest bit");
+    const size_t qs_stride = (size_t)a.group * M * attn_part_floats(HD);  // next segment of the same vector
+    const int n_work = a.n_kv_heads * a.group * M * HALVES;               // (vector, 64 dims) per warp
+    const int lane = threadIdx.x & 31;
     const int n_warps = gridDim.x * (kConsumers / 32);
-    // warp-major over the CTAs: the first work items go to warp 0 of every CTA
-    for (int wk = warp * gridDim.x + blockIdx.x; wk < n_work; wk += n_warps) {
-        const int gv = wk / HALVES, hf = wk - gv * HALVES;
-        const int kvh = gv / NV, v = gv - kvh * NV;
-        const int e = hf * 64 + 2 * lane;
-        const int m = v / G, gi = v - m * G;
-        const int nsg = (pos0 + m) / SP + 1;
-        const float* pv = a.part + (size_t)kvh * a.n_chunks * qs_stride + (size_t)v * part_v;
+    for (int wk = combine_first(); wk < n_work;) {
+        const int e = (wk & (HALVES - 1)) * 64 + 2 * lane, nsg = c.nsg;
+        const float* pv = c.pv;
         float mx = -INFINITY, l = 0.f, o0 = 0.f, o1 = 0.f;
         for (int q0 = 0; q0 < nsg; q0 += B) {
             const int nb = min(B, nsg - q0);
@@ -1290,8 +1320,9 @@ __device__ void attn_combine(const AttnArgs& a, int M, int pos0) {
             mx = bm;
         }
         const float inv = 1.f / l;
-        const size_t at = (size_t)m * a.n_heads * HD + (size_t)(kvh * G + gi) * HD + e;
-        store_pair(a.out_hi + at, a.out_lo + at, o0 * inv, o1 * inv);
+        store_pair(a.out_hi + c.at, a.out_lo + c.at, o0 * inv, o1 * inv);
+        wk += n_warps;
+        if (wk < n_work) c = combine_item<HD>(a, M, pos0, wk);
     }
 }
 
@@ -1532,6 +1563,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams
                     }
                     if (ct && threadIdx.x == 0) ct[2] = globaltimer();
                     barrier_arrive();
+                    const CombineItem first = combine_item<HD>(op.at, p.M, pos0, combine_first());
                     if (threadIdx.x == 0) {
                         mbar_arrive(&left);
                         ok = barrier_wait();
@@ -1541,7 +1573,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams
                         failed = true;
                         break;
                     }
-                    attn_combine<HD>(op.at, p.M, pos0);
+                    attn_combine<HD>(op.at, p.M, pos0, first);
                 }
             }
             if (ct && threadIdx.x == 0) ct[3] = globaltimer();

@@ -109,10 +109,18 @@ struct AttnArgs {
     bf16* out_lo;
     float* part;         // segment partials [Hkv][n_chunks][G*M][attn_part_floats(hd)]: o[hd], max, sum, 2 pad
     int M, n_heads, n_kv_heads, head_dim, max_seq, n_chunks;
+    int group;           // query heads per KV head
+    unsigned group_inv;  // ceil(2^24 / group), or 0 for groups of 1024 and more (AttnArgs::row_of)
     float scale;         // 1/sqrt(hd)
     const DecodeState* st;
     int* err;            // device error flag (checked builds)
+    // input row v / group of query vector v < 16 group: the product's error, v (group_inv
+    // group - 2^24) / 2^24 < 16 group^2 / 2^24 of a group, stays below one vector
+    __host__ __device__ int row_of(int v) const {
+        return group_inv ? (int)((unsigned)v * group_inv >> 24) : v / group;
+    }
 };
+inline unsigned attn_group_inv(int group) { return group < 1024 ? ((1u << 24) + group - 1) / group : 0u; }
 
 // ---------------------------------------------------------------------------
 // forward kernel (forward_kernel.cu): one persistent cooperative launch per
