@@ -479,7 +479,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm
             const int box = 2 * ft + (int)rank;
             const int tok0 = tt * a.nt + quarter * hc;
             const int n_col = min(hc, a.rows - tok0);  // valid columns of this warp (may be <= 0)
-            ok = mb_wait(acc_full + b, (fph >> b) & 1u, a.err);
+            // (by the warp: a lane alone must not leave its tcgen05.ld, votes and shuffles)
+            ok = __all_sync(0xffffffffu, mb_wait(acc_full + b, (fph >> b) & 1u, a.err));
             fph ^= 1u << b;
             if (!ok) break;
             fence_after();
