@@ -176,8 +176,11 @@ int ssd_debug_forward(ssd_handle* h, int draft, const int32_t* tokens, int n_row
  * `barrier` (1 = the barrier after the embedding) unreachable and to give up
  * waiting after wait_limit_s seconds; that forward then returns
  * SSD_ERR_TIMEOUT, its logits are unspecified and the handle stays usable
- * (the next forward runs normally).  barrier = 0 disarms.  The hook applies
- * to that one forward only, never to ssd_generate or ssd_prefill.
+ * (the next forward runs normally).  barrier + 65536 * s with s >= 1 arms the
+ * s-th forward (drafts, then the verification) of the first round of the next
+ * ssd_generate instead: the round's forwards queued behind it do nothing (no
+ * KV row is written) and the call returns SSD_ERR_TIMEOUT.  barrier = 0
+ * disarms.  The hook applies to that one forward only, never to ssd_prefill.
  * 0 < wait_limit_s <= 10.  Errors: INVALID_ARG. */
 int ssd_debug_stall_barrier(ssd_handle* h, int barrier, double wait_limit_s);
 
@@ -201,7 +204,7 @@ int ssd_debug_spec_accept(ssd_handle* h, const float* p, const float* q, int Kd,
  * (their share of one replay, read from the forward kernel's device trace).
  * KV positions [max_seq - rows, max_seq) are overwritten: if they reach into
  * the prefilled prompt, the next ssd_generate needs a prompt again.
- * 1 <= rows <= 16, reps >= 1.  Errors: INVALID_ARG, CUDA. */
+ * 1 <= rows <= 16, reps >= 1.  Errors: INVALID_ARG, CUDA, TIMEOUT. */
 int ssd_debug_time_forward(ssd_handle* h, int draft, int rows, int gemm_only, int reps,
                            float* ms_per_forward, int* launches, double* weight_bytes);
 
@@ -224,7 +227,7 @@ int ssd_debug_time_forward(ssd_handle* h, int draft, int rows, int gemm_only, in
  * barrier arrive, [5] barrier release, [6] number of work units (items),
  * [7] release of the attention's inner grid barrier (0 for projections);
  * max_ctas >= the grid (the SM count), *n_ctas = the grid.
- * Errors: INVALID_ARG, CUDA. */
+ * Errors: INVALID_ARG, CUDA, TIMEOUT. */
 int ssd_debug_trace_forward(ssd_handle* h, int draft, int rows, float* op_us, int* op_types,
                             int max_ops, int* n_ops, int detail_op, unsigned long long* unit_trace,
                             unsigned long long* cta_trace, int max_ctas, int* n_ctas);

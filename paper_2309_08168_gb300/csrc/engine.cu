@@ -142,10 +142,11 @@ struct ssd_handle {
     PrefillPlan pf{};
     std::vector<PrefillLayer> pf_layers;
     CUtensorMap* pf_tmaps = nullptr;
-    // bounded waits of the forward kernel; test hook: one forward of
-    // ssd_debug_forward with an unreachable grid barrier (ssd_debug_stall_barrier)
+    // bounded waits of the forward kernel; test hook (ssd_debug_stall_barrier): one
+    // forward with an unreachable grid barrier, of ssd_debug_forward (stall_step 0) or
+    // the stall_step-th of the first round of ssd_generate
     unsigned long long wait_ns = 2000000000ull;
-    int stall_barrier = 0;
+    int stall_barrier = 0, stall_step = 0;
     unsigned long long stall_wait_ns = 0;
 };
 
@@ -561,18 +562,18 @@ double forward_weight_bytes(const ssd_handle* h, bool draft, bool gemm_only) {
 
 unsigned* accept_counter(ssd_handle* h) { return h->counters; }
 
-int step_launches(ssd_handle* h, int kind, int M, int mode, int* n_launch) {
+int step_launches(ssd_handle* h, int kind, int M, int mode, int* n_launch, int stall_barrier = 0) {
     const int V = h->cfg.vocab;
     int n = 0;
     if (kind == G_DRAFT) {
-        int rc = forward(h, 1, SRC_DRAFT, nullptr, 0, true, true, &n);
+        int rc = forward(h, 1, SRC_DRAFT, nullptr, 0, true, true, &n, nullptr, stall_barrier);
         if (rc) return rc;
         *n_launch = n + 1;
         if (mode == SSD_GREEDY) CUDA_TRY(launch_greedy_draft(h->logits, V, h->st, h->stream), "draft argmax");
         else CUDA_TRY(launch_sample_draft(h->logits, V, h->st, h->q_rows, h->stream), "draft sample");
         return SSD_OK;
     }
-    int rc = forward(h, M, SRC_VERIFY, nullptr, 0, false, true, &n);
+    int rc = forward(h, M, SRC_VERIFY, nullptr, 0, false, true, &n, nullptr, stall_barrier);
     if (rc) return rc;
     *n_launch = n + 1;
     if (mode == SSD_GREEDY)
@@ -976,6 +977,22 @@ int ssd_generate(ssd_handle* h, const int32_t* prompt, int n_prompt, int n_new, 
         int rc = get_graph(h, G_DRAFT, 1, mode, &g_draft, &draft_launches);
         if (rc) return rc;
     }
+    // the step-th forward of the round: its graph, or the launches themselves with
+    // the armed stall (test hook)
+    const int stall = h->stall_step > 0 ? h->stall_barrier : 0, stall_step = h->stall_step;
+    if (stall) h->stall_barrier = h->stall_step = 0;
+    auto launch = [&](cudaGraphExec_t g, int kind, int M, int round, int step) -> int {
+        if (stall && round == 0 && step == stall_step) {
+            const unsigned long long wait_ns = h->wait_ns;
+            int n = 0;
+            h->wait_ns = h->stall_wait_ns;
+            const int rc = step_launches(h, kind, M, mode, &n, stall);
+            h->wait_ns = wait_ns;
+            return rc;
+        }
+        CUDA_TRY(cudaGraphLaunch(g, h->stream), kind == G_DRAFT ? "draft step" : "verification step");
+        return SSD_OK;
+    };
     const size_t need_events = 3 * (size_t)n_new + 2;
     while (h->events.size() < need_events) {
         cudaEvent_t ev;
@@ -995,7 +1012,8 @@ int ssd_generate(ssd_handle* h, const int32_t* prompt, int n_prompt, int n_new, 
         }
         cudaEvent_t* ev = &h->events[2 + 3 * (size_t)round];
         CUDA_TRY(cudaEventRecord(ev[0], h->stream), "event");
-        for (int j = 0; j < Kd; ++j) CUDA_TRY(cudaGraphLaunch(g_draft, h->stream), "draft step");
+        for (int j = 0; j < Kd; ++j)
+            if (int rc = launch(g_draft, G_DRAFT, 1, round, j + 1)) return rc;
         CUDA_TRY(cudaEventRecord(ev[1], h->stream), "event");
         // with the draft exit the round's draft count is known on the device
         // only: read it before choosing the verification's row count
@@ -1010,7 +1028,7 @@ int ssd_generate(ssd_handle* h, const int32_t* prompt, int n_prompt, int n_new, 
             if (rc) return rc;
         }
         launches += (long long)Kd * draft_launches + verify_launches;
-        CUDA_TRY(cudaGraphLaunch(g_verify, h->stream), "verification step");
+        if (int rc = launch(g_verify, G_VERIFY, Kv + 1, round, Kd + 1)) return rc;
         CUDA_TRY(cudaEventRecord(ev[2], h->stream), "event");
         static_assert(offsetof(DecodeState, err) == offsetof(DecodeState, emitted) + sizeof(int), "read together");
         CUDA_TRY(cudaMemcpyAsync(h->emitted_host, &h->st->emitted, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream),
@@ -1063,7 +1081,7 @@ int ssd_debug_forward(ssd_handle* h, int draft, const int32_t* tokens, int n_row
         if (tokens[i] < 0 || tokens[i] >= h->cfg.vocab) return fail(SSD_ERR_INVALID_ARG, "token out of range");
     CUDA_TRY(cudaSetDevice(h->device), "set device");
     if (int rc = begin_launches(h)) return rc;
-    const int stall = h->stall_barrier;
+    const int stall = h->stall_step == 0 ? h->stall_barrier : 0;
     const unsigned long long wait_ns = h->wait_ns;
     if (stall) {  // armed by ssd_debug_stall_barrier for this one forward
         h->wait_ns = h->stall_wait_ns;
@@ -1084,7 +1102,8 @@ int ssd_debug_stall_barrier(ssd_handle* h, int barrier, double wait_limit_s) {
     if (!h) return fail(SSD_ERR_INVALID_ARG, "NULL handle");
     if (barrier < 0 || !(wait_limit_s > 0.0) || wait_limit_s > 10.0)
         return fail(SSD_ERR_INVALID_ARG, "need barrier >= 0 and 0 < wait_limit_s <= 10");
-    h->stall_barrier = barrier;
+    h->stall_barrier = barrier & 0xffff;
+    h->stall_step = h->stall_barrier ? barrier >> 16 : 0;
     h->stall_wait_ns = (unsigned long long)(wait_limit_s * 1e9);
     return SSD_OK;
 }
@@ -1095,10 +1114,13 @@ int trace_forward(ssd_handle* h, cudaGraphExec_t exec, int n_ops, std::vector<fl
                   std::vector<unsigned long long>* units = nullptr) {
     std::vector<unsigned long long> t(trace_words(h));
     CUDA_TRY(cudaMemsetAsync(h->trace, 0, t.size() * sizeof(unsigned long long), h->stream), "trace reset");
+    if (int rc = begin_launches(h)) return rc;
     CUDA_TRY(cudaGraphLaunch(exec, h->stream), "traced replay");
+    if (int rc = read_error(h)) return rc;
     CUDA_TRY(cudaMemcpyAsync(t.data(), h->trace, t.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                              h->stream), "trace read");
     CUDA_TRY(cudaStreamSynchronize(h->stream), "trace");
+    if (int rc = end_launches(h)) return rc;
     us->resize(n_ops);
     for (int o = 0; o < n_ops; ++o) (*us)[o] = (float)((double)(t[o + 1] - t[o]) * 1e-3);
     if (units) *units = t;
@@ -1107,7 +1129,6 @@ int trace_forward(ssd_handle* h, cudaGraphExec_t exec, int n_ops, std::vector<fl
 
 int capture_debug_forward(ssd_handle* h, int draft, int rows, bool traced, cudaGraphExec_t* exec, int* n) {
     const int pos0 = h->cfg.max_seq - rows;
-    if (int rc = begin_launches(h)) return rc;
     const int dt[kMaxRows] = {};
     cudaGraph_t g = nullptr;
     CUDA_TRY(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
@@ -1139,19 +1160,23 @@ int ssd_debug_time_forward(ssd_handle* h, int draft, int rows, int gemm_only, in
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
+    rc = begin_launches(h);
     if (e == cudaSuccess) e = cudaGraphLaunch(exec, h->stream);  // warm-up
     if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
     for (int r = 0; r < reps && e == cudaSuccess; ++r) e = cudaGraphLaunch(exec, h->stream);
     if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
-    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+    if (!rc) rc = read_error(h);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (!rc && e == cudaSuccess) rc = end_launches(h);  // (replays behind a failed one do nothing)
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     cudaGraphExecDestroy(exec);
-    if (e != cudaSuccess) {
+    if (rc || e != cudaSuccess) {
         if (traced) cudaGraphExecDestroy(traced);
         CUDA_TRY(e, "timing");
+        return rc;
     }
     ms /= reps;
     *launches = n;
@@ -1197,8 +1222,8 @@ int ssd_debug_trace_forward(ssd_handle* h, int draft, int rows, float* op_us, in
     if (rc) return rc;
     std::vector<float> us;
     std::vector<unsigned long long> units;
-    CUDA_TRY(cudaGraphLaunch(traced, h->stream), "warm-up");
-    rc = trace_forward(h, traced, n_ops, &us, &units);
+    rc = trace_forward(h, traced, n_ops, &us);  // warm-up
+    if (!rc) rc = trace_forward(h, traced, n_ops, &us, &units);
     cudaGraphExecDestroy(traced);
     if (rc) return rc;
     std::vector<FwdOp> ops = build_ops(h, draft != 0);

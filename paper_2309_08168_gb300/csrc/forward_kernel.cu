@@ -1384,7 +1384,7 @@ template <int R, int HD>
 __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ float r_s[kMaxRows];
-    __shared__ int s_pos0, s_skip;
+    __shared__ int s_pos0, s_leave;
     __shared__ unsigned s_seq;
     __shared__ uint32_t s_tmem;
     constexpr int S = GemmSmem<R>::S;
@@ -1405,8 +1405,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams
         else if (p.src == SRC_DRAFT) pos0 = p.st->len + p.st->j;
         else pos0 = p.st->len;
         s_pos0 = pos0;
-        // a draft step after the round's drafting stage ended (draft exit): no work
-        s_skip = p.src == SRC_DRAFT && *(volatile int*)&p.st->exited;
+        // no work: a draft step after the round's drafting stage ended (draft exit),
+        // or a forward queued behind a failed one, which may have left the barrier
+        // counters and the sequence number anywhere (the host clears them)
+        s_leave = (p.src == SRC_DRAFT && *(volatile int*)&p.st->exited) || *(volatile int*)p.err;
         s_seq = *(volatile unsigned*)p.seq;  // this forward's number (advanced by CTA 0 below)
         for (int st = 0; st < S; ++st) {
             mbar_init(full + st, 1);
@@ -1424,7 +1426,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) forward_kernel(const FwdParams
         if (p.trace && blockIdx.x == 0) p.trace[0] = globaltimer();
     }
     __syncthreads();
-    if (s_skip) return;
+    if (s_leave) return;
     if (mma_warp) {  // TMEM for the two projection accumulators (freed at the end)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
                      "r"(kTmemCols)

@@ -151,7 +151,8 @@ struct FwdParams {
     bf16* xn_lo;
     float* ss;            // per-128-column sums of h^2 [16][d/128]
     unsigned* bar;        // [2] grid-barrier counters: launch number seq counts on bar[seq & 1], zero at
-                          // launch, and zeroes the other one for the next launch
+                          // launch, and zeroes the other one for the next launch (a launch that finds
+                          // the error flag set leaves at once)
     unsigned* seq;        // forward sequence number (tags split-K partials; +1 per launch)
     int* err;             // device error code
     // Profiling hook: nullptr, or globaltimer stamps: [0, n_ops] start, end of
