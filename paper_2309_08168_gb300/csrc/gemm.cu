@@ -55,11 +55,16 @@ __device__ __forceinline__ float ld_cluster(uint32_t saddr, unsigned rank) {
     asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(r) : "memory");
     return v;
 }
-// 16 weight bytes, read once: not kept in L1.  volatile, like the MMAs, so that
-// the loads stay as far ahead of them as they are written
+// 16 weight bytes, read once: not kept in L1.  Not the non-coherent path (.nc): the
+// weights may come from the kernel before, which can still run when this one starts
+// (calls back to back over 12 matrices, 16 x 4096 x 4096 12.0 us, 11.5 with .nc; 4 x 4096
+// x 32000 50.0 / 49.9, 8 x 8192 x 8192 26.5 / 26.5; .cg 12.2 / 52.9 / 28.8, .cs 12.0 / 49.7 /
+// 26.6).
+// volatile, like the MMAs, so that the loads stay as far ahead of them as they are
+// written
 __device__ __forceinline__ uint4 ld_weights(const bf16* p) {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                  : "l"(p));
     return v;
