@@ -48,9 +48,11 @@ __global__ void __launch_bounds__(kNormThreads) pf_embed_kernel(const bf16* __re
 // row stays in registers between the sum and the scaling up to d = 8192.  Bound
 // by L2 (h was just written there): 511 rows of d 4096, 5.6 us; one
 // feature a thread and two passes over h took 7.5.
-__global__ void __launch_bounds__(kNormThreads) pf_norm_kernel(const float* __restrict__ h,
-                                                               const bf16* __restrict__ g, int d, float eps,
-                                                               bf16* __restrict__ x_hi, bf16* __restrict__ x_lo) {
+// (h through __ldcg: the kernel that writes it may still run when this one starts,
+// so its loads must not be taken for loads of constants.)
+__global__ void __launch_bounds__(kNormThreads) pf_norm_kernel(const float* h, const bf16* __restrict__ g, int d,
+                                                               float eps, bf16* __restrict__ x_hi,
+                                                               bf16* __restrict__ x_lo) {
     constexpr int KEEP = 8;
     __shared__ float s_part[kNormThreads / 32];
     pdl_launch_dependents();
@@ -62,13 +64,13 @@ __global__ void __launch_bounds__(kNormThreads) pf_norm_kernel(const float* __re
 #pragma unroll
     for (int k = 0; k < KEEP; ++k) {
         const int i = threadIdx.x + k * kNormThreads;
-        v[k] = i < n4 ? hr[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[k] = i < n4 ? __ldcg(hr + i) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     float ss = 0.f;
 #pragma unroll
     for (int k = 0; k < KEEP; ++k) ss += (v[k].x * v[k].x + v[k].y * v[k].y) + (v[k].z * v[k].z + v[k].w * v[k].w);
     for (int i = threadIdx.x + KEEP * kNormThreads; i < n4; i += kNormThreads) {
-        const float4 x = hr[i];
+        const float4 x = __ldcg(hr + i);
         ss += (x.x * x.x + x.y * x.y) + (x.z * x.z + x.w * x.w);
     }
     ss = warp_sum(ss);
@@ -99,7 +101,7 @@ __global__ void __launch_bounds__(kNormThreads) pf_norm_kernel(const float* __re
         const int i = threadIdx.x + k * kNormThreads;
         if (i < n4) store(i, v[k]);
     }
-    for (int i = threadIdx.x + KEEP * kNormThreads; i < n4; i += kNormThreads) store(i, hr[i]);
+    for (int i = threadIdx.x + KEEP * kNormThreads; i < n4; i += kNormThreads) store(i, __ldcg(hr + i));
 }
 
 // ---------------------------------------------------------------------------
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(kAttThreads, 1) pf_attn_kernel(const AttArgs a
             for (int i = 0; i < 8; ++i) {
                 const int r = warp * 32 + i0 + i * RPI + lane / LPR, e = (lane % LPR) * 4;
                 x[i] = qr0 + r < a.n_rows
-                           ? *reinterpret_cast<const float4*>(a.q + (size_t)(qr0 + r) * qd + head * HD + e)
+                           ? __ldcg(reinterpret_cast<const float4*>(a.q + (size_t)(qr0 + r) * qd + head * HD + e))
                            : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
