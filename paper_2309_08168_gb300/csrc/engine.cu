@@ -275,13 +275,16 @@ int build_tmaps(ssd_handle* h) {
 //   w_gate, w_up one map {K, 16, 2, rows / 16} whose third stride is the distance
 //                between the two matrices: one box is 128 rows, 16 of gate, 16 of
 //                up, ..., so that a TMEM lane quadrant holds both (at w_gate's
-//                place; the lower matrix comes first).  A tensor map's strides
-//                end at 2^40: matrices further apart get a map each, {K, rows},
-//                box of 16 rows, and eight copies per tile instead of one
+//                place; the lower matrix comes first)
 //   wq wk wv     {K, 16, 2, hd / 32, heads} with strides of 1 row, hd / 2 rows,
 //                16 rows and hd rows: one box is 128 rows, 16 of the first
 //                half of a head's dims, then their 16 rotation partners, ...
 //   planes       {K, rows, 2}, box of tok / 2 rows of hi and of lo
+// The strides of the first two do not grow from dimension to dimension, as the
+// driver's documentation has it (the drivers in use take them), end at 2^40 and
+// cannot be 0 (one matrix as gate and up).  Where such a map does not exist the
+// matrices get plain ones, {K, rows}, box of 16 rows, and eight copies bring the
+// same 128 rows.  SSD_PLAIN_TMAPS=1 in the environment chooses those (for tests).
 int build_prefill(ssd_handle* h) {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -290,8 +293,9 @@ int build_prefill(ssd_handle* h) {
     if (!fn || q != cudaDriverEntryPointSuccess) return fail(SSD_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
     auto enc = (PFN_cuTensorMapEncodeTiled_v12000)fn;
     const ssd_config& c = h->cfg;
-    const int L = c.n_layers, d = c.d_model, qd = c.n_heads * c.head_dim;
+    const int L = c.n_layers, d = c.d_model, qd = c.n_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim;
     PrefillPlan& P = h->pf;
+    h->pf_layers.resize(L);
     std::vector<CUtensorMap> maps((size_t)7 * L + 3 * kPfTokClasses);
     auto rows2 = [&](CUtensorMap* m, const void* base, int K, int rows, int box_rows) {
         return encode_weight(enc, m, base, K, rows, box_rows);
@@ -303,15 +307,12 @@ int build_prefill(ssd_handle* h) {
         cuuint32_t box[5] = {64, 16, 2, (cuuint32_t)(hd / 32), (cuuint32_t)(128 / hd)};
         return encode_map(enc, m, base, 5, dims, strides, box);
     };
-    auto far_apart = [](const bf16* g, const bf16* u) {
-        const uintptr_t x = (uintptr_t)g, y = (uintptr_t)u;
-        return (x < y ? y - x : x - y) >= ((uintptr_t)1 << 40);
-    };
+    const char* env = std::getenv("SSD_PLAIN_TMAPS");
+    const bool plain = env && env[0] == '1';
+    // nonzero: no such map (another form will do)
     auto pair4 = [&](CUtensorMap* m, const bf16* g, const bf16* u) {
-        if (far_apart(g, u)) {
-            const int r = rows2(m, g, d, c.ffn, 16);
-            return r ? r : rows2(m + 1, u, d, c.ffn, 16);
-        }
+        const uintptr_t x = (uintptr_t)g, y = (uintptr_t)u, dist = x < y ? y - x : x - y;
+        if (plain || dist == 0 || dist >= ((uintptr_t)1 << 40)) return 1;
         const bf16 *lo = g < u ? g : u, *hi = g < u ? u : g;
         const cuuint64_t row = (cuuint64_t)d * 2;
         cuuint64_t dims[4] = {(cuuint64_t)d, 16, 2, (cuuint64_t)(c.ffn / 16)};
@@ -328,11 +329,23 @@ int build_prefill(ssd_handle* h) {
     int rc = 0;
     for (int l = 0; l < L && !rc; ++l) {
         CUtensorMap* m = &maps[(size_t)7 * l];
-        if (!rc) rc = heads5(m + 0, h->wq[l], c.n_heads);
-        if (!rc) rc = heads5(m + 1, h->wk[l], c.n_kv_heads);
-        if (!rc) rc = heads5(m + 2, h->wv[l], c.n_kv_heads);
+        PrefillLayer& Ly = h->pf_layers[l];
+        Ly.qkv_rows16 = plain || heads5(m + 0, h->wq[l], c.n_heads) || heads5(m + 1, h->wk[l], c.n_kv_heads) ||
+                        heads5(m + 2, h->wv[l], c.n_kv_heads);
+        if (Ly.qkv_rows16) {
+            rc = rows2(m + 0, h->wq[l], d, qd, 16);
+            if (!rc) rc = rows2(m + 1, h->wk[l], d, kvd, 16);
+            if (!rc) rc = rows2(m + 2, h->wv[l], d, kvd, 16);
+        }
         if (!rc) rc = rows2(m + 3, h->wo[l], qd, d, 128);
-        if (!rc) rc = pair4(m + 4, h->w_gate[l], h->w_up[l]);
+        Ly.swapped = h->w_up[l] < h->w_gate[l];
+        Ly.tm_w[5] = nullptr;
+        if (!rc && pair4(m + 4, h->w_gate[l], h->w_up[l])) {
+            Ly.swapped = 0;
+            Ly.tm_w[5] = h->pf_tmaps + (m + 5 - maps.data());
+            rc = rows2(m + 4, h->w_gate[l], d, c.ffn, 16);
+            if (!rc) rc = rows2(m + 5, h->w_up[l], d, c.ffn, 16);
+        }
         if (!rc) rc = rows2(m + 6, h->w_down[l], c.ffn, d, 128);
     }
     const size_t a0 = (size_t)7 * L;
@@ -344,13 +357,10 @@ int build_prefill(ssd_handle* h) {
     if (rc) return rc;
     CUDA_TRY(cudaMemcpy(h->pf_tmaps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice),
              "prefill tensor map upload");
-    h->pf_layers.resize(L);
     for (int l = 0; l < L; ++l) {
         PrefillLayer& Ly = h->pf_layers[l];
-        for (int i = 0; i < 7; ++i) Ly.tm_w[i] = h->pf_tmaps + 7 * l + i;
-        Ly.swapped = h->w_up[l] < h->w_gate[l];
-        if (far_apart(h->w_gate[l], h->w_up[l])) Ly.swapped = 0;
-        else Ly.tm_w[5] = nullptr;
+        for (int i = 0; i < 7; ++i)
+            if (i != 5) Ly.tm_w[i] = h->pf_tmaps + 7 * l + i;
         Ly.attn_norm = h->attn_norm[l];
         Ly.mlp_norm = h->mlp_norm[l];
         Ly.k_cache = h->kc + (size_t)l * h->kv_layer;

@@ -511,6 +511,7 @@ int prefill_chunk(PrefillPlan& P, const int* toks, int n, int pos0, cudaStream_t
         a.tm_w[0] = L.tm_w[0];
         a.tm_w[1] = L.tm_w[1];
         a.tm_w[2] = L.tm_w[2];
+        a.rows16 = L.qkv_rows16;
         a.n_heads = P.n_heads;
         a.n_kv_heads = P.n_kv_heads;
         a.head_dim = P.head_dim;

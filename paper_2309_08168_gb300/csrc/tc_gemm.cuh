@@ -79,7 +79,8 @@ struct TcArgs {
     // TMA maps.  Weights: RESID {K, N}, box {64, 128}; SWIGLU gate and up in one
     // map {K, 16, 2, N / 16}, box {64, 16, 2, 4} (the lower matrix in memory
     // first: swapped = 1 if that is up), or [1] != nullptr: gate, up {K, N}, box
-    // {64, 16} each; QKV wq, wk, wv as {K, 16, 2, hd / 32, heads}, box = 128 rows.
+    // {64, 16} each; QKV wq, wk, wv as {K, 16, 2, hd / 32, heads}, box = 128 rows, or
+    // (rows16) {K, N}, box {64, 16}.
     // Tokens: planes as {K, rows, 2}, box {64, nt / 2, 2}.
     const void* tm_w[3];
     const void* tm_x;
@@ -89,6 +90,7 @@ struct TcArgs {
     int stages;            // ring depth
     int N;                 // output features (SWIGLU: ffn)
     int swapped;           // SWIGLU: lanes 0-15 hold up, 16-31 gate
+    int rows16;            // QKV: eight boxes of 16 rows instead of one of 128
     TcSched sched;
     float* ws;             // [pairs][2][256][128] fp32 partial sums
     unsigned* flags;       // [pairs][2][16] epoch of the partial sums a warp left
@@ -390,7 +392,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm
                 const uint32_t bar = full0 + 8u * (uint32_t)st_i;
                 if (rank == 0) mb_arrive_tx(full + st_i, 2u * (unsigned)stage_bytes);
                 if (EPI == TC_QKV) {
-                    tma5d_head(st, map, kb * kBK, row0, bar);
+                    if (!a.rows16) {
+                        tma5d_head(st, map, kb * kBK, row0, bar);
+                    } else {  // the same rows, 16 at a time: heads row0 .., a half's 16, their partners, ...
+                        const int per = a.head_dim >> 4;
+                        for (int p = 0; p < 8; ++p) {
+                            const int j = p % per;
+                            tma2d(st + p * 2048, map, kb * kBK,
+                                  (row0 + p / per) * a.head_dim + (j & 1) * (a.head_dim >> 1) + (j >> 1) * 16, bar);
+                        }
+                    }
                 } else if (EPI == TC_SWIGLU) {
                     if (a.tm_w[1] == nullptr) {
                         tma4d_pair(st, map, kb * kBK, box * 4, bar);
