@@ -49,8 +49,9 @@ __global__ void __launch_bounds__(kNormThreads) pf_embed_kernel(const bf16* __re
 // by L2 (h was just written there): 511 rows of d 4096, 5.6 us; one
 // feature a thread and two passes over h took 7.5.
 // (h through __ldcg: the kernel that writes it may still run when this one starts,
-// so its loads must not be taken for loads of constants.)
-__global__ void __launch_bounds__(kNormThreads) pf_norm_kernel(const float* h, const bf16* __restrict__ g, int d,
+// so its loads must not be taken for loads of constants.  Four CTAs an SM: at 66
+// registers, three, 7.2 us.)
+__global__ void __launch_bounds__(kNormThreads, 4) pf_norm_kernel(const float* h, const bf16* __restrict__ g, int d,
                                                                float eps, bf16* __restrict__ x_hi,
                                                                bf16* __restrict__ x_lo) {
     constexpr int KEEP = 8;
