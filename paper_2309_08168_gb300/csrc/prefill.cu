@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(kAttThreads, 1) pf_attn_kernel(const AttArgs a
                 ok = __all_sync(0xffffffffu, tc::mb_wait(pv_done + ((j - 1) & 1), (unsigned)((j - 1) >> 1) & 1u, a.err));
                 if (!ok) break;
                 tc::fence_after();
-                const float nm = fmaxf(mx, bm), f = exp2f(mx - nm);
+                const float nm = fmaxf(mx, bm), f = nm == -INFINITY ? 1.f : exp2f(mx - nm);
                 for (int c = 0; c < HD; c += 32) {
                     uint32_t o[32];
                     att_ld32(tl + c, o);
@@ -399,12 +399,14 @@ __global__ void __launch_bounds__(kAttThreads, 1) pf_attn_kernel(const AttArgs a
                 l *= f;
                 mx = nm;
             }
+            // (a row whose scores so far are all -inf, against infinite keys: weights 0)
+            const float ref = mx == -INFINITY ? 0.f : mx;
             uint32_t hi[32], lo[32];
             float l4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-                const float p0 = exp2f(__uint_as_float(u0[2 * i]) - mx), p1 = exp2f(__uint_as_float(u0[2 * i + 1]) - mx);
-                const float p2 = exp2f(__uint_as_float(u1[2 * i]) - mx), p3 = exp2f(__uint_as_float(u1[2 * i + 1]) - mx);
+                const float p0 = exp2f(__uint_as_float(u0[2 * i]) - ref), p1 = exp2f(__uint_as_float(u0[2 * i + 1]) - ref);
+                const float p2 = exp2f(__uint_as_float(u1[2 * i]) - ref), p3 = exp2f(__uint_as_float(u1[2 * i + 1]) - ref);
                 l4[i & 3] += (p0 + p1) + (p2 + p3);
                 split_h2(p0, p1, hi[i], lo[i]);
                 split_h2(p2, p3, hi[i + 16], lo[i + 16]);
