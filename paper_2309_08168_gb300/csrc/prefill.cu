@@ -475,6 +475,7 @@ int prefill_configure() {
         e = (int)cudaFuncSetAttribute(pf_attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)AttSmem<64>::BYTES);
     if (!e) e = tc::tc_configure<tc::TC_QKV>();
+    if (!e) e = tc::tc_configure<tc::TC_QKV, true>();
     if (!e) e = tc::tc_configure<tc::TC_RESID>();
     if (!e) e = tc::tc_configure<tc::TC_SWIGLU>();
     return e;
@@ -514,7 +515,6 @@ int prefill_chunk(PrefillPlan& P, const int* toks, int n, int pos0, cudaStream_t
         a.tm_w[0] = L.tm_w[0];
         a.tm_w[1] = L.tm_w[1];
         a.tm_w[2] = L.tm_w[2];
-        a.rows16 = L.qkv_rows16;
         a.n_heads = P.n_heads;
         a.n_kv_heads = P.n_kv_heads;
         a.head_dim = P.head_dim;
@@ -524,7 +524,7 @@ int prefill_chunk(PrefillPlan& P, const int* toks, int n, int pos0, cudaStream_t
         a.k_cache = L.k_cache;
         a.v_cache = L.v_cache;
         a.rope = P.rope;
-        e = tc::tc_launch<tc::TC_QKV>(a, s);
+        e = L.qkv_rows16 ? tc::tc_launch<tc::TC_QKV, true>(a, s) : tc::tc_launch<tc::TC_QKV>(a, s);
         if (e) break;
         AttArgs t{};
         t.q = P.q;

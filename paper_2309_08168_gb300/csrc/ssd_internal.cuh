@@ -175,7 +175,7 @@ constexpr int kPfTokClasses = 8;  // token tiles of 32 (class + 1) rows
 struct PrefillLayer {
     const void* tm_w[7];  // TMA maps of wq wk wv wo w_gate w_up w_down (TcArgs::tm_w; w_up: nullptr if in w_gate's)
     int swapped;          // w_up lies below w_gate (TcArgs::swapped)
-    int qkv_rows16;       // the maps of wq wk wv have boxes of 16 rows (TcArgs::rows16)
+    int qkv_rows16;       // the maps of wq wk wv have boxes of 16 rows
     const bf16* attn_norm;
     const bf16* mlp_norm;
     f16* k_cache;  // this layer's [Hkv][max_seq][hd]

@@ -80,7 +80,7 @@ struct TcArgs {
     // map {K, 16, 2, N / 16}, box {64, 16, 2, 4} (the lower matrix in memory
     // first: swapped = 1 if that is up), or [1] != nullptr: gate, up {K, N}, box
     // {64, 16} each; QKV wq, wk, wv as {K, 16, 2, hd / 32, heads}, box = 128 rows, or
-    // (rows16) {K, N}, box {64, 16}.
+    // (ROWS16) {K, N}, box {64, 16}.
     // Tokens: planes as {K, rows, 2}, box {64, nt / 2, 2}.
     const void* tm_w[3];
     const void* tm_x;
@@ -90,7 +90,6 @@ struct TcArgs {
     int stages;            // ring depth
     int N;                 // output features (SWIGLU: ffn)
     int swapped;           // SWIGLU: lanes 0-15 hold up, 16-31 gate
-    int rows16;            // QKV: eight boxes of 16 rows instead of one of 128
     TcSched sched;
     float* ws;             // [pairs][2][256][128] fp32 partial sums
     unsigned* flags;       // [pairs][2][16] epoch of the partial sums a warp left
@@ -321,7 +320,8 @@ __device__ __forceinline__ void pair_up(const float (&v)[16], int upper, float (
 // ---------------------------------------------------------------------------
 // the kernel: grid = 2 * pairs, clusters of 2
 // ---------------------------------------------------------------------------
-template <int EPI>
+// ROWS16 (QKV): the weights in eight boxes of 16 rows per k block instead of one of 128
+template <int EPI, bool ROWS16>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm_kernel(const TcArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -392,10 +392,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm
                 const uint32_t bar = full0 + 8u * (uint32_t)st_i;
                 if (rank == 0) mb_arrive_tx(full + st_i, 2u * (unsigned)stage_bytes);
                 if (EPI == TC_QKV) {
-                    if (!a.rows16) {
+                    if (!ROWS16) {
                         tma5d_head(st, map, kb * kBK, row0, bar);
                     } else {  // the same rows, 16 at a time: heads row0 .., a half's 16, their partners, ...
                         const int per = a.head_dim >> 4;
+#pragma unroll
                         for (int p = 0; p < 8; ++p) {
                             const int j = p % per;
                             tma2d(st + p * 2048, map, kb * kBK,
@@ -704,9 +705,9 @@ inline void tc_plan(TcArgs& a, int n_ft, int pairs, int K) {
     a.stages = kRingBytes / stage < kMaxStages ? kRingBytes / stage : kMaxStages;
 }
 
-template <int EPI>
+template <int EPI, bool ROWS16 = false>
 inline int tc_configure() {
-    return (int)cudaFuncSetAttribute(tc_gemm_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return (int)cudaFuncSetAttribute(tc_gemm_kernel<EPI, ROWS16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kSmemBytes);
 }
 
@@ -726,9 +727,9 @@ inline int launch_pdl(void (*k)(P...), dim3 grid, int threads, size_t smem, cuda
     return (int)cudaLaunchKernelEx(&cfg, k, args...);
 }
 
-template <int EPI>
+template <int EPI, bool ROWS16 = false>
 inline int tc_launch(const TcArgs& a, cudaStream_t s) {
-    return launch_pdl(tc_gemm_kernel<EPI>, dim3(2 * a.sched.pairs), kThreads, kSmemBytes, s, a);
+    return launch_pdl(tc_gemm_kernel<EPI, ROWS16>, dim3(2 * a.sched.pairs), kThreads, kSmemBytes, s, a);
 }
 
 }  // namespace tc
