@@ -155,18 +155,14 @@ __device__ __forceinline__ int unit_owner(long long u, long long U, long long G)
 // An op's units are split over the first min(U, grid) CTAs, so every CTA that
 // takes part owns at least one unit and the owners of consecutive units are
 // consecutive CTAs (the segment arithmetic of the projection op relies on it).
-// A tile of at most kWholeChunks chunks is one CTA's if there is a CTA for every
-// tile: two or three units one after the other take 0.35 us each, the split-K
-// exchange ~1 us (tiny model, a forward of 5 rows: 100.4 us, split 101.0).
-constexpr int kWholeChunks = 3;
-__device__ __forceinline__ long long op_ctas(long long U, int n_chunks) {
-    const long long G = gridDim.x;
-    if (n_chunks <= kWholeChunks && U <= G * n_chunks) return U / n_chunks;
-    return U < G ? U : G;
-}
+// Keeping tiles of two or three chunks whole (units one after the other instead of a
+// split-K exchange) is no gain: forwards of 1 / 5 / 16 rows take 188.5 / 209.0 / 253.2 us
+// so at d 384 (8 layers) and 165.4 / 189.6 / 247.7 split, 86.1 / 96.4 / 127.7 against
+// 85.8 / 95.8 / 129.0 at d 256.
+__device__ __forceinline__ long long op_ctas(long long U) { return U < gridDim.x ? U : (long long)gridDim.x; }
 
-__device__ __forceinline__ void my_units(long long U, int n_chunks, int* u_begin, int* n_my) {
-    const long long G = op_ctas(U, n_chunks), b = blockIdx.x;
+__device__ __forceinline__ void my_units(long long U, int* u_begin, int* n_my) {
+    const long long G = op_ctas(U), b = blockIdx.x;
     if (b >= G) { *u_begin = 0; *n_my = 0; return; }
     *u_begin = (int)(b * U / G);
     *n_my = (int)((b + 1) * U / G) - *u_begin;
@@ -517,7 +513,7 @@ __device__ bool gemm_produce(const GemmArgs& a, int epi, unsigned char* smem, Pi
     using L = GemmSmem<R>;
     constexpr int S = L::S;
     int u_begin, n_my;
-    my_units(a.n_units, a.n_chunks, &u_begin, &n_my);
+    my_units(a.n_units, &u_begin, &n_my);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (n_my > 0 && elect_one()) prefetch_tmap(a.tm_x[plane_cls(R)]);
     __syncwarp();
@@ -556,7 +552,7 @@ __device__ bool gemm_mma(int n_units, int n_chunks, unsigned char* smem, Pipe& p
     using L = GemmSmem<R>;
     constexpr int S = L::S, NP = L::NP;
     int u_begin, n_my;
-    my_units(n_units, n_chunks, &u_begin, &n_my);
+    my_units(n_units, &u_begin, &n_my);
     constexpr uint32_t idesc = umma_idesc(NP);
     const uint64_t desc0 = umma_desc(smem_u32(smem));  // (descriptors count 16-byte steps)
     int chunk = u_begin % n_chunks;
@@ -602,10 +598,10 @@ __device__ bool gemm_consume(const GemmArgs& a, int epi, int M, int pos0, unsign
     float* ys = reinterpret_cast<float*>(smem + L::YS);  // [128][16]
     bool ok = true;
 
-    const long long U = a.n_units, G = op_ctas(U, a.n_chunks);
+    const long long U = a.n_units, G = op_ctas(U);
     const int b = blockIdx.x;
     int u_begin, n_my;
-    my_units(U, a.n_chunks, &u_begin, &n_my);
+    my_units(U, &u_begin, &n_my);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // 1 / rms of each input row from the previous op's per-tile sums of

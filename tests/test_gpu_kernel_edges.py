@@ -23,8 +23,8 @@ last tenth of the nucleus is drawn from.  High temperatures put most of the row 
 threshold is searched in, top_p next to 1 takes the search down to zero.
 
 Decode: forwards around the first segment's end (position 128), where
-attention without partials takes over, and with K of one to four chunks,
-where a tile is one CTA's: every row the same bits as alone.
+attention without partials takes over, and with K of one to four chunks
+(the shortest splits): every row the same bits as alone.
 """
 import numpy as np
 import pytest
