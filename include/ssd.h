@@ -253,7 +253,10 @@ int ssd_debug_trace_forward(ssd_handle* h, int draft, int rows, float* op_us, in
  * with SSD_ERR_CAPACITY before any launch.  The first call on each device does
  * a one-time set-up with that device current (kernel attributes); make that
  * first call before any stream capture.  Faults inside the kernel are not
- * reported by this call (it returns once the work is enqueued).
+ * reported by this call (it returns once the work is enqueued); builds with
+ * the device-side checks enabled (SSD_CHECKED=1) check the alignment and the
+ * bounds of the kernel's accesses, read the check flag back after the kernel,
+ * which makes the call synchronous, and report a failed check as SSD_ERR_CUDA.
  * Errors: INVALID_ARG, CAPACITY, CUDA. */
 int ssd_linear_noalloc(const void* w, const float* x, float* y, int N, int K, int M,
                        void* cuda_stream);

@@ -46,7 +46,19 @@ struct LinearArgs {
     float* y;
     int N, K, M;
     int kc;  // k per CTA of the cluster, a multiple of 64
+
+    // what the accesses of a checked build have to satisfy
+    __host__ __device__ bool weights_in(const bf16* p, size_t elems) const {
+        return ((uintptr_t)p & 15u) == 0 && p >= w && p + elems <= w + (size_t)N * K;
+    }
+    __host__ __device__ bool inputs_in(const float* p, size_t elems) const {
+        return ((uintptr_t)p & 15u) == 0 && p >= x && p + elems <= x + (size_t)M * K;
+    }
+    __host__ __device__ bool output_in(const float* p) const { return p >= y && p < y + (size_t)M * N; }
 };
+#ifdef SSD_CHECKED
+__device__ int g_linear_err;  // code of the first failed check
+#endif
 
 __device__ __forceinline__ float ld_cluster(uint32_t saddr, unsigned rank) {
     uint32_t r;
@@ -62,8 +74,9 @@ __device__ __forceinline__ float ld_cluster(uint32_t saddr, unsigned rank) {
 // 26.6).
 // volatile, like the MMAs, so that the loads stay as far ahead of them as they are
 // written
-__device__ __forceinline__ uint4 ld_weights(const bf16* p) {
-    uint4 v;
+__device__ __forceinline__ uint4 ld_weights(const LinearArgs& a, const bf16* p) {
+    uint4 v = make_uint4(0, 0, 0, 0);
+    SSD_GUARD(&g_linear_err, a.weights_in(p, 8), 101)
     asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                  : "l"(p));
@@ -109,10 +122,10 @@ __global__ void __launch_bounds__(kLinThreads, LinShape<P>::CTAS) linear_kernel(
         const int k = k0 + b * 64;
         const uint4 z = make_uint4(0, 0, 0, 0);
         const bool in0 = k + t * 8 < k1, in1 = k + 32 + t * 8 < k1;
-        d[0] = in0 ? ld_weights(w0 + k) : z;
-        d[1] = in0 ? ld_weights(w1 + k) : z;
-        d[2] = in1 ? ld_weights(w0 + k + 32) : z;
-        d[3] = in1 ? ld_weights(w1 + k + 32) : z;
+        d[0] = in0 ? ld_weights(a, w0 + k) : z;
+        d[1] = in0 ? ld_weights(a, w1 + k) : z;
+        d[2] = in1 ? ld_weights(a, w0 + k + 32) : z;
+        d[3] = in1 ? ld_weights(a, w1 + k + 32) : z;
     };
     // The weights on their way into L2 while the previous kernel ends (a prefetch
     // returns nothing, so it may run ahead of a kernel that writes them).  Calls
@@ -121,6 +134,7 @@ __global__ void __launch_bounds__(kLinThreads, LinShape<P>::CTAS) linear_kernel(
     if (threadIdx.x < kLinRows && k1 > k0) {
         const bf16* row = a.w + (size_t)min(tile * kLinRows + (int)threadIdx.x, a.N - 1) * a.K + k0;
         const unsigned bytes = (unsigned)min(k1 - k0, kPrefetchK) * 2u;  // (K is a multiple of 16: 32-byte steps)
+        SSD_GUARD(&g_linear_err, a.weights_in(row, bytes / 2), 102)
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(row), "r"(bytes) : "memory");
     }
     pdl_wait();  // weights and activations may come from the previous kernel
@@ -143,10 +157,13 @@ __global__ void __launch_bounds__(kLinThreads, LinShape<P>::CTAS) linear_kernel(
             uint4 hi = make_uint4(0, 0, 0, 0), lo = make_uint4(0, 0, 0, 0);
             if (n < a.M && k < k1) {
                 const float4* src = reinterpret_cast<const float4*>(a.x + (size_t)n * a.K + k);
+                SSD_GUARD(&g_linear_err, a.inputs_in(reinterpret_cast<const float*>(src), 8), 103)
                 split8(__ldcg(src), __ldcg(src + 1), hi, lo);
             }
-            *reinterpret_cast<uint4*>(xs + n * pitch + cc * 16) = hi;
-            *reinterpret_cast<uint4*>(xs + (P + n) * pitch + cc * 16) = lo;
+            SSD_GUARD(&g_linear_err, n < P && cc * 16 + 16 <= pitch, 104) {
+                *reinterpret_cast<uint4*>(xs + n * pitch + cc * 16) = hi;
+                *reinterpret_cast<uint4*>(xs + (P + n) * pitch + cc * 16) = lo;
+            }
         }
         __syncthreads();
         for (int b = 0; b < cb; b += kLinFold) {
@@ -200,6 +217,7 @@ __global__ void __launch_bounds__(kLinThreads, LinShape<P>::CTAS) linear_kernel(
             for (unsigned q = 1; q < 8; ++q)
                 if (q < n_ranks) s += v[q];
         }
+        SSD_GUARD(&g_linear_err, a.output_in(a.y + (size_t)m * a.N + n), 105)
         a.y[(size_t)m * a.N + n] = s;
     }
     if (n_ranks > 1) lin_cluster_sync();  // the other ranks have read this CTA's sums
@@ -306,5 +324,18 @@ extern "C" int ssd_linear_noalloc(const void* w, const float* x, float* y, int N
     e = (cudaError_t)(M > 8 ? launch_linear<16>(a, ranks, s) : launch_linear<8>(a, ranks, s));
     if (e != cudaSuccess)
         return set_last_error(SSD_ERR_CUDA, (std::string("ssd_linear_noalloc: ") + cudaGetErrorString(e)).c_str());
+#ifdef SSD_CHECKED
+    // read the flag back (which makes the call synchronous), clear it for the next call, report it
+    int derr = 0, *flag = nullptr;
+    e = cudaGetSymbolAddress((void**)&flag, g_linear_err);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&derr, flag, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && derr) e = cudaMemsetAsync(flag, 0, sizeof(int), s);
+    if (e != cudaSuccess)
+        return set_last_error(SSD_ERR_CUDA, (std::string("ssd_linear_noalloc: ") + cudaGetErrorString(e)).c_str());
+    if (derr)
+        return set_last_error(SSD_ERR_CUDA,
+                              ("ssd_linear_noalloc: device check failed with code " + std::to_string(derr)).c_str());
+#endif
     return SSD_OK;
 }
