@@ -1,11 +1,22 @@
 """Sizes where the kernels' tiles, splits and fast paths begin and end.
 
-Prompt encoding (one number per prompt: the relative 2-norm error of the last
-row's logits against the fp64 oracle).  K and V are rounded to fp16 (2^-11 of
+Prompt encoding (the relative 2-norm error of the last row's logits against the
+fp64 oracle).  K and V are rounded to fp16 (2^-11 of
 their size each), everything else carries 16 bits or more, so the error of an
 output is a few times 2^-11 of what attention contributes: bound 4 * 2^-11.
 With large scores (S in magnitude) a score's own error, 2^-11 S, moves its
 weight by as much: bound 4 * 2^-11 * (1 + S).
+
+Such a bound lets one wrong row of a long prompt pass: attention is nearly uniform,
+so a row of 514 is 0.2 % of it.  The cache that the prompt kernels leave is therefore
+also compared with one that the decode kernel wrote, 16 rows at a time, through
+forwards at positions around the ends of tiles and blocks.  Both round the same
+K and V to fp16; sums in another order turn a rounding around here and there, by 2^-11
+of one value, and an output averages over many: bound 2^-11 (measured 2e-4).  A wrong
+row in the reference is seen by every later position that is tested.  With large
+scores, if all hd elements of a key turned around, with random signs, a score would
+move by 2^-11 S / sqrt(hd): bound 2^-11 * (1 + S / sqrt(hd)) (measured 2e-3 of 7e-3; an
+accumulator that is not rescaled is off by 2^8).
 
 Stand-alone projection: activations as bf16 pairs (2^-17 per element, in the
 2-norm about half of that), 32-bit sums: bound 1e-5.  A row's result is the
@@ -58,6 +69,33 @@ def prompt_error(w, hw, dw, P, seed, max_seq=None):
     return np.linalg.norm(got - ref) / np.linalg.norm(ref)
 
 
+EDGES = (1, 2, 15, 16, 17, 31, 32, 33, 63, 64, 65, 96, 127, 128, 129, 160, 191, 192, 193, 255, 256, 257, 258, 288, 384,
+         511, 512)
+
+
+class CachePair:
+    """The prompt's cache by the prompt kernels and by the decode kernel, and the
+    relative 2-norm distance of the logits at a position over the two."""
+
+    def __init__(self, w, dw, P, seed):
+        import paper_2309_08168_gb300 as ssd
+        torch.cuda.synchronize()
+        self.prompt = synth.prompt(P, seed=seed, vocab=w.vocab)
+        self.new, self.ref = (ssd.Decoder(config_for(w, P + 8), dw, on_device=True) for _ in range(2))
+        for i in range(0, P, 16):
+            self.ref.debug_forward(False, self.prompt[i:i + 16], i)
+        self.positions = sorted({p for p in EDGES if p < P} | {P - 1})
+
+    def error(self, p):
+        self.new.prefill(self.prompt)  # (the forward below writes row p)
+        got, ref = (d.debug_forward(False, self.prompt[p:p + 1], p)[0].astype(np.float64) for d in (self.new, self.ref))
+        return np.linalg.norm(got - ref) / np.linalg.norm(ref)
+
+    def close(self):
+        self.new.close()
+        self.ref.close()
+
+
 # token tiles of 32 .. 256 rows and their edges; GQA, an odd number of 128-row
 # boxes of q / k / v, ffn not a multiple of the tile
 @pytest.mark.parametrize("P", [18, 33, 34, 65, 66, 97, 161, 257, 258, 290, 514])
@@ -67,12 +105,32 @@ def test_prompt_token_tiles(P):
     assert prompt_error(w, hw, synth.host_to_device_weights(hw), P, seed=P) <= 4 * EPS
 
 
+@pytest.mark.parametrize("P", [18, 33, 66, 161, 258, 514])
+def test_prompt_rows(P):
+    w = model()
+    caches = CachePair(w, synth.host_to_device_weights(synth.host_weights(w, seed=21)), P, seed=P)
+    for p in caches.positions:
+        assert caches.error(p) <= EPS, p
+    # the same with one row of the reference replaced by another token's
+    row = P // 2
+    caches.ref.debug_forward(False, [(caches.prompt[row] + 1) % w.vocab], row)
+    for p in caches.positions:
+        if p > row:
+            assert caches.error(p) > EPS, p
+    caches.close()
+
+
 @pytest.mark.parametrize("heads,kv_heads,hd,d,ffn", [(1, 1, 128, 128, 64), (3, 3, 128, 384, 1040), (6, 2, 64, 640, 80),
                                                      (8, 1, 128, 1024, 2736)])
 def test_prompt_shapes(heads, kv_heads, hd, d, ffn):
     w = model(heads, kv_heads, hd, d, ffn)
     hw = synth.host_weights(w, seed=22)
-    assert prompt_error(w, hw, synth.host_to_device_weights(hw), 150, seed=5) <= 4 * EPS
+    dw = synth.host_to_device_weights(hw)
+    assert prompt_error(w, hw, dw, 150, seed=5) <= 4 * EPS
+    caches = CachePair(w, dw, 150, seed=5)
+    for p in caches.positions:
+        assert caches.error(p) <= EPS, p
+    caches.close()
 
 
 # scores large enough that the running maximum moves after the first key block
@@ -84,8 +142,13 @@ def test_prompt_attention_rescale(P):
     for layer in hw["layers"]:
         for name in ("wq", "wk"):
             layer[name] = synth.round_bf16_host(synth.bf16_bits_to_f64(layer[name]) * scale).reshape(layer[name].shape)
-    S = 4 * (0.02 * scale) ** 2 * w.d_model / np.sqrt(w.head_dim) * np.sqrt(w.head_dim)
-    assert prompt_error(w, hw, synth.host_to_device_weights(hw), P, seed=6) <= 4 * EPS * (1 + S)
+    S = 4 * (0.02 * scale) ** 2 * w.d_model
+    dw = synth.host_to_device_weights(hw)
+    assert prompt_error(w, hw, dw, P, seed=6) <= 4 * EPS * (1 + S)
+    caches = CachePair(w, dw, P, seed=6)
+    for p in caches.positions:
+        assert caches.error(p) <= EPS * (1 + S / np.sqrt(w.head_dim)), p
+    caches.close()
 
 
 # clusters of 1, 2, 4 and 8 CTAs, more than one chunk of 1024 k, ends of rows,
