@@ -12,8 +12,8 @@
 //            rewrites KV for every layer and ends in the acceptance kernel;
 //   accept : n accepted drafts plus a correction / bonus token are emitted,
 //            len <- len + 1 + n (the KV rollback is this length pointer).
-// Everything between two rounds stays on the device; the host reads one int
-// (tokens emitted so far) per round to size the next round.
+// Everything between two rounds stays on the device; the host reads two ints
+// (tokens emitted so far, the error flag) per round to size the next round.
 #include <cmath>
 #include <cstddef>
 #include <cstdlib>
@@ -137,8 +137,7 @@ struct ssd_handle {
     int last_prompt_token = 0;
     bool sync_check = false;
     // prefill on the tensor cores (prefill.cu): plan, per-layer arguments and
-    // TMA maps (box 64 x 128); used for prompts of more than 16 rows
-    bool pf_on = false;
+    // TMA maps; used for prompts of more than 16 rows
     PrefillPlan pf{};
     std::vector<PrefillLayer> pf_layers;
     CUtensorMap* pf_tmaps = nullptr;
@@ -388,7 +387,6 @@ GemmArgs proj_args(ssd_handle* h, int N, int K, int n_tiles) {
     a.n_chunks = (K + kFKC - 1) / kFKC;
     a.n_units = n_tiles * a.n_chunks;
     a.partial = h->partial;
-    a.err = &h->st->err;
     a.inv_dim = 1.0f / (float)h->cfg.d_model;
     a.eps = h->cfg.rms_eps;
     return a;
@@ -415,7 +413,6 @@ std::vector<FwdOp> build_ops(ssd_handle* h, bool draft) {
             q.type = OP_QKV;
             GemmArgs& a = q.g;
             a = proj_args(h, qd + 2 * kvd, d, (qd + 2 * kvd) / kFTile);
-            a.w0 = h->wq[l]; a.w1 = h->wk[l]; a.w2 = h->wv[l];
             a.tm_w[0] = h->tmaps + tmap_weight(l, 0);
             a.tm_w[1] = h->tmaps + tmap_weight(l, 1);
             a.tm_w[2] = h->tmaps + tmap_weight(l, 2);
@@ -434,15 +431,14 @@ std::vector<FwdOp> build_ops(ssd_handle* h, bool draft) {
             t.tm_k = h->tmaps + tmap_kv(h, 0); t.tm_v = h->tmaps + tmap_kv(h, 1); t.kv_z0 = l * c.n_kv_heads;
             t.out_hi = h->at_hi; t.out_lo = h->at_lo;
             t.part = h->attn_part;
-            t.n_heads = c.n_heads; t.n_kv_heads = c.n_kv_heads; t.head_dim = c.head_dim;
+            t.n_heads = c.n_heads; t.n_kv_heads = c.n_kv_heads;
             t.group = c.n_heads / c.n_kv_heads; t.group_inv = attn_group_inv(t.group);
-            t.max_seq = c.max_seq; t.n_chunks = h->n_chunks;
-            t.scale = 1.0f / std::sqrt((float)c.head_dim); t.st = h->st; t.err = &h->st->err;
+            t.n_chunks = h->n_chunks;
+            t.scale = 1.0f / std::sqrt((float)c.head_dim);
             ops.push_back(at);
             FwdOp o{};
             o.type = OP_RESID;
             o.g = proj_args(h, d, qd, d_tiles);
-            o.g.w0 = h->wo[l];
             o.g.tm_w[0] = h->tmaps + tmap_weight(l, 3);
             set_x_maps(h, o.g, 1);
             o.g.out_f32 = h->h; o.g.ldo = d;
@@ -453,7 +449,6 @@ std::vector<FwdOp> build_ops(ssd_handle* h, bool draft) {
             FwdOp gu{};
             gu.type = OP_SWIGLU;
             gu.g = proj_args(h, 2 * c.ffn, d, (c.ffn + 63) / 64);
-            gu.g.w0 = h->w_gate[l]; gu.g.w1 = h->w_up[l];
             gu.g.tm_w[0] = h->tmaps + tmap_weight(l, 4);
             gu.g.tm_w[1] = h->tmaps + tmap_weight(l, 5);
             set_x_maps(h, gu.g, 0);
@@ -463,7 +458,6 @@ std::vector<FwdOp> build_ops(ssd_handle* h, bool draft) {
             FwdOp w{};
             w.type = OP_RESID;
             w.g = proj_args(h, d, c.ffn, d_tiles);
-            w.g.w0 = h->w_down[l];
             w.g.tm_w[0] = h->tmaps + tmap_weight(l, 6);
             set_x_maps(h, w.g, 2);
             w.g.out_f32 = h->h; w.g.ldo = d;
@@ -474,7 +468,6 @@ std::vector<FwdOp> build_ops(ssd_handle* h, bool draft) {
     FwdOp lg{};
     lg.type = OP_LOGITS;
     lg.g = proj_args(h, c.vocab, d, (c.vocab + kFTile - 1) / kFTile);
-    lg.g.w0 = h->lm_head;
     lg.g.tm_w[0] = h->tmaps + 7 * c.n_layers;
     set_x_maps(h, lg.g, 0);
     lg.g.ss_in = h->ss; lg.g.ss_in_tiles = d_tiles;
@@ -830,10 +823,8 @@ int ssd_create(const ssd_config* cfg, const ssd_weights* w, void* cuda_stream, s
     if (e != cudaSuccess) return bail(fail(SSD_ERR_CUDA, std::string("init: ") + cudaGetErrorString(e)));
     if ((rc = build_tmaps(h)) || (rc = upload_ops(h, false)) || (rc = upload_ops(h, true))) return bail(rc);
 
-    // prefill on the tensor cores: needs the q / k / v widths in whole
-    // 128-row boxes; otherwise prompts run through the decode kernel
-    h->pf_on = true;
-    if (h->pf_on) {
+    // prefill on the tensor cores (the q / k / v widths are whole 128-row boxes)
+    {
         PrefillPlan& P = h->pf;
         P.n_layers = L;
         P.d = d;
@@ -920,7 +911,7 @@ int ssd_prefill(ssd_handle* h, const int32_t* prompt, int n_prompt) {
     if (n_prompt > 1)
         CUDA_TRY(cudaMemcpyAsync(h->tok, prompt, sizeof(int) * (n_prompt - 1), cudaMemcpyHostToDevice, h->stream),
                  "prompt upload");
-    if (h->pf_on && n_prompt - 1 > kMaxRows) {
+    if (n_prompt - 1 > kMaxRows) {
         // tensor-core prefill, chunks of up to pf.rows positions
         for (int p0 = 0; p0 < n_prompt - 1; p0 += h->pf.rows) {
             const int n = std::min(h->pf.rows, n_prompt - 1 - p0);

@@ -15,7 +15,6 @@ constexpr int kMaxRows = 16;      // rows of one forward (verification K+1 <= 16
 constexpr int kMaxK = 15;         // drafts per round
 constexpr int kGemmThreads = 256; // consumer threads of a forward CTA
 constexpr int kAttnChunk = 64;    // KV positions per attention CTA (absolute chunks)
-constexpr int kAttnThreads = 256;
 constexpr int kFTile = 128;       // forward kernel: weight rows per tile (tcgen05 M, TMEM lanes)
 constexpr int kFKC = 128;         // forward kernel: k per work unit (128 rows x 128 k = 32 KB of weights)
 constexpr int kPartWords = 6 * 128;  // 128-bit words of a segment's partial: [2][3][128], three input rows each
@@ -55,9 +54,6 @@ struct DecodeState {
 enum GemmEpi { EPI_LOGITS = 0, EPI_RESID = 1, EPI_SWIGLU = 2, EPI_QKV = 3 };
 
 struct GemmArgs {
-    const bf16* w0;      // weight segment 0 (wq / w_gate / the only matrix)
-    const bf16* w1;      // segment 1 (wk / w_up)
-    const bf16* w2;      // segment 2 (wv)
     int N;               // logical output rows
     int K;               // reduction length (row length of every segment)
     int n_tiles;         // row tiles
@@ -72,7 +68,6 @@ struct GemmArgs {
     f16* k_cache;        // this layer: [Hkv][max_seq][hd] fp16
     f16* v_cache;
     const float2* rope;  // [max_seq][hd/2] (cos, sin)
-    int* err;            // device error flag
     const float* ss_in;  // [M][ss_in_tiles] sums of squares of the pre-norm row (nullptr: no norm)
     int ss_in_tiles;
     float inv_dim, eps;  // RMSNorm scale of row m: rsqrt(sum(ss_in[m]) * inv_dim + eps)
@@ -86,7 +81,7 @@ struct GemmArgs {
     // {K, rows} with box {64, 128} (SwiGLU gate / up: {64, 64}), one copy per
     // 64-wide k box of a unit; x maps view the planes as {K, 16, 2} with box
     // {64, R, 2}, one copy per k box.
-    const void* tm_w[3];  // w0, w1, w2
+    const void* tm_w[3];  // the matrices (q / k / v, gate / up, or one)
     const void* tm_x[kPlaneClasses];  // input planes for R = 1 | 4 | 8 | 12 | 16
 };
 
@@ -108,12 +103,10 @@ struct AttnArgs {
     bf16* out_hi;        // [M][H*hd] output planes: hi = rn(o), lo = rn(o - hi)
     bf16* out_lo;
     float* part;         // segment partials [Hkv][n_chunks][G*M][attn_part_floats(hd)]: o[hd], max, sum, 2 pad
-    int M, n_heads, n_kv_heads, head_dim, max_seq, n_chunks;
+    int n_heads, n_kv_heads, n_chunks;
     int group;           // query heads per KV head
     unsigned group_inv;  // ceil(2^24 / group), or 0 for groups of 1024 and more (AttnArgs::row_of)
     float scale;         // 1/sqrt(hd)
-    const DecodeState* st;
-    int* err;            // device error flag (checked builds)
     // input row v / group of query vector v < 16 group: the product's error, v (group_inv
     // group - 2^24) / 2^24 < 16 group^2 / 2^24 of a group, stays below one vector
     __host__ __device__ int row_of(int v) const {
@@ -221,7 +214,7 @@ int set_last_error(int code, const char* msg);
 
 // launchers (return cudaError_t)
 
-// src for launch_embed
+// where a forward's tokens and first position come from
 enum EmbedSrc { SRC_TOKENS = 0, SRC_DRAFT = 1, SRC_VERIFY = 2 };
 
 int launch_greedy_draft(const float* logits, int V, DecodeState* st, cudaStream_t s);
@@ -249,9 +242,6 @@ int launch_spec_accept_batch(const float* p_rows, const float* q_rows, int V, in
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
-__device__ __forceinline__ float2 f16x2(uint32_t w) {
-    return __half22float2(*reinterpret_cast<const __half2*>(&w));
-}
 
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
@@ -279,16 +269,6 @@ __device__ __forceinline__ bool elect_one() {
     return p != 0;
 }
 
-// 16-byte async copy global -> shared; src_bytes = 0 zero-fills the slot.
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem, int src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_u32(smem)),
-                 "l"(gmem), "r"(src_bytes));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
-}
 // Programmatic dependent launch: let the next kernel in the stream start its
 // prologue now / wait until the previous kernel's results are visible.
 __device__ __forceinline__ void pdl_launch_dependents() {
