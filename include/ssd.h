@@ -145,6 +145,10 @@ int ssd_set_draft_exit(ssd_handle* h, int enable, float gamma0, float alpha, flo
  * positions [0, n_prompt-1); prompt[n_prompt-1] becomes the first round's
  * x_last, so every generated token comes from a decoding round.  prompt is a
  * host array of token ids in [0, vocab); 1 <= n_prompt <= max_seq.
+ * A prompt GEMM whose tiles are split over CTAs has CTAs that wait, up to 2 s,
+ * for sums of CTAs with lower block numbers.  CUDA does not promise that those
+ * are dispatched first; the call returns SSD_ERR_TIMEOUT if they have not run
+ * in that time (say, because other work holds their SMs), and may be repeated.
  * Errors: INVALID_ARG, CAPACITY, CUDA, TIMEOUT. */
 int ssd_prefill(ssd_handle* h, const int32_t* prompt, int n_prompt);
 

@@ -9,10 +9,11 @@
 //
 // CTA = 8 warps x 16 weight rows = 128 rows, over a range of K.  A warp loads
 // its weights from global memory into MMA fragments directly, 16 bytes a
-// thread, two or four 64-wide k blocks (128 KB an SM) ahead of the MMAs: thread (g, t) reads 8 consecutive bf16 of rows g and g + 8, which the A and
-// B fragments both interpret as the same logical k slots, so the product is
-// unchanged, and a quad reads whole 128-byte lines.  The activations pass
-// through shared memory as bf16 pairs, up to 1024 k at a time.
+// thread, two or four 64-wide k blocks ahead of the MMAs: thread (g, t) reads 8
+// consecutive bf16 of rows g and g + 8, which the A and B fragments both interpret
+// as the same logical k slots, so the product is unchanged, and a quad reads whole
+// 128-byte lines.  The activations pass through shared memory as bf16 pairs, up
+// to 1024 k at a time.
 //
 // Few row tiles: K is split over a cluster of 2, 4 or 8 CTAs, which add their
 // sums through distributed shared memory in rank order: no scratch in global
@@ -47,7 +48,7 @@ struct LinearArgs {
     int N, K, M;
     int kc;  // k per CTA of the cluster, a multiple of 64
 
-    // what the accesses of a checked build have to satisfy
+#ifdef SSD_CHECKED  // what the kernel's accesses have to satisfy
     __host__ __device__ bool weights_in(const bf16* p, size_t elems) const {
         return ((uintptr_t)p & 15u) == 0 && p >= w && p + elems <= w + (size_t)N * K;
     }
@@ -55,6 +56,7 @@ struct LinearArgs {
         return ((uintptr_t)p & 15u) == 0 && p >= x && p + elems <= x + (size_t)M * K;
     }
     __host__ __device__ bool output_in(const float* p) const { return p >= y && p < y + (size_t)M * N; }
+#endif
 };
 #ifdef SSD_CHECKED
 __device__ int g_linear_err;  // code of the first failed check
@@ -87,10 +89,11 @@ __device__ __forceinline__ void lin_cluster_sync() {
 }
 
 // P = 8 or 16 activation rows; the MMA's N side holds P rows of x_hi, then P of
-// x_lo.  128 KB of weights in flight per SM either way: 4 CTAs with 2
-// blocks a warp ahead where registers allow it (P = 8; N 22016, K 4096, cold:
-// 45 us against 61 with 2 CTAs and 4 blocks), else 2 CTAs with 4 blocks (P = 16;
-// N = K = 4096: 18.0 us against 20.1).
+// x_lo.  4 CTAs an SM with 2 blocks a warp ahead where registers allow it (P = 8;
+// N 22016, K 4096, cold: 45 us against 61 with 2 CTAs and 4 blocks), else 2 CTAs with
+// 4 blocks (P = 16; N = K = 4096, cold, before the L2 prefetch: 18.0 us against 20.1).
+// Where the grid fills every SM so, 128 KB of weights are in flight per SM; with few
+// row tiles less: 256 CTAs for N = 4096 leave 48 of 152 SMs with one.
 template <int P>
 struct LinShape {
     static constexpr int CTAS = P == 8 ? 4 : 2, DEPTH = P == 8 ? 2 : 4;
@@ -295,12 +298,13 @@ extern "C" int ssd_linear_noalloc(const void* w, const float* x, float* y, int N
     if (M < 1 || M > kMaxRows || N < 1 || K < 16 || K % 16)
         return set_last_error(SSD_ERR_INVALID_ARG,
                               "ssd_linear_noalloc: need 1 <= M <= 16, N >= 1, K a positive multiple of 16");
-    // the sizes the call takes (ssd.h): the kernel itself needs no scratch
+    // the sizes the call takes (ssd.h)
     const size_t tiles64 = ((size_t)N + 63) / 64, need = K > 512 ? (size_t)((K + 511) / 512) * M * 64 * tiles64 : 0;
     if (tiles64 > 4096 || need > (size_t(1) << 20))
         return set_last_error(SSD_ERR_CAPACITY,
-                              ("ssd_linear_noalloc: problem counts " + std::to_string(need) + " scratch floats and " +
-                               std::to_string(tiles64) + " tiles; the limits are 1048576 floats and 4096 tiles")
+                              ("ssd_linear_noalloc: sizes beyond the call's limits (kept from the time it had scratch "
+                               "memory): " + std::to_string(tiles64) + " of 4096 tiles of 64 rows, " +
+                               std::to_string(need) + " of 1048576 partial sums")
                                   .c_str());
     int dev = 0, n_sms = 0;
     cudaError_t e = cudaGetDevice(&dev);

@@ -334,8 +334,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) tc_gemm
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank();
-    // the highest ranges start first: a pair only waits for partial sums of
-    // pairs with higher numbers, which were dispatched before it
+    // the highest ranges start first: a pair only waits for partial sums of pairs
+    // with higher numbers, whose blocks come first in dispatch order (which CUDA does
+    // not promise: the wait is bounded)
     const int pair = a.sched.pairs - 1 - (int)(blockIdx.x >> 1);
     const int S = a.stages, stage_bytes = kATile + a.nt * 128;
     if (threadIdx.x == 0) {

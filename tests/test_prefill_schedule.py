@@ -6,8 +6,8 @@ Checked for each shape: the token tiles cover the rows; every (tile, k block)
 is computed exactly once; a segment that starts inside a tile is its pair's
 first one (a pair has one workspace slot); and the pair that finalises a tile
 counts exactly the pairs that left partial sums of it, which are the next ones
-in number (they are dispatched before it, so it never waits for a pair that
-cannot run).
+in number (their blocks come before its own, so in the usual order of dispatch it
+never waits for a pair that cannot run).
 """
 import os
 import subprocess
