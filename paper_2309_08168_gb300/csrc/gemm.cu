@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kLinThreads, LinShape<P>::CTAS) linear_kernel(
     };
     // The weights on their way into L2 while the previous kernel ends (a prefetch
     // returns nothing, so it may run ahead of a kernel that writes them).  Calls
-    // back to back, 0 / 256 / 512 k ahead: 16 x 4096 x 4096 12.3 / 11.2 / 10.7 us,
+    // back to back, 0 / 256 / 512 k ahead (loads through .nc): 16 x 4096 x 4096 12.3 / 11.2 / 10.7 us,
     // 4 x 4096 x 32000 51.3 / 48.5 / 49.8, 8 x 8192 x 8192 28.2 / 25.8 / 27.0.
     if (threadIdx.x < kLinRows && k1 > k0) {
         const bf16* row = a.w + (size_t)min(tile * kLinRows + (int)threadIdx.x, a.N - 1) * a.K + k0;
